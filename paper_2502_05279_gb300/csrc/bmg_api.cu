@@ -185,8 +185,8 @@ struct Level {
   float* f32 = nullptr;
   int tile32 = -1;        // FP32 sweeps: -1 row kernel (in place), else tile shape of the one-pass kernel
   int pair32 = -1;        // >= 0: pairs of sweeps run as one two-sweep launch of this shape (needs tile32 >= 0)
-  double* lcp = nullptr;  // line relaxation: elimination multipliers (FP64 cycle)
-  float* lcp32 = nullptr; // the same for the FP32 cycle
+  LineFactor<double> lfac[2];   // line relaxation: factored x-lines, y-lines (FP64 cycle; one allocation each, at c)
+  LineFactor<float> lfac32[2];  // the same for the FP32 cycle
   float* x32b = nullptr;  // second iterate of a tile-swept level (sweeps alternate x32 <-> x32b)
   int fused = 0;          // 1: the cycle's multiply-adds on this level are fused (BMG_ARITH_FUSED)
   int tile64 = -1;        // FP64 sweeps: -1 row kernel (in place), else shape of the FP64 one-pass kernel
@@ -347,7 +347,7 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
   auto relax64 = [&](int sweeps) {
     if (is_line(h->smoother))
       step(h, l, BMG_K_RELAX, 0,
-           [&] { launch_line<double, double>(v, L.kind, f, x, L.lcp, sweeps, line_dir(h->smoother), done, s); });
+           [&] { launch_line_solve(v, L.kind, f, x, L.lfac[0], L.lfac[1], sweeps, line_dir(h->smoother), done, s); });
     else if (L.tile64 >= 0)
       for (int k = 0; k < sweeps; ++k) {
         double* nxt = cur == x ? L.x64b : x;
@@ -373,8 +373,8 @@ void relax32(bmg_hierarchy* h, const StencilView<float, S>& v, int l, int sweeps
   Level& L = h->lv[l];
   if (is_line(h->smoother)) {
     step(h, l, BMG_K_RELAX, 1, [&] {
-      launch_line<float, S>(v, L.kind, (const float*)L.f32, L.x32, L.lcp32, sweeps, line_dir(h->smoother), done,
-                            h->ws);
+      launch_line_solve(v, L.kind, (const float*)L.f32, L.x32, L.lfac32[0], L.lfac32[1], sweeps,
+                        line_dir(h->smoother), done, h->ws);
     });
     return;
   }
@@ -874,14 +874,34 @@ int force_tile(bmg_hierarchy* h) {
   return BMG_OK;
 }
 
-// BMG_SMOOTHER_LINE / _LINE_Y / _LINE_XY: the multiplier scratch of every relaxed level.
-int alloc_line(bmg_hierarchy* h) {
+// BMG_SMOOTHER_LINE / _LINE_Y / _LINE_XY: the factored lines of every relaxed
+// level, for the axes the smoother uses.
+int build_lines(bmg_hierarchy* h) {
+  const int dir = line_dir(h->smoother);
   for (int l = 0; l + 1 < h->nlev; ++l) {
     Level& L = h->lv[l];
-    int rc = h->precision == BMG_FP64 ? dalloc(&L.lcp, plane_size(L.n)) : galloc(&L.lcp32, L.n, 1, h->ws);
-    if (rc) return rc;
+    const size_t ps = plane_size(L.n);
+    for (int axis = 0; axis < 2; ++axis) {
+      if (dir == (axis == 0 ? LINE_Y : LINE_X)) continue;
+      if (h->precision == BMG_FP64) {
+        LineFactor<double>& F = L.lfac[axis];
+        if (int rc = dalloc(&F.c, 4 * ps)) return rc;
+        F.m = F.c + ps;
+        F.y = F.m + ps;
+        F.yl = F.y + ps;
+        launch_line_factor(view64(L), axis, F, h->ws);
+      } else {
+        LineFactor<float>& F = L.lfac32[axis];
+        if (int rc = dalloc(&F.c, 2 * ps)) return rc;
+        F.m = F.c + ps;
+        if (L.bf16)
+          launch_line_factor(viewbf(L), axis, F, h->ws);
+        else
+          launch_line_factor(view32(L), axis, F, h->ws);
+      }
+    }
   }
-  return BMG_OK;
+  return cuda_check(cudaGetLastError(), "line factors");
 }
 
 // The tuners' result caches are process-wide; setups running on several host
@@ -1118,8 +1138,10 @@ void free_level(Level& L, bool shared_ops = false) {
   cudaFree(L.ci);
   cudaFree(L.x);
   cudaFree(L.f);
-  cudaFree(L.lcp);
-  gfree(L.lcp32);
+  for (int axis = 0; axis < 2; ++axis) {
+    cudaFree(L.lfac[axis].c);
+    cudaFree(L.lfac32[axis].c);
+  }
   gfree(L.st32);
   gfree(L.off16);
   gfree(L.od32);
@@ -1410,7 +1432,7 @@ int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* o, bmg_hiera
   if (!rc) rc = order_after_user(h);
   if (!rc) rc = setup_impl(h, A, h->n, o);
   const bool line = is_line(h->smoother);
-  if (!rc && line) rc = alloc_line(h);
+  if (!rc && line) rc = build_lines(h);
   if (!rc && !line && h->smoother >= BMG_SMOOTHER_TILE) rc = force_tile(h);
   if (!rc && !line && h->use_graph) rc = autotune_solo(h);
   if (!rc && !line && h->use_graph)   // the level-fused tail relaxes by points

@@ -571,10 +571,6 @@ void launch_line(const StencilView<T, S>& v, int kind, const T* f, T* x, T* cp, 
 }
 template void launch_line<double, double>(const StencilView<double, double>&, int, const double*, double*, double*,
                                           int, int, const int*, cudaStream_t);
-template void launch_line<float, float>(const StencilView<float, float>&, int, const float*, float*, float*, int,
-                                        int, const int*, cudaStream_t);
-template void launch_line<float, __nv_bfloat16>(const StencilView<float, __nv_bfloat16>&, int, const float*, float*,
-                                                float*, int, int, const int*, cudaStream_t);
 
 template <typename T>
 void launch_interp_correct(int n, const T* ci, const T* ec, T* x, const int* done, cudaStream_t s, int fused) {

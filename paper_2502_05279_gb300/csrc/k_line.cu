@@ -1,0 +1,320 @@
+// Zebra line relaxation with factored lines: the elimination of a line's
+// tridiagonal matrix depends on the operator only, so a hierarchy forms it once
+// at setup and a sweep only carries right-hand sides through it.
+//
+// What bounds it.  The Thomas recurrence is a chain along the line, and its
+// rounding is fixed, so a half sweep costs at least (line length) x (dependent
+// FP64 operations per point).  On GB300 a dependent FP64 operation takes about
+// 63 cycles, a warp's FP64 instruction occupies its quarter of the SM for about
+// 60 of them whatever the number of active lanes, and an FP64 division takes
+// 560 (measured on one warp).  The unfactored form (line_row_body) pays two
+// divisions per point and waits for its uncoalesced loads on the same thread:
+// 720 us per half sweep at 511^2.
+// Layout of the work.  One warp per CTA runs the chains of R lines, one per
+// lane, and issues nothing else; the CTA's other warps form the right-hand
+// sides g = f - (couplings to the fixed lines) of the next LC positions, fetch
+// the factors, and store the previous positions' results, all through shared
+// memory, so that their loads coalesce and their FP64 work runs on the other
+// three quarters of the SM.  Per point the chain is a product, a difference and
+// line_div's four operations forward, and two operations backward: 511 x 8 x 63
+// cycles, about 130 us per half sweep at 511^2.
+#include "cycle_device.cuh"
+
+namespace bmg {
+using namespace dev;
+namespace {
+
+constexpr int LC = 32;              // positions per stage
+constexpr int LINE_THREADS = 256;   // warp 0: the chains; warps 1 .. 7: everything else
+
+// s / m, correctly rounded, from y = fl(1/m) and yl = fl(y (1 - m y)), so that
+// y + yl = 1/m to about 2^-104 relative.  q0 = fl(s y + fl(s yl)) is then less
+// than one ulp from s / m, the residual s - m q0 is exact in one FMA, and the
+// last FMA rounds s / m correctly (Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990,
+// theorem on the final quotient step: q0 within one ulp, y the rounded
+// reciprocal, no over- or underflow).  y = 0 marks an m outside 2^[-200, 200];
+// such an m, and an s outside 2^[-623, 623] other than zero, take the division.
+// The tests are on the bit patterns: comparisons would use the FP64 pipe.
+__device__ __noinline__ double line_div_slow(double s, double m) { return rdiv(s, m); }
+
+__device__ __forceinline__ double line_div(double s, double m, double y, double yl) {
+  // the four operations first: their dependent chain does not wait for the tests
+  const double q0 = __fma_rn(s, y, rmul(s, yl));
+  double q = __fma_rn(__fma_rn(-m, q0, s), y, q0);
+  const unsigned hs = (unsigned)__double2hiint(s), es = (hs >> 20) & 0x7ffu;
+  if (es - 400u > 1246u || __double2hiint(y) == 0) {
+    if (__double2hiint(y) != 0 && (hs << 1) == 0 && __double2loint(s) == 0)   // +-0 / m
+      q = __hiloint2double((int)((hs ^ (unsigned)__double2hiint(m)) & 0x80000000u), 0);
+    else
+      q = line_div_slow(s, m);
+  }
+  return q;
+}
+
+// Point of position q (1 .. n) on line w (1 .. n): x-lines run along i, y-lines along j.
+template <int AXIS>
+__device__ __forceinline__ size_t line_point(int ld, int w, int q) {
+  return AXIS == 0 ? (size_t)w * ld + q : (size_t)q * ld + w;
+}
+
+// Couplings of p to the previous and the next point of its line.
+template <int AXIS, typename T, typename S>
+__device__ __forceinline__ T line_prev(const StencilView<T, S>& v, size_t p) {
+  return cvt<T>(AXIS == 0 ? v.W[p] : v.S_[p]);
+}
+template <int AXIS, typename T, typename S>
+__device__ __forceinline__ T line_next(const StencilView<T, S>& v, size_t p) {
+  return cvt<T>(AXIS == 0 ? v.W[p + 1] : v.S_[p + v.ld]);
+}
+
+// m_1 = a_O, m_q = a_O - a_prev c_{q-1}, c_q = a_next / m_q; one thread per line.
+// LF positions are read ahead of the chain.
+template <typename T, typename S, int AXIS>
+__global__ void k_line_factor(StencilView<T, S> v, T* __restrict__ c, T* __restrict__ m) {
+  constexpr int LF = 8;
+  const int n = v.n, ld = v.ld;
+  const int w = 1 + blockIdx.x * blockDim.x + threadIdx.x;
+  if (w > n) return;
+  T cp = T(0);
+  for (int q0 = 1; q0 <= n; q0 += LF) {
+    T o[LF], a[LF], b[LF];
+#pragma unroll
+    for (int k = 0; k < LF; ++k) {
+      const size_t p = line_point<AXIS>(ld, w, q0 + k <= n ? q0 + k : n);
+      o[k] = v.O[p];
+      a[k] = line_prev<AXIS>(v, p);
+      b[k] = line_next<AXIS>(v, p);
+    }
+#pragma unroll
+    for (int k = 0; k < LF; ++k) {
+      if (q0 + k > n) break;
+      const size_t p = line_point<AXIS>(ld, w, q0 + k);
+      const T mm = q0 + k == 1 ? o[k] : rsub(o[k], rmul(a[k], cp));
+      cp = rdiv(b[k], mm);
+      if (BMG_IN(DBG_LINE_STORE, p, (size_t)(n + 2) * ld)) {
+        c[p] = cp;
+        m[p] = mm;
+      }
+    }
+  }
+}
+
+// y = fl(1/m) and yl = fl(y (1 - m y)) for line_div; y = 0 where it must not be used.
+__global__ void k_line_recip(int n, const double* __restrict__ m, double* __restrict__ y, double* __restrict__ yl) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x + 1, j = blockIdx.y * blockDim.y + threadIdx.y + 1;
+  if (i > n || j > n) return;
+  const size_t p = (size_t)j * (n + 2) + i;
+  if (!BMG_IN(DBG_LINE_STORE, p, (size_t)(n + 2) * (n + 2))) return;
+  const double mm = m[p];
+  const unsigned e = ((unsigned)__double2hiint(mm) >> 20) & 0x7ffu;
+  const bool ok = e - 823u <= 400u;
+  const double r = ok ? rdiv(1.0, mm) : 0.0;
+  y[p] = r;
+  yl[p] = ok ? rmul(__fma_rn(-mm, r, 1.0), r) : 0.0;
+}
+
+// Right-hand side of p: f minus the couplings to the two fixed lines, in the
+// order of line_row_body (S, N, SW, NE, NW, SE) or line_col_body (W, E, SW, NE, SE, NW).
+template <int AXIS, bool NINE, typename T, typename S>
+__device__ __forceinline__ T line_rhs(const StencilView<T, S>& v, const T* __restrict__ f, const T* x, size_t p) {
+  const int ld = v.ld;
+  T g = f[p];
+  if (AXIS == 0) {
+    g = rsub(g, rmul(cvt<T>(v.S_[p]), x[p - ld]));
+    g = rsub(g, rmul(cvt<T>(v.S_[p + ld]), x[p + ld]));
+    if (NINE) {
+      g = rsub(g, rmul(cvt<T>(v.SW[p]), x[p - ld - 1]));
+      g = rsub(g, rmul(cvt<T>(v.SW[p + ld + 1]), x[p + ld + 1]));
+      g = rsub(g, rmul(cvt<T>(v.NW[p]), x[p + ld - 1]));
+      g = rsub(g, rmul(cvt<T>(v.NW[p + 1 - ld]), x[p + 1 - ld]));
+    }
+  } else {
+    g = rsub(g, rmul(cvt<T>(v.W[p]), x[p - 1]));
+    g = rsub(g, rmul(cvt<T>(v.W[p + 1]), x[p + 1]));
+    if (NINE) {
+      g = rsub(g, rmul(cvt<T>(v.SW[p]), x[p - ld - 1]));
+      g = rsub(g, rmul(cvt<T>(v.SW[p + ld + 1]), x[p + ld + 1]));
+      g = rsub(g, rmul(cvt<T>(v.NW[p + 1 - ld]), x[p + 1 - ld]));
+      g = rsub(g, rmul(cvt<T>(v.NW[p]), x[p + ld - 1]));
+    }
+  }
+  return g;
+}
+
+// One stage's inputs and its results, [line][position] with a padded row.
+template <typename T, int R>
+struct LineStage {
+  T g[R][LC + 1], a[R][LC + 1], m[R][LC + 1], y[R][LC + 1], yl[R][LC + 1], out[R][LC + 1];
+};
+
+// The lines first, first + 2, ... of one parity, R per CTA, solved in place on
+// x.  The lines of the other parity are only read, so every CTA's inputs are
+// fixed for the launch; a CTA reads of its own lines only what it wrote itself.
+template <typename T, typename S, bool NINE, int AXIS, int R>
+__global__ void __launch_bounds__(LINE_THREADS)
+    k_line_solve(StencilView<T, S> v, const T* __restrict__ f, T* x, LineFactor<T> fac, int first, const int* done) {
+  extern __shared__ __align__(16) unsigned char line_smem[];
+  pdl_enter();
+  if (stopped(done)) return;
+  LineStage<T, R>* st = reinterpret_cast<LineStage<T, R>*>(line_smem);
+  const int n = v.n, ld = v.ld, stages = (n + LC - 1) / LC;
+  const int w0 = first + 2 * R * (int)blockIdx.x;
+  const int tid = threadIdx.x, help = tid - 32;
+  // helpers: point (line r, position offset t) number e of a stage; consecutive
+  // threads take consecutive addresses
+  auto each = [&](int k, auto&& fn) {
+#pragma unroll 2
+    for (int e = help; e < R * LC; e += LINE_THREADS - 32) {
+      const int r = AXIS == 0 ? e / LC : e % R, t = AXIS == 0 ? e % LC : e / R;
+      const int w = w0 + 2 * r, q = 1 + k * LC + t;
+      if (w <= n && q <= n) fn(r, t, line_point<AXIS>(ld, w, q));
+    }
+  };
+  auto fetch = [&](int k) {
+    LineStage<T, R>& b = st[k & 1];
+    each(k, [&](int r, int t, size_t p) {
+      b.a[r][t] = line_prev<AXIS>(v, p);
+      b.m[r][t] = fac.m[p];
+      if constexpr (sizeof(T) == 8) {
+        b.y[r][t] = fac.y[p];
+        b.yl[r][t] = fac.yl[p];
+      }
+      b.g[r][t] = line_rhs<AXIS, NINE>(v, f, x, p);
+    });
+  };
+  auto fetch_back = [&](int k) {
+    LineStage<T, R>& b = st[k & 1];
+    each(k, [&](int r, int t, size_t p) {
+      b.a[r][t] = fac.c[p];
+      b.g[r][t] = x[p];
+    });
+  };
+  auto store = [&](int k) {
+    LineStage<T, R>& b = st[k & 1];
+    each(k, [&](int r, int t, size_t p) {
+      if (BMG_IN(DBG_LINE_STORE, p, (size_t)(n + 2) * ld)) x[p] = b.out[r][t];
+    });
+  };
+  const bool chain = tid < R && w0 + 2 * tid <= n;
+  const int r = tid;
+  T d = T(0);
+  // forward: d_q = (g_q - a_prev d_{q-1}) / m_q
+  if (help >= 0) fetch(0);
+  __syncthreads();
+  for (int k = 0; k < stages; ++k) {
+    if (help >= 0) {
+      if (k > 0) store(k - 1);
+      if (k + 1 < stages) fetch(k + 1);
+    } else if (chain) {
+      LineStage<T, R>& b = st[k & 1];
+      const int cnt = n - k * LC < LC ? n - k * LC : LC;
+#pragma unroll 4
+      for (int t = 0; t < cnt; ++t) {
+        const T s = k + t == 0 ? b.g[r][t] : rsub(b.g[r][t], rmul(b.a[r][t], d));
+        if constexpr (sizeof(T) == 8)
+          d = line_div(s, b.m[r][t], b.y[r][t], b.yl[r][t]);
+        else
+          d = rdiv(s, b.m[r][t]);
+        b.out[r][t] = d;
+      }
+    }
+    __syncthreads();
+  }
+  if (help >= 0) store(stages - 1);
+  __syncthreads();   // the CTA's forward results are in x
+  // backward: x_n = d_n, x_q = d_q - c_q x_{q+1}
+  if (help >= 0) fetch_back(stages - 1);
+  __syncthreads();
+  for (int k = stages - 1; k >= 0; --k) {
+    if (help >= 0) {
+      if (k + 1 < stages) store(k + 1);
+      if (k > 0) fetch_back(k - 1);
+    } else if (chain) {
+      LineStage<T, R>& b = st[k & 1];
+      const int cnt = n - k * LC < LC ? n - k * LC : LC;
+#pragma unroll 4
+      for (int t = cnt - 1; t >= 0; --t) {
+        d = 1 + k * LC + t == n ? b.g[r][t] : rsub(b.g[r][t], rmul(b.a[r][t], d));
+        b.out[r][t] = d;
+      }
+    }
+    __syncthreads();
+  }
+  if (help >= 0) store(0);
+}
+
+template <typename T, typename S, int AXIS, int R>
+void half_sweep(const StencilView<T, S>& v, int kind, const T* f, T* x, const LineFactor<T>& fac, int first,
+                int lines, const int* done, cudaStream_t s) {
+  constexpr size_t bytes = 2 * sizeof(LineStage<T, R>);
+  const unsigned g = (unsigned)((lines + R - 1) / R);
+  if (kind == 9) {
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        k_line_solve<T, S, true, AXIS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    (void)attr;
+    pdl_launch(k_line_solve<T, S, true, AXIS, R>, g, LINE_THREADS, bytes, s, v, f, x, fac, first, done);
+  } else {
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        k_line_solve<T, S, false, AXIS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    (void)attr;
+    pdl_launch(k_line_solve<T, S, false, AXIS, R>, g, LINE_THREADS, bytes, s, v, f, x, fac, first, done);
+  }
+  count_launch();
+}
+
+// Lines per CTA: 8 while that gives at most one CTA per SM (two CTAs on an SM
+// may put their chain warps on the same quarter, which runs them at half speed
+// each), then 16 and 32 lanes of the same chain warp, which cost it nothing.
+template <typename T, typename S, int AXIS>
+void sweep_axis(const StencilView<T, S>& v, int kind, const T* f, T* x, const LineFactor<T>& fac, const int* done,
+                cudaStream_t s) {
+  constexpr int SMS = 152;
+  for (int first = 1; first <= 2; ++first) {
+    const int lines = first == 1 ? (v.n + 1) / 2 : (v.n - 1) / 2;
+    if (lines <= 0) continue;
+    if (lines <= 8 * SMS)
+      half_sweep<T, S, AXIS, 8>(v, kind, f, x, fac, first, lines, done, s);
+    else if (lines <= 16 * SMS)
+      half_sweep<T, S, AXIS, 16>(v, kind, f, x, fac, first, lines, done, s);
+    else
+      half_sweep<T, S, AXIS, 32>(v, kind, f, x, fac, first, lines, done, s);
+  }
+}
+
+}  // namespace
+
+template <typename T, typename S>
+void launch_line_factor(const StencilView<T, S>& v, int axis, const LineFactor<T>& fac, cudaStream_t s) {
+  constexpr int TPB = 32;
+  const unsigned g = (unsigned)((v.n + TPB - 1) / TPB);
+  if (axis == 0)
+    k_line_factor<T, S, 0><<<g, TPB, 0, s>>>(v, fac.c, fac.m);
+  else
+    k_line_factor<T, S, 1><<<g, TPB, 0, s>>>(v, fac.c, fac.m);
+  count_launch();
+  if constexpr (sizeof(T) == 8) {
+    k_line_recip<<<dim3((v.n + 31) / 32, (v.n + 7) / 8), dim3(32, 8), 0, s>>>(v.n, fac.m, fac.y, fac.yl);
+    count_launch();
+  }
+}
+
+template <typename T, typename S>
+void launch_line_solve(const StencilView<T, S>& v, int kind, const T* f, T* x, const LineFactor<T>& fx,
+                       const LineFactor<T>& fy, int sweeps, int dir, const int* done, cudaStream_t s) {
+  for (int k = 0; k < sweeps; ++k) {
+    if (dir != LINE_Y) sweep_axis<T, S, 0>(v, kind, f, x, fx, done, s);
+    if (dir != LINE_X) sweep_axis<T, S, 1>(v, kind, f, x, fy, done, s);
+  }
+}
+
+#define BMG_INST(T, S)                                                                                         \
+  template void launch_line_factor<T, S>(const StencilView<T, S>&, int, const LineFactor<T>&, cudaStream_t); \
+  template void launch_line_solve<T, S>(const StencilView<T, S>&, int, const T*, T*, const LineFactor<T>&,   \
+                                        const LineFactor<T>&, int, int, const int*, cudaStream_t);
+BMG_INST(double, double)
+BMG_INST(float, float)
+BMG_INST(float, __nv_bfloat16)
+#undef BMG_INST
+
+}  // namespace bmg

@@ -61,6 +61,20 @@ enum { LINE_X = 0, LINE_Y = 1, LINE_XY = 2 };
 template <typename T, typename S>
 void launch_line(const StencilView<T, S>& v, int kind, const T* f, T* x, T* cp, int sweeps, int dir,
                  const int* done, cudaStream_t s);
+// The factored form a hierarchy uses (k_line.cu): per axis and level the
+// multipliers c and pivots m of every line's elimination, and in FP64 m's
+// rounded reciprocal y with its remainder yl, arrays of the level's (n+2)^2
+// layout filled by launch_line_factor (axis 0: x-lines, 1: y-lines).  fx, fy:
+// the factors of the axes that dir needs.  The same results as launch_line.
+template <typename T>
+struct LineFactor {
+  T *c = nullptr, *m = nullptr, *y = nullptr, *yl = nullptr;
+};
+template <typename T, typename S>
+void launch_line_factor(const StencilView<T, S>& v, int axis, const LineFactor<T>& fac, cudaStream_t s);
+template <typename T, typename S>
+void launch_line_solve(const StencilView<T, S>& v, int kind, const T* f, T* x, const LineFactor<T>& fx,
+                       const LineFactor<T>& fy, int sweeps, int dir, const int* done, cudaStream_t s);
 // FP32 / BF16 level arrays are allocated with STRIP_GUARD zeroed elements
 // before and after each array (plane), every array starting on a 256-byte
 // boundary; planes of one level are plane_stride32(n) elements apart.  The
