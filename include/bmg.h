@@ -127,7 +127,7 @@ typedef struct {
   int inner_cycles;     /* FP32 V-cycles per refinement step (0 = 1) */
   int bf16_levels;      /* levels with BF16 stencils under BMG_BF16_IR (0 = 2) */
   int use_graph;        /* 1 (default): replay one captured CUDA graph per cycle, autotune the
-                           row-kernel tiles and run the coarse levels (n <= 63 FP32, n <= 15 FP64)
+                           row-kernel tiles and run the coarse levels (n <= 63 FP32, n <= 31 FP64)
                            as one level-fused launch; 0: plain launches, one per step */
   int krylov;           /* BMG_KRYLOV_NONE (default): stationary V-cycle iteration;
                            BMG_KRYLOV_FCG: flexible CG with one cycle as preconditioner */

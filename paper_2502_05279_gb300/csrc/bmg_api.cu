@@ -332,7 +332,7 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
   cudaStream_t s = h->ws;
   if (l == h->tail_l) {
     step(h, l, BMG_K_TAIL, 0,
-         [&] { launch_tail<double>((const TailDesc<double>*)h->d_tail, 1, L.n, done, s, L.fused); });
+         [&] { launch_tail<double>((const TailDesc<double>*)h->d_tail, 1, L.n, h->nlev - l, done, s, L.fused); });
     return;
   }
   if (l == h->nlev - 1) {
@@ -421,7 +421,7 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done) {
   cudaStream_t s = h->ws;
   if (l == h->tail_l) {
     step(h, l, BMG_K_TAIL, 1,
-         [&] { launch_tail<float>((const TailDesc<float>*)h->d_tail, 1, L.n, done, s, L.fused); });
+         [&] { launch_tail<float>((const TailDesc<float>*)h->d_tail, 1, L.n, h->nlev - l, done, s, L.fused); });
     return;
   }
   if (l == h->nlev - 1) {
@@ -833,6 +833,7 @@ int build_tail(bmg_hierarchy* h, int lmin) {
   d.nu1 = h->nu1;
   d.nu2 = h->nu2;
   d.top_kind = h->lv[lt].kind;
+  d.zero = lt > 0;
   d.done = nullptr;
   for (int k = 0; k < d.nlev; ++k) {
     Level& L = h->lv[lt + k];
@@ -1989,7 +1990,7 @@ void append_desc(bmg_batch::Group& g, const LevelDesc<T, S>& d) {
 // buffers rhs/x and upload them (the device addresses never change, so a
 // captured graph stays valid).  With rhs == NULL only the group sizes are set.
 // First level of problem p that joins its level-fused tail (-1: none): the
-// rule of the solo hierarchy (FP64 from level 1, n <= 15; FP32 from level 0,
+// rule of the solo hierarchy (FP64 from level 1, n <= 31; FP32 from level 0,
 // n <= 63, not BF16), only when graphs are in use.
 int batch_tail_level(bmg_batch* B, bmg_hierarchy* h) {
   if (!B->use_graph) return -1;
@@ -2007,6 +2008,7 @@ void append_tail(bmg_batch* B, bmg_hierarchy* h, int lt, const int* done, int b)
   d.nu1 = B->nu1;
   d.nu2 = B->nu2;
   d.top_kind = h->lv[lt].kind;
+  d.zero = lt > 0;
   d.done = done;
   for (int k = 0; k < d.nlev; ++k) {
     Level& L = h->lv[lt + k];
@@ -2180,11 +2182,11 @@ void batch_vcycle(bmg_batch* B) {
     }
     if (B->tail_count[b]) {   // problems whose remaining levels run in one level-fused launch
       if (B->precision == BMG_FP64)
-        launch_tail<double>((const TailDesc<double>*)B->tail_dev[b], B->tail_count[b], B->tail_n[b], nullptr, B->ws,
-                            B->arith);
+        launch_tail<double>((const TailDesc<double>*)B->tail_dev[b], B->tail_count[b], B->tail_n[b], b + 1, nullptr,
+                            B->ws, B->arith);
       else
-        launch_tail<float>((const TailDesc<float>*)B->tail_dev[b], B->tail_count[b], B->tail_n[b], nullptr, B->ws,
-                           B->arith);
+        launch_tail<float>((const TailDesc<float>*)B->tail_dev[b], B->tail_count[b], B->tail_n[b], b + 1, nullptr,
+                           B->ws, B->arith);
     }
   }
   for (auto& g : B->stages[0]) group_coarse(B, g);

@@ -38,6 +38,41 @@ template <bool FU> __device__ __forceinline__ float msub(float s, float a, float
   return FU ? __fmaf_rn(-a, b, s) : rsub(s, rmul(a, b));
 }
 
+// ---- quotients by a divisor that is known ahead ----
+// s / m, correctly rounded, from y = fl(1/m) and yl = fl(y (1 - m y)), so that
+// y + yl = 1/m to about 2^-104 relative.  q0 = fl(s y + fl(s yl)) is then less
+// than one ulp from s / m, the residual s - m q0 is exact in one FMA, and the
+// last FMA rounds s / m correctly (Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990,
+// theorem on the final quotient step: q0 within one ulp, y the rounded
+// reciprocal, no over- or underflow).  y = 0 marks an m outside 2^[-200, 200];
+// such an m, and an s outside 2^[-623, 623] other than zero, take the division.
+// Four dependent operations of 63 cycles against 560 for the division.  The
+// tests are on the bit patterns: comparisons would use the FP64 pipe.
+static __device__ __noinline__ double quot_slow(double s, double m) { return rdiv(s, m); }
+
+__device__ __forceinline__ double quot(double s, double m, double y, double yl) {
+  // the four operations first: their dependent chain does not wait for the tests
+  const double q0 = __fma_rn(s, y, rmul(s, yl));
+  double q = __fma_rn(__fma_rn(-m, q0, s), y, q0);
+  const unsigned hs = (unsigned)__double2hiint(s), es = (hs >> 20) & 0x7ffu;
+  if (es - 400u > 1246u || __double2hiint(y) == 0) {
+    if (__double2hiint(y) != 0 && (hs << 1) == 0 && __double2loint(s) == 0)   // +-0 / m
+      q = __hiloint2double((int)((hs ^ (unsigned)__double2hiint(m)) & 0x80000000u), 0);
+    else
+      q = quot_slow(s, m);
+  }
+  return q;
+}
+
+__device__ __forceinline__ double quot_recip(double m, double* yl) {
+  const unsigned e = ((unsigned)__double2hiint(m) >> 20) & 0x7ffu;
+  const bool ok = e - 823u <= 400u;
+  const double y = ok ? rdiv(1.0, m) : 0.0;
+  *yl = ok ? rmul(__fma_rn(-m, y, 1.0), y) : 0.0;
+  return y;
+}
+
 // ---- storage -> compute conversion (exact for every pair used) ----
 template <typename T> __device__ __forceinline__ T cvt(double v) { return (T)v; }
 template <typename T> __device__ __forceinline__ T cvt(float v) { return (T)v; }

@@ -1445,45 +1445,7 @@ __device__ __forceinline__ void finalize_body(const double* __restrict__ partial
   ctl->scale_next = scale_of(rho);
 }
 
-// ---- coarsest solve: forward and back substitution ------------------------------------
-// L L^T x = f with every thread of the block taking part.  Forward, right-looking:
-// once y_k = s_k / L_kk is known, every row i > k subtracts L_ik y_k; each row still
-// receives its terms in increasing k, the order of the row-by-row loop, so the
-// result is the same bits.  Backward, thread 0: row i's sum runs over k = i+1 .. m-1
-// in increasing order and starts with x_{i+1}, so the rows form one chain.  The
-// factor is staged in shared memory when it is small (a chain through L2 would
-// pay a round trip per term).  y is unused (kept for the callers' layout).
 constexpr int COARSE_M_MAX = 225;   // coarsest level n <= 15
-constexpr int COARSE_M_SMEM = 9;    // factors of m <= 9 unknowns (n = 3) go to shared memory
-template <typename T>
-__device__ __forceinline__ void coarse_solve_body(int n, const double* __restrict__ L, const T* __restrict__ f,
-                                                  T* __restrict__ x, double* __restrict__ y) {
-  __shared__ double ys[COARSE_M_MAX];
-  __shared__ double Ls[COARSE_M_SMEM * COARSE_M_SMEM];
-  (void)y;
-  const int m = n * n, ld = n + 2;
-  const bool staged = m <= COARSE_M_SMEM;
-  const double* Lp = staged ? Ls : L;
-  for (int k = threadIdx.x; k < m; k += blockDim.x) ys[k] = (double)f[(size_t)(k / n + 1) * ld + (k % n + 1)];
-  if (staged)
-    for (int k = threadIdx.x; k < m * m; k += blockDim.x) Ls[k] = L[k];
-  __syncthreads();
-  for (int k = 0; k < m; ++k) {
-    if (threadIdx.x == 0) ys[k] = rdiv(ys[k], Lp[(size_t)k * m + k]);
-    __syncthreads();
-    const double yk = ys[k];
-    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) ys[i] = rsub(ys[i], rmul(Lp[(size_t)i * m + k], yk));
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int i = m - 1; i >= 0; --i) {
-      double s = ys[i];
-      for (int k = i + 1; k < m; ++k) s = rsub(s, rmul(Lp[(size_t)k * m + i], ys[k]));   // ys[k] = x_k
-      ys[i] = rdiv(s, Lp[(size_t)i * m + i]);
-    }
-  __syncthreads();
-  for (int k = threadIdx.x; k < m; k += blockDim.x) x[(size_t)(k / n + 1) * ld + (k % n + 1)] = (T)ys[k];
-}
 
 // ---- iterative refinement ------------------------------------------------------------------
 // s * fl64(e) for a positive normal power of two s (the refinement scales).
@@ -1609,112 +1571,8 @@ struct TailDesc {
   int nlev;     // levels in lv (the last is the coarsest)
   int nu1, nu2;
   int top_kind; // stencil kind of lv[0] (5 or 9); the levels below are 9-point
+  int zero;     // 1: the top level's iterate is zero on entry (it is a coarse level of the cycle)
   const int* done;
 };
 
-namespace dev {
-
-// Half of a four-colour sweep over one CTA: the rows of parity pj, their odd-i
-// points, a barrier, their even-i points, a barrier (the order of k_gs_rows).
-template <typename T, typename S, bool FU = false>
-__device__ __forceinline__ void gs_half_block(const StencilView<T, S>& v, const T* f, T* x, int pj) {
-  const int n = v.n;
-  const int R = pj ? (n + 1) / 2 : (n - 1) / 2;
-  const int Po = (n + 1) / 2, Pe = (n - 1) / 2;
-  for (int k = threadIdx.x; k < R * Po; k += blockDim.x) {
-    int j = 2 * (k / Po) + (pj ? 1 : 2), i = 2 * (k % Po) + 1;
-    gs_point<T, S, true, FU>(v, f, x, (size_t)j * v.ld + i);
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < R * Pe; k += blockDim.x) {
-    int j = 2 * (k / Pe) + (pj ? 1 : 2), i = 2 * (k % Pe) + 2;
-    gs_point<T, S, true, FU>(v, f, x, (size_t)j * v.ld + i);
-  }
-  __syncthreads();
-}
-
-// One red-black colour over one CTA (5-point levels).
-template <typename T, typename S, bool FU = false>
-__device__ __forceinline__ void gs_checker_block(const StencilView<T, S>& v, const T* f, T* x, int c) {
-  const int n = v.n;
-  const int per_row = (n + 1) / 2;
-  for (int k = threadIdx.x; k < n * per_row; k += blockDim.x) {
-    int j = k / per_row + 1;
-    int i = 2 * (k % per_row) + 1 + ((j + 1 + c) & 1);
-    if (i <= n) gs_point<T, S, false, FU>(v, f, x, (size_t)j * v.ld + i);
-  }
-  __syncthreads();
-}
-
-template <typename T, bool FU = false>
-__device__ __forceinline__ void relax_block(const LevelDesc<T, T>& q, int kind, int sweeps) {
-  for (int s = 0; s < sweeps; ++s) {
-    if (kind == 9) {
-      gs_half_block<T, T, FU>(q.v, q.f, q.x, 1);
-      gs_half_block<T, T, FU>(q.v, q.f, q.x, 0);
-    } else {
-      gs_checker_block<T, T, FU>(q.v, q.f, q.x, 0);
-      gs_checker_block<T, T, FU>(q.v, q.f, q.x, 1);
-    }
-  }
-}
-
-// Residual + Fig. 2 restriction, one coarse point per thread iteration; the
-// nine fine residuals are formed where they are needed (same values as the
-// tiled kernel: each is the same expression of the same data).
-template <typename T, bool NINE, bool FU = false>
-__device__ __forceinline__ void resid_restrict_block(const LevelDesc<T, T>& q) {
-  const StencilView<T, T>& v = q.v;
-  const int n = v.n, ld = v.ld, nc = (n - 1) / 2, ldc = nc + 2;
-  const size_t psc = plane_size(nc);
-  for (int k = threadIdx.x; k < nc * nc; k += blockDim.x) {
-    int ic = k % nc + 1, jc = k / nc + 1;
-    size_t pf = (size_t)(2 * jc) * ld + 2 * ic;
-    auto r = [&](int dx, int dy) {
-      size_t p = pf + (size_t)((long long)dy * ld + dx);
-      return row_residual<T, T, NINE, true, FU>(v, q.x, p, q.f[p]);
-    };
-    auto w = [&](int kk, int dic, int djc) { return q.ci[kk * psc + (size_t)(jc + djc) * ldc + (ic + dic)]; };
-    T t = rmul(w(CI_LNE, 0, 0), r(-1, -1));
-    t = madd<FU>(t, w(CI_LA, 0, 0), r(0, -1));
-    t = madd<FU>(t, w(CI_LNW, 1, 0), r(1, -1));
-    t = madd<FU>(t, w(CI_LR, 0, 0), r(-1, 0));
-    t = radd(t, r(0, 0));
-    t = madd<FU>(t, w(CI_LL, 1, 0), r(1, 0));
-    t = madd<FU>(t, w(CI_LSE, 0, 1), r(-1, 1));
-    t = madd<FU>(t, w(CI_LB, 0, 1), r(0, 1));
-    t = madd<FU>(t, w(CI_LSW, 1, 1), r(1, 1));
-    size_t pc = (size_t)jc * ldc + ic;
-    if (BMG_IN(DBG_RESTRICT_STORE, pc, (size_t)ldc * ldc)) {
-      q.fc[pc] = t;
-      q.xc[pc] = T(0);
-    }
-  }
-  __syncthreads();
-}
-
-template <typename T, bool FU = false>
-__device__ __forceinline__ void tail_body(const TailDesc<T>& d, int top_kind) {
-  for (int l = 0; l + 1 < d.nlev; ++l) {
-    const int kind = l == 0 ? top_kind : 9;
-    relax_block<T, FU>(d.lv[l], kind, d.nu1);
-    if (kind == 9)
-      resid_restrict_block<T, true, FU>(d.lv[l]);
-    else
-      resid_restrict_block<T, false, FU>(d.lv[l]);
-  }
-  const LevelDesc<T, T>& c = d.lv[d.nlev - 1];
-  coarse_solve_body<T>(c.v.n, c.L, c.f, c.x, c.y);
-  __syncthreads();
-  for (int l = d.nlev - 2; l >= 0; --l) {
-    const LevelDesc<T, T>& q = d.lv[l];
-    const int nc = (q.v.n - 1) / 2;
-    for (int k = threadIdx.x; k < (nc + 1) * (nc + 1); k += blockDim.x)
-      interp_body<T, FU>(q.v.n, q.ci, q.xc, q.x, q.x, k % (nc + 1) + 1, k / (nc + 1) + 1);
-    __syncthreads();
-    relax_block<T, FU>(q, l == 0 ? top_kind : 9, d.nu2);
-  }
-}
-
-}  // namespace dev
 }  // namespace bmg

@@ -6,7 +6,7 @@
 // the batched kernels.
 #include <cstdint>
 
-#include "cycle_device.cuh"
+#include "block_device.cuh"
 
 namespace bmg {
 
@@ -203,8 +203,7 @@ __global__ void k_coarse_solve(int n, const double* __restrict__ L, const T* __r
                                double* __restrict__ y, const int* done) {
   pdl_enter();
   if (stopped(done)) return;
-  if (blockIdx.x != 0) return;
-  coarse_solve_body<T>(n, L, f, x, y);
+  coarse_body<T>(n, L, f, x);
 }
 
 // x += scale_applied * e32, IRU_COLS points of a row per thread, BX apart.

@@ -16,7 +16,7 @@
 // the factors, and store the previous positions' results, all through shared
 // memory, so that their loads coalesce and their FP64 work runs on the other
 // three quarters of the SM.  Per point the chain is a product, a difference and
-// line_div's four operations forward, and two operations backward: 511 x 8 x 63
+// quot's four operations forward, and two operations backward: 511 x 8 x 63
 // cycles, about 130 us per half sweep at 511^2.
 #include "cycle_device.cuh"
 
@@ -26,31 +26,6 @@ namespace {
 
 constexpr int LC = 32;              // positions per stage
 constexpr int LINE_THREADS = 256;   // warp 0: the chains; warps 1 .. 7: everything else
-
-// s / m, correctly rounded, from y = fl(1/m) and yl = fl(y (1 - m y)), so that
-// y + yl = 1/m to about 2^-104 relative.  q0 = fl(s y + fl(s yl)) is then less
-// than one ulp from s / m, the residual s - m q0 is exact in one FMA, and the
-// last FMA rounds s / m correctly (Markstein, "Computation of elementary
-// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990,
-// theorem on the final quotient step: q0 within one ulp, y the rounded
-// reciprocal, no over- or underflow).  y = 0 marks an m outside 2^[-200, 200];
-// such an m, and an s outside 2^[-623, 623] other than zero, take the division.
-// The tests are on the bit patterns: comparisons would use the FP64 pipe.
-__device__ __noinline__ double line_div_slow(double s, double m) { return rdiv(s, m); }
-
-__device__ __forceinline__ double line_div(double s, double m, double y, double yl) {
-  // the four operations first: their dependent chain does not wait for the tests
-  const double q0 = __fma_rn(s, y, rmul(s, yl));
-  double q = __fma_rn(__fma_rn(-m, q0, s), y, q0);
-  const unsigned hs = (unsigned)__double2hiint(s), es = (hs >> 20) & 0x7ffu;
-  if (es - 400u > 1246u || __double2hiint(y) == 0) {
-    if (__double2hiint(y) != 0 && (hs << 1) == 0 && __double2loint(s) == 0)   // +-0 / m
-      q = __hiloint2double((int)((hs ^ (unsigned)__double2hiint(m)) & 0x80000000u), 0);
-    else
-      q = line_div_slow(s, m);
-  }
-  return q;
-}
 
 // Point of position q (1 .. n) on line w (1 .. n): x-lines run along i, y-lines along j.
 template <int AXIS>
@@ -100,18 +75,15 @@ __global__ void k_line_factor(StencilView<T, S> v, T* __restrict__ c, T* __restr
   }
 }
 
-// y = fl(1/m) and yl = fl(y (1 - m y)) for line_div; y = 0 where it must not be used.
+// m's reciprocal and its remainder for quot.
 __global__ void k_line_recip(int n, const double* __restrict__ m, double* __restrict__ y, double* __restrict__ yl) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x + 1, j = blockIdx.y * blockDim.y + threadIdx.y + 1;
   if (i > n || j > n) return;
   const size_t p = (size_t)j * (n + 2) + i;
   if (!BMG_IN(DBG_LINE_STORE, p, (size_t)(n + 2) * (n + 2))) return;
-  const double mm = m[p];
-  const unsigned e = ((unsigned)__double2hiint(mm) >> 20) & 0x7ffu;
-  const bool ok = e - 823u <= 400u;
-  const double r = ok ? rdiv(1.0, mm) : 0.0;
-  y[p] = r;
-  yl[p] = ok ? rmul(__fma_rn(-mm, r, 1.0), r) : 0.0;
+  double rl;
+  y[p] = quot_recip(m[p], &rl);
+  yl[p] = rl;
 }
 
 // Right-hand side of p: f minus the couplings to the two fixed lines, in the
@@ -213,7 +185,7 @@ __global__ void __launch_bounds__(LINE_THREADS)
       for (int t = 0; t < cnt; ++t) {
         const T s = k + t == 0 ? b.g[r][t] : rsub(b.g[r][t], rmul(b.a[r][t], d));
         if constexpr (sizeof(T) == 8)
-          d = line_div(s, b.m[r][t], b.y[r][t], b.yl[r][t]);
+          d = quot(s, b.m[r][t], b.y[r][t], b.yl[r][t]);
         else
           d = rdiv(s, b.m[r][t]);
         b.out[r][t] = d;
