@@ -193,6 +193,7 @@ struct Level {
   double* x64b = nullptr; // second iterate of an FP64 level swept by the one-pass kernel
   float* pk32 = nullptr;  // the FP32 / BF16 stencil packed per point (StencilView::pk)
   int pair_rr = 0;        // 1: the two pre-smoothing sweeps, the residual and the restriction in one pass
+  int lrows = 0;          // > 0: the level's halves of the cycle run as one launch each, tiles of this many block rows
 };
 
 StencilView<double, double> view64(const Level& L) {
@@ -327,6 +328,9 @@ void gfree(T* p) {
   if (p) cudaFree(p - STRIP_GUARD);
 }
 
+// Level l >= 1 starts its part of the cycle from a zero iterate without reading one.
+bool zero_aware(const bmg_hierarchy* h, int l) { return l == h->tail_l || (h->lv[l].lrows > 0 && !h->prof); }
+
 void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* done) {
   Level& L = h->lv[l];
   cudaStream_t s = h->ws;
@@ -341,6 +345,14 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
   }
   auto v = view64(L);
   Level& C = h->lv[l + 1];
+  if (L.lrows > 0 && !h->prof) {   // one launch down, one up; the result is in x as below
+    launch_level_down(v, L.kind, (const double*)L.ci, f, l > 0 ? (const double*)nullptr : (const double*)x, L.x64b,
+                      C.f, zero_aware(h, l + 1) ? (double*)nullptr : C.x, h->nu1, L.lrows, done, s);
+    vcycle64(h, l + 1, C.x, C.f, done);
+    launch_level_up(v, L.kind, (const double*)L.ci, (const double*)C.x, f, (const double*)L.x64b, x, h->nu2, L.lrows,
+                    done, s);
+    return;
+  }
   // One-pass level: each sweep reads *cur and writes the other of x / x64b;
   // the interpolation writes the array from which nu2 sweeps end in x.
   double* cur = x;
@@ -430,6 +442,21 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done) {
     return;
   }
   Level& C = h->lv[l + 1];
+  if (L.lrows > 0 && !h->prof) {   // one launch down, one up
+    auto both = [&](const auto& v) {
+      launch_level_down(v, L.kind, (const float*)L.ci32, (const float*)L.f32,
+                        l > 0 ? (const float*)nullptr : (const float*)L.x32, L.x32b, C.f32,
+                        zero_aware(h, l + 1) ? (float*)nullptr : C.x32, h->nu1, L.lrows, done, s);
+      vcycle32(h, l + 1, done);
+      launch_level_up(v, L.kind, (const float*)L.ci32, (const float*)C.x32, (const float*)L.f32,
+                      (const float*)L.x32b, L.x32, h->nu2, L.lrows, done, s);
+    };
+    if (L.bf16)
+      both(viewbf(L));
+    else
+      both(view32(L));
+    return;
+  }
   float* cur = L.x32;
   auto pre = [&](const auto& v) {
     if (L.pair_rr && h->nu1 == 2) {   // temporal blocking: sweeps, residual and restriction in one pass
@@ -749,7 +776,7 @@ int tune_level32(Level& L, const StencilView<float, S>& v, cudaStream_t s) {
   if (!rc) rc = tune_tile(v, s, &shape, &ms_tile);
   if (rc) return rc;
   if (ms_tile < ms_rows) {
-    if ((rc = galloc(&L.x32b, L.n, 1, s))) return rc;
+    if (!L.x32b && (rc = galloc(&L.x32b, L.n, 1, s))) return rc;
     L.tile32 = shape;
     int pshape = -1;
     float ms_pair = 0;
@@ -811,8 +838,45 @@ int tune_level64(Level& L, cudaStream_t s) {
   if (!rc) rc = tune_tile64(view64(L), s, &shape, &ms_tile);
   if (rc) return rc;
   if (ms_tile < ms_rows) {
-    if ((rc = dalloc_zero(&L.x64b, plane_size(L.n), s))) return rc;
+    if (!L.x64b && (rc = dalloc_zero(&L.x64b, plane_size(L.n), s))) return rc;
     L.tile64 = shape;
+  }
+  return BMG_OK;
+}
+
+// Block rows per tile of a level whose halves of the cycle run as one launch
+// each (0: its steps are launched separately).  The change of a whole cycle
+// when one level runs by halves, us, fused arithmetic (8 / 16 / 32 rows):
+//   FP64  63: -15 / -6    127: -12 / -4    255: -3 / -10   511: 0 / -17   1023: +121 / +55
+//   FP32  127: -11 / -11 / -11   255: -14 / -13 / -11   511: -12 / -15 / -17
+//         1023: +4 / -13 / -9    2047: +66 / -2 / +12
+// (one rounding per operation: within a few us of these).  Small FP64 levels
+// want few warps per SM quarter, each of whose FP64 instructions takes 60
+// cycles; larger ones a small halo.  In FP32 32 rows pay while their tiles,
+// one to an SM, fit the chip at once.
+int level_rows(bool f64, int n) {
+  if (f64) return n > 511 || n < 31 ? 0 : n <= 127 ? 8 : 16;
+  return n > 1023 || n < 31 ? 0 : n == 511 ? 32 : 16;
+}
+
+// Whether levels of the hierarchy may run by halves: graphs on, nothing forced,
+// sweep counts that the tiles' halos allow.
+bool by_halves(const bmg_hierarchy* h) {
+  return h->use_graph && h->smoother == BMG_SMOOTHER_AUTO && h->fuse_restrict == BMG_FUSE_AUTO && h->nu1 >= 1 &&
+         h->nu2 >= 1 && h->nu1 <= LEVEL_NU_MAX && h->nu2 <= LEVEL_NU_MAX;
+}
+
+// The levels that run by halves, and their second iterates.
+int choose_level_halves(bmg_hierarchy* h) {
+  if (!by_halves(h)) return BMG_OK;
+  const bool f64 = h->precision == BMG_FP64;
+  for (int l = 0; l + 1 < h->nlev; ++l) {
+    Level& L = h->lv[l];
+    if (h->tail_l >= 0 && l >= h->tail_l) break;
+    L.lrows = level_rows(f64, L.n);
+    if (L.lrows <= 0) continue;
+    int rc = f64 ? dalloc_zero(&L.x64b, plane_size(L.n), h->ws) : galloc(&L.x32b, L.n, 1, h->ws);
+    if (rc) return rc;
   }
   return BMG_OK;
 }
@@ -822,8 +886,11 @@ int tune_level64(Level& L, cudaStream_t s) {
 template <typename T>
 int build_tail(bmg_hierarchy* h, int lmin) {
   int lt = -1;
+  // In FP64 the 31^2 level takes 12 us (23 us with one rounding per operation)
+  // of the tail's one SM and 9 us by halves over several.
+  const int nmax = sizeof(T) == 8 && by_halves(h) ? 15 : tail_max_n<T>();
   for (int l = lmin; l + 1 < h->nlev; ++l)
-    if (h->lv[l].n <= tail_max_n<T>() && !h->lv[l].bf16) {
+    if (h->lv[l].n <= nmax && !h->lv[l].bf16) {
       lt = l;
       break;
     }
@@ -916,7 +983,7 @@ int autotune_solo(bmg_hierarchy* h) {
   std::lock_guard<std::mutex> guard(tune_lock());
   for (int l = 0; l + 1 < h->nlev; ++l) {
     Level& L = h->lv[l];
-    if (L.kind != 9 || L.n < 127) continue;
+    if (L.kind != 9 || L.n < 127 || (l > 0 && L.lrows > 0)) continue;
     int rc = BMG_OK;
     if (h->precision == BMG_FP64)
       rc = h->smoother == BMG_SMOOTHER_AUTO ? tune_level64(L, h->ws)
@@ -988,7 +1055,7 @@ int choose_pair_restrict(bmg_hierarchy* h) {
   for (int l = 0; l + 1 < h->nlev; ++l) {
     if (h->tail_l >= 0 && l >= h->tail_l) break;
     Level& L = h->lv[l];
-    if (L.kind != 9 || L.tile32 < 0 || L.pair32 < 0) continue;
+    if (L.kind != 9 || L.tile32 < 0 || L.pair32 < 0 || L.lrows > 0) continue;
     if (h->fuse_restrict == BMG_FUSE_ON) {
       L.pair_rr = 1;
       continue;
@@ -1435,9 +1502,10 @@ int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* o, bmg_hiera
   const bool line = is_line(h->smoother);
   if (!rc && line) rc = build_lines(h);
   if (!rc && !line && h->smoother >= BMG_SMOOTHER_TILE) rc = force_tile(h);
-  if (!rc && !line && h->use_graph) rc = autotune_solo(h);
   if (!rc && !line && h->use_graph)   // the level-fused tail relaxes by points
     rc = h->precision == BMG_FP64 ? build_tail<double>(h, 1) : build_tail<float>(h, 0);
+  if (!rc && !line) rc = choose_level_halves(h);
+  if (!rc && !line && h->use_graph) rc = autotune_solo(h);
   if (!rc && !line) rc = choose_pair_restrict(h);
   if (!rc) rc = ensure_ctl(h, 64);
   if (rc) {

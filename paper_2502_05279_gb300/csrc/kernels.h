@@ -123,6 +123,20 @@ bool launch_gs_pair(const StencilView<float, S>& v, const float* f, const float*
 constexpr int GS_TILE64_SHAPES = 4;
 void launch_gs_tile64(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                       int shape, const int* done, cudaStream_t s);
+// One level's half of the cycle in one launch (k_level.cu), tiles of 32 x rows
+// blocks of 2 x 2 points (rows <= 16 in FP64, 32 in FP32).  down: nu1 sweeps on
+// xin (NULL: zero) into xout, the residual restricted into fc, and xc (may be
+// NULL) zeroed.  up: xout = nu2 sweeps on xin + P ec.  xout != xin; 1 <= nu <=
+// LEVEL_NU_MAX and rows >= 2 nu1 + 4.  The same bits as the separate launches.
+// v, ci, and for up also f and xin, must have been written before the launch
+// that precedes on the stream started.
+constexpr int LEVEL_NU_MAX = 2;
+template <typename T, typename S>
+void launch_level_down(const StencilView<T, S>& v, int kind, const T* ci, const T* f, const T* xin, T* xout, T* fc,
+                       T* xc, int nu1, int rows, const int* done, cudaStream_t s);
+template <typename T, typename S>
+void launch_level_up(const StencilView<T, S>& v, int kind, const T* ci, const T* ec, const T* f, const T* xin,
+                     T* xout, int nu2, int rows, const int* done, cudaStream_t s);
 template <typename T, typename S>
 void launch_resid_restrict(const StencilView<T, S>& v, int kind, const T* ci, const T* x, const T* f, T* fc,
                            T* xc, const int* done, cudaStream_t s);
