@@ -946,29 +946,33 @@ int force_tile(bmg_hierarchy* h) {
 // level, for the axes the smoother uses.
 int build_lines(bmg_hierarchy* h) {
   const int dir = line_dir(h->smoother);
+  LineJobs<double, double> j64;
+  LineJobs<float, float> j32;
+  LineJobs<float, __nv_bfloat16> jbf;
   for (int l = 0; l + 1 < h->nlev; ++l) {
     Level& L = h->lv[l];
     const size_t ps = plane_size(L.n);
     for (int axis = 0; axis < 2; ++axis) {
       if (dir == (axis == 0 ? LINE_Y : LINE_X)) continue;
-      if (h->precision == BMG_FP64) {
-        LineFactor<double>& F = L.lfac[axis];
-        if (int rc = dalloc(&F.c, 4 * ps)) return rc;
+      auto add = [&](auto& jobs, const auto& v, auto& F, int arrays) {
+        if (int rc = dalloc(&F.c, arrays * ps)) return rc;
         F.m = F.c + ps;
-        F.y = F.m + ps;
-        F.yl = F.y + ps;
-        launch_line_factor(view64(L), axis, F, h->ws);
-      } else {
-        LineFactor<float>& F = L.lfac32[axis];
-        if (int rc = dalloc(&F.c, 2 * ps)) return rc;
-        F.m = F.c + ps;
-        if (L.bf16)
-          launch_line_factor(viewbf(L), axis, F, h->ws);
-        else
-          launch_line_factor(view32(L), axis, F, h->ws);
-      }
+        if (arrays == 4) {
+          F.y = F.m + ps;
+          F.yl = F.y + ps;
+        }
+        jobs.job[jobs.count++] = {v.O, axis == 0 ? v.W : v.S_, F.c, F.m, L.n, axis};
+        return (int)BMG_OK;
+      };
+      const int rc = h->precision == BMG_FP64 ? add(j64, view64(L), L.lfac[axis], 4)
+                     : L.bf16                 ? add(jbf, viewbf(L), L.lfac32[axis], 2)
+                                              : add(j32, view32(L), L.lfac32[axis], 2);
+      if (rc) return rc;
     }
   }
+  launch_line_factor(j64, h->ws);
+  launch_line_factor(j32, h->ws);
+  launch_line_factor(jbf, h->ws);
   return cuda_check(cudaGetLastError(), "line factors");
 }
 

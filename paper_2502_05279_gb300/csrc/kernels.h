@@ -64,14 +64,30 @@ void launch_line(const StencilView<T, S>& v, int kind, const T* f, T* x, T* cp, 
 // The factored form a hierarchy uses (k_line.cu): per axis and level the
 // multipliers c and pivots m of every line's elimination, and in FP64 m's
 // rounded reciprocal y with its remainder yl, arrays of the level's (n+2)^2
-// layout filled by launch_line_factor (axis 0: x-lines, 1: y-lines).  fx, fy:
+// layout filled by launch_line_factor.  fx, fy:
 // the factors of the axes that dir needs.  The same results as launch_line.
 template <typename T>
 struct LineFactor {
   T *c = nullptr, *m = nullptr, *y = nullptr, *yl = nullptr;
 };
+// The lines of one level and axis to be factored: diagonal o, the plane of
+// couplings to the previous point (W for x-lines, S for y-lines), c and m, and
+// in FP64 y and yl in the two arrays after m.
 template <typename T, typename S>
-void launch_line_factor(const StencilView<T, S>& v, int axis, const LineFactor<T>& fac, cudaStream_t s);
+struct LineJob {
+  const T* o;
+  const S* prev;
+  T *c, *m;
+  int n, axis;
+};
+constexpr int LINE_JOBS = 32;   // two axes of up to 16 levels
+template <typename T, typename S>
+struct LineJobs {
+  LineJob<T, S> job[LINE_JOBS];
+  int count = 0;
+};
+template <typename T, typename S>
+void launch_line_factor(const LineJobs<T, S>& jobs, cudaStream_t s);
 template <typename T, typename S>
 void launch_line_solve(const StencilView<T, S>& v, int kind, const T* f, T* x, const LineFactor<T>& fx,
                        const LineFactor<T>& fy, int sweeps, int dir, const int* done, cudaStream_t s);
