@@ -27,6 +27,8 @@ struct bmg_mlp {
   float *tg_X = nullptr, *tg_Z1 = nullptr, *tg_Z2 = nullptr, *tg_out = nullptr, *tg_dout = nullptr,
         *tg_partial = nullptr;
   int* tg_err = nullptr;
+  size_t tg_aux_count = 0;
+  double* tg_aux = nullptr;
 };
 
 #define CK(call)                               \
@@ -76,26 +78,30 @@ int ensure_ws(bmg_mlp* m, int n, int K) {
 bool level_size_ok(int n) { return n >= 3 && ((n + 1) & n) == 0; }
 
 void free_tg(bmg_mlp* m) {
-  void* ptrs[] = {m->tg_X, m->tg_Z1, m->tg_Z2, m->tg_out, m->tg_dout, m->tg_partial, m->tg_err};
+  void* ptrs[] = {m->tg_X, m->tg_Z1, m->tg_Z2, m->tg_out, m->tg_dout, m->tg_partial, m->tg_err, m->tg_aux};
   for (void* p : ptrs) cudaFree(p);
   m->tg_X = m->tg_Z1 = m->tg_Z2 = m->tg_out = m->tg_dout = m->tg_partial = nullptr;
   m->tg_err = nullptr;
-  m->tg_rows = 0;
+  m->tg_aux = nullptr;
+  m->tg_rows = m->tg_aux_count = 0;
 }
 
-int ensure_tg(bmg_mlp* m, size_t rows) {
-  if (rows <= m->tg_rows) return BMG_OK;
+int ensure_tg(bmg_mlp* m, size_t rows, size_t aux) {
+  if (rows <= m->tg_rows && aux <= m->tg_aux_count) return BMG_OK;
+  if (rows < m->tg_rows) rows = m->tg_rows;
+  if (aux < m->tg_aux_count) aux = m->tg_aux_count;
   free_tg(m);
   int rc;
   if ((rc = alloc0(&m->tg_X, rows * MLP_IN)) || (rc = alloc0(&m->tg_Z1, rows * MLP_HID)) ||
       (rc = alloc0(&m->tg_Z2, rows * MLP_HID)) || (rc = alloc0(&m->tg_out, rows * MLP_OUT)) ||
       (rc = alloc0(&m->tg_dout, rows * MLP_OUT)) ||
       (rc = alloc0(&m->tg_partial, (size_t)mlp_backward_blocks((int)rows) * MLP_PARAMS)) ||
-      (rc = alloc0(&m->tg_err, 1))) {
+      (rc = alloc0(&m->tg_err, 1)) || (rc = alloc0(&m->tg_aux, aux))) {
     free_tg(m);
     return rc;
   }
   m->tg_rows = rows;
+  m->tg_aux_count = aux;
   return BMG_OK;
 }
 
@@ -107,13 +113,10 @@ int mlp_level0_interp(const void* mp, int n, const double* st, double* ci, cudaS
   const bmg_mlp* m = (const bmg_mlp*)mp;
   int nc = (n - 1) / 2;
   size_t M = (size_t)nc * nc;
-  float *X = nullptr, *delta = nullptr;
-  CK(cudaMallocAsync((void**)&X, M * MLP_IN * sizeof(float), s));
+  float* delta = nullptr;
   CK(cudaMallocAsync((void**)&delta, M * MLP_OUT * sizeof(float), s));
-  launch_features(n, st, X, s);
-  launch_mlp_infer(X, (int)M, m->par, delta, s);
+  launch_mlp_infer(n, st, m->par, delta, s);
   launch_learned_ci(n, st, delta, ci, nullptr, s);
-  CK(cudaFreeAsync(X, s));
   CK(cudaFreeAsync(delta, s));
   return cuda_check(cudaGetLastError(), "learned interpolation");
 }
@@ -218,7 +221,7 @@ int bmg_mlp_twogrid(bmg_mlp* m, int ncrop, int n, const double* coefs, int K, co
   const size_t rows = (size_t)ncrop * nc * nc;
   if (rows > (size_t)1 << 30) return set_error(BMG_EINVAL, "bmg_mlp_twogrid: too many crops");
   int rc;
-  if ((rc = ensure_tg(m, rows))) return rc;
+  if ((rc = ensure_tg(m, rows, (size_t)ncrop * 4 * plane_size(nc)))) return rc;
   CK(cudaMemsetAsync(m->tg_err, 0, sizeof(int), s));
   const float* delta = nullptr;
   if (eref) {
@@ -226,7 +229,8 @@ int bmg_mlp_twogrid(bmg_mlp* m, int ncrop, int n, const double* coefs, int K, co
     launch_mlp_fwd(m->tg_X, (int)rows, m->par, m->tg_Z1, m->tg_Z2, m->tg_out, s);
     delta = m->tg_out;
   }
-  if ((rc = launch_twogrid(n, ncrop, K, coefs, vecs, delta, eref, 1.0 / ncrop, energies, m->tg_dout, m->tg_err, s)))
+  if ((rc = launch_twogrid(n, ncrop, K, coefs, vecs, delta, eref, 1.0 / ncrop, energies, m->tg_dout, m->tg_aux,
+                           m->tg_err, s)))
     return rc;
   int bad = 0;
   CK(cudaMemcpyAsync(&bad, m->tg_err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -259,13 +263,7 @@ int bmg_mlp_adam(bmg_mlp* m, float lr, void* stream) {
 int bmg_mlp_infer(const bmg_mlp* m, int n, const double* coef, float* delta, void* stream) {
   if (!m || !level_size_ok(n) || !coef || !delta) return set_error(BMG_EINVAL, "bmg_mlp_infer: bad argument");
   cudaStream_t s = (cudaStream_t)stream;
-  int nc = (n - 1) / 2;
-  size_t M = (size_t)nc * nc;
-  float* X = nullptr;
-  CK(cudaMallocAsync((void**)&X, M * MLP_IN * sizeof(float), s));
-  launch_features(n, coef, X, s);
-  launch_mlp_infer(X, (int)M, m->par, delta, s);
-  CK(cudaFreeAsync(X, s));
+  launch_mlp_infer(n, coef, m->par, delta, s);
   CK(cudaGetLastError());
   return cuda_check(cudaStreamSynchronize(s), "bmg_mlp_infer");
 }

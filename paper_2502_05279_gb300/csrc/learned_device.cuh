@@ -19,11 +19,39 @@ __device__ __forceinline__ double delta_at(const float* delta, int nc, int ic, i
   return (double)delta[((size_t)(jc - 1) * nc + (ic - 1)) * MLP_OUT + k];
 }
 
+// fl32(fl64(s / o)) for both feature sums s of a point over its diagonal o.  The
+// quotients are formed to about 2^-39 from one reciprocal (the hardware's
+// approximation and one Newton step) and rounded to 24 bits on the bit pattern;
+// only where a quotient lies within about 2^-36 of a rounding boundary, or outside
+// 2^[-100, 100], is it divided out: six FP64 operations a point, against about
+// 22 with two divisions (FP64 is what bounds the features).
+static __device__ __noinline__ float feature_slow(double s, double o) { return __double2float_rn(rdiv(s, o)); }
+
+__device__ __forceinline__ float feature_round(double q, double s, double o) {
+  const unsigned hi = (unsigned)__double2hiint(q), lo = (unsigned)__double2loint(q), e = (hi >> 20) & 0x7ffu;
+  const unsigned low = lo & 0x1fffffffu;           // the 29 bits that rounding drops; half is 2^28
+  if (e - 923u > 200u || low - 0x0ffe0000u <= 0x40000u) return feature_slow(s, o);
+  const unsigned bits = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  return __uint_as_float(bits + (low >> 28));      // (a carry moves into the exponent, as it should)
+}
+
+__device__ __forceinline__ float2 feature_pair(double w, double e, double s, double n, double o) {
+  const double sx = radd(w, e), sy = radd(s, n);
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(o));
+  y = __fma_rn(y, __fma_rn(-o, y, 1.0), y);
+  return make_float2(feature_round(sx * y, sx, o), feature_round(sy * y, sy, o));
+}
+
+// exp(second logit) / exp(first logit): one exponential (about 25 FP64
+// operations) per edge point instead of two.
+__device__ __forceinline__ double logit_ratio(double second, double first) { return exp(rsub(second, first)); }
+
 // Edge points of cell (ic, jc), 0 <= ic, jc <= nc+1: x-edge (2ic-1, 2jc) between
 // (ic-1, jc) [its E logit] and (ic, jc) [its W logit]; y-edge (2ic, 2jc-1)
 // between (ic, jc-1) [N logit] and (ic, jc) [S logit].  An edge point keeps
 // Dendy's total weight S_D = -(col_1 + col_2)/D and splits it in the shares
-// u_k = -col_k exp(logit).  aux (optional, 4 coarse planes) keeps S_D and the
+// u_k = -col_k exp(logit), both divided by exp(first logit).  aux (optional, 4 coarse planes) keeps S_D and the
 // first share q for the gradient.
 __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int nc, const float* delta, int ic, int jc,
                                           double* ci, double* aux) {
@@ -36,9 +64,8 @@ __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int n
     double colE = radd(radd(A.a<8>(p, ld), A.a<2>(p, ld)), A.a<6>(p, ld));
     double D = radd(radd(A.a<3>(p, ld), A.a<0>(p, ld)), A.a<4>(p, ld));
     sdx = -rdiv(radd(colW, colE), D);
-    double uW = rmul(-colW, exp(delta_at(delta, nc, ic - 1, jc, 1)));
-    double uE = rmul(-colE, exp(delta_at(delta, nc, ic, jc, 0)));
-    qx = rdiv(uW, radd(uW, uE));
+    double uE = rmul(-colE, logit_ratio(delta_at(delta, nc, ic, jc, 0), delta_at(delta, nc, ic - 1, jc, 1)));
+    qx = rdiv(-colW, radd(-colW, uE));
     ll = rmul(sdx, qx);
     lr = rmul(sdx, rsub(1.0, qx));
   }
@@ -48,9 +75,8 @@ __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int n
     double rowN = radd(radd(A.a<7>(p, ld), A.a<4>(p, ld)), A.a<6>(p, ld));
     double D = radd(radd(A.a<1>(p, ld), A.a<0>(p, ld)), A.a<2>(p, ld));
     sdy = -rdiv(radd(rowS, rowN), D);
-    double uS = rmul(-rowS, exp(delta_at(delta, nc, ic, jc - 1, 3)));
-    double uN = rmul(-rowN, exp(delta_at(delta, nc, ic, jc, 2)));
-    qy = rdiv(uS, radd(uS, uN));
+    double uN = rmul(-rowN, logit_ratio(delta_at(delta, nc, ic, jc, 2), delta_at(delta, nc, ic, jc - 1, 3)));
+    qy = rdiv(-rowS, radd(-rowS, uN));
     lb = rmul(sdy, qy);
     la = rmul(sdy, rsub(1.0, qy));
   }
@@ -82,10 +108,13 @@ __device__ __forceinline__ void centre_cell(const Planes<double>& A, int ld, int
   double lb_e = ci[CI_LB * psc + pc], la_e = ci[CI_LA * psc + pc];
   double ll_s = ci[CI_LL * psc + pc - ldc], lr_s = ci[CI_LR * psc + pc - ldc];
   double ll_n = ci[CI_LL * psc + pc], lr_n = ci[CI_LR * psc + pc];
-  ci[CI_LSW * psc + pc] = -rdiv(radd(radd(aSW, rmul(aW, lb_w)), rmul(aS, ll_s)), aO);
-  ci[CI_LSE * psc + pc] = -rdiv(radd(radd(aSE, rmul(aE, lb_e)), rmul(aS, lr_s)), aO);
-  ci[CI_LNW * psc + pc] = -rdiv(radd(radd(aNW, rmul(aW, la_w)), rmul(aN, ll_n)), aO);
-  ci[CI_LNE * psc + pc] = -rdiv(radd(radd(aNE, rmul(aE, la_e)), rmul(aN, lr_n)), aO);
+  // one division and four quotients by the same divisor (quot rounds as the division does)
+  double yl;
+  const double y = quot_recip(aO, &yl);
+  ci[CI_LSW * psc + pc] = -quot(radd(radd(aSW, rmul(aW, lb_w)), rmul(aS, ll_s)), aO, y, yl);
+  ci[CI_LSE * psc + pc] = -quot(radd(radd(aSE, rmul(aE, lb_e)), rmul(aS, lr_s)), aO, y, yl);
+  ci[CI_LNW * psc + pc] = -quot(radd(radd(aNW, rmul(aW, la_w)), rmul(aN, ll_n)), aO, y, yl);
+  ci[CI_LNE * psc + pc] = -quot(radd(radd(aNE, rmul(aE, la_e)), rmul(aN, lr_n)), aO, y, yl);
 }
 
 }  // namespace learned
