@@ -213,7 +213,55 @@ StencilView<float, __nv_bfloat16> viewbf(const Level& L) {
 
 }  // namespace
 
+namespace {
+// Device memory of one hierarchy (or of one tuning run), given back as a whole
+// when its owner goes.  Arrays are cut from chunks, zeroed when they are made;
+// an array of more than half a chunk gets an allocation of its own.  A
+// cudaMalloc or cudaFree takes 10 to 20 us and a hierarchy has about ninety
+// arrays: at 1023^2 they were half of the 2.0 ms of a setup and all of the 1.2
+// ms of a release.
+struct Arena {
+  std::vector<void*> blocks;
+  char* cur = nullptr;
+  size_t left = 0, chunk = (size_t)2 << 20;
+  Arena() = default;
+  Arena(const Arena&) = delete;
+  Arena& operator=(const Arena&) = delete;
+  ~Arena() {
+    for (void* b : blocks) cudaFree(b);
+  }
+  // Chunks of about four planes of the finest level, 2 to 64 MB.
+  void size_for(int n) {
+    chunk = std::min(std::max(4 * plane_size(n) * sizeof(double), (size_t)2 << 20), (size_t)64 << 20);
+  }
+  int take(void** p, size_t bytes, bool zero, cudaStream_t s) {
+    *p = nullptr;
+    if (alloc_fault()) return cuda_check(cudaErrorMemoryAllocation, "cudaMalloc");
+    bytes = (bytes + 255) & ~(size_t)255;
+    const bool own = bytes > chunk / 2;
+    if (!own && bytes <= left) {
+      *p = cur;
+      cur += bytes;
+      left -= bytes;
+      return BMG_OK;
+    }
+    void* b = nullptr;
+    CK(cudaMalloc(&b, own ? bytes : chunk));
+    blocks.push_back(b);
+    if (zero || !own) CK(cudaMemsetAsync(b, 0, own ? bytes : chunk, s));
+    *p = b;
+    if (!own) {
+      cur = (char*)b + bytes;
+      left = chunk - bytes;
+    }
+    return BMG_OK;
+  }
+};
+
+}  // namespace
+
 struct bmg_hierarchy {
+  Arena mem;              // every device array below but ctl
   int n = 0, nlev = 0, precision = BMG_FP64, nu1 = 2, nu2 = 1, inner = 1, use_graph = 1, coarsest = 3, krylov = 0;
   int interp = BMG_INTERP_DENDY, interp_used = BMG_INTERP_DENDY;
   int smoother = BMG_SMOOTHER_AUTO;
@@ -252,9 +300,6 @@ struct bmg_hierarchy {
   // level-fused tail: levels >= tail_l run in one launch (-1: none)
   int tail_l = -1;
   void* d_tail = nullptr;   // TailDesc<double> or TailDesc<float> in device memory
-  // a batch member that borrows the operator arrays (stencils, weights, Cholesky
-  // factor and its workspace) of another hierarchy and owns only its state
-  bool shared_ops = false;
   // general sizes: the caller's grid nx x ny, embedded in the n x n level 0; the
   // solve runs on the embedded right-hand side and iterate (NULL when nx = ny = n)
   int nx = 0, ny = 0;
@@ -262,6 +307,7 @@ struct bmg_hierarchy {
   double* xpad = nullptr;
   // periodic sides: the hierarchy of periodic.cu (nlev stays 0, lv empty)
   PerHier* per = nullptr;
+  bool member = false;   // a batch member that borrows another hierarchy's operator arrays
 };
 
 namespace {
@@ -291,41 +337,28 @@ void step(bmg_hierarchy* h, int level, int kernel, int fp32, F&& f) {
 }
 
 template <typename T>
-int dalloc(T** p, size_t count) {
+int dalloc(Arena& m, T** p, size_t count, cudaStream_t s) {
   *p = nullptr;
-  if (count == 0) return BMG_OK;
-  CK(dev_malloc((void**)p, count * sizeof(T)));
-  return BMG_OK;
+  return count == 0 ? (int)BMG_OK : m.take((void**)p, count * sizeof(T), false, s);
 }
 
-// dalloc, zeroed on stream s; nothing stays allocated when either step fails.
+// dalloc, zeroed on stream s.
 template <typename T>
-int dalloc_zero(T** p, size_t count, cudaStream_t s) {
-  int rc = dalloc(p, count);
-  if (!rc && count) rc = cuda_check(cudaMemsetAsync(*p, 0, count * sizeof(T), s), "cudaMemsetAsync");
-  if (rc) {
-    cudaFree(*p);
-    *p = nullptr;
-  }
-  return rc;
+int dalloc_zero(Arena& m, T** p, size_t count, cudaStream_t s) {
+  *p = nullptr;
+  return count == 0 ? (int)BMG_OK : m.take((void**)p, count * sizeof(T), true, s);
 }
 
 // FP32 / BF16 level arrays: `planes` planes of level size n, plane_stride32(n)
 // elements apart, with STRIP_GUARD zeroed elements before the first and after
-// every plane; *p is the first plane (256-byte aligned).  Freed by gfree.
+// every plane; *p is the first plane (256-byte aligned).
 template <typename T>
-int galloc(T** p, int n, int planes, cudaStream_t s) {
+int galloc(Arena& m, T** p, int n, int planes, cudaStream_t s) {
   *p = nullptr;
-  const size_t count = STRIP_GUARD + planes * plane_stride32(n);
   T* raw = nullptr;
-  if (int e = dalloc_zero(&raw, count, s)) return e;
+  if (int e = dalloc_zero(m, &raw, STRIP_GUARD + planes * plane_stride32(n), s)) return e;
   *p = raw + STRIP_GUARD;
   return BMG_OK;
-}
-
-template <typename T>
-void gfree(T* p) {
-  if (p) cudaFree(p - STRIP_GUARD);
 }
 
 // Level l >= 1 starts its part of the cycle from a zero iterate without reading one.
@@ -649,7 +682,8 @@ int tune_rows(const StencilView<T, S>& v, cudaStream_t s, int* best_out, float* 
   }
   size_t ps = plane_size(v.n);
   T* scratch = nullptr;
-  if (int e = dalloc_zero(&scratch, 2 * ps, s)) return e;
+  Arena tmp;
+  if (int e = dalloc_zero(tmp, &scratch, 2 * ps, s)) return e;
   float best = 1e30f;
   int best_cl = base, rc = BMG_OK;
   for (int cl = base; cl <= 8 && !rc; cl *= 2) {
@@ -662,7 +696,6 @@ int tune_rows(const StencilView<T, S>& v, cudaStream_t s, int* best_out, float* 
       best_cl = cl;
     }
   }
-  cudaFree(scratch);
   if (rc) return rc;
   cache[key] = {best_cl, best};
   tune_file_put(fkey, TuneRecord{{best_cl}, best});
@@ -691,7 +724,8 @@ int tune_tile(const StencilView<float, S>& v, cudaStream_t s, int* best_out, flo
   }
   size_t ps = plane_stride32(v.n);
   float* scratch = nullptr;   // x, x', f laid out like a level's arrays
-  int rc0 = galloc(&scratch, v.n, 3, s);
+  Arena tmp;
+  int rc0 = galloc(tmp, &scratch, v.n, 3, s);
   if (rc0) return rc0;
   const float* f = scratch + 2 * ps;
   float best = 1e30f;
@@ -708,7 +742,6 @@ int tune_tile(const StencilView<float, S>& v, cudaStream_t s, int* best_out, flo
       best_shape = shape;
     }
   }
-  gfree(scratch);
   if (!rc && strip_timeouts()) rc = set_error(BMG_ETIMEOUT, "one-pass sweep: bulk copies did not complete");
   if (rc) return rc;
   cache[key] = {best_shape, best};
@@ -738,7 +771,8 @@ int tune_pair(const StencilView<float, S>& v, cudaStream_t s, int* best_out, flo
   }
   size_t ps = plane_stride32(v.n);
   float* scratch = nullptr;   // x, x', f laid out like a level's arrays
-  int rc = galloc(&scratch, v.n, 3, s);
+  Arena tmp;
+  int rc = galloc(tmp, &scratch, v.n, 3, s);
   if (rc) return rc;
   const float* f = scratch + 2 * ps;
   float best = 1e30f;
@@ -756,7 +790,6 @@ int tune_pair(const StencilView<float, S>& v, cudaStream_t s, int* best_out, flo
       best_shape = shape;
     }
   }
-  gfree(scratch);
   if (!rc && strip_timeouts()) rc = set_error(BMG_ETIMEOUT, "two-sweep pass: bulk copies did not complete");
   if (rc) return rc;
   cache[key] = {best_shape, best};
@@ -770,13 +803,13 @@ int tune_pair(const StencilView<float, S>& v, cudaStream_t s, int* best_out, flo
 // iterate when the tile kernel wins, and then also weighs one two-sweep pass
 // against two one-pass sweeps.
 template <typename S>
-int tune_level32(Level& L, const StencilView<float, S>& v, cudaStream_t s) {
+int tune_level32(Arena& m, Level& L, const StencilView<float, S>& v, cudaStream_t s) {
   float ms_rows = 0, ms_tile = 0;
   int shape = 0, rc = tune_rows(v, s, &L.cl32, &ms_rows);
   if (!rc) rc = tune_tile(v, s, &shape, &ms_tile);
   if (rc) return rc;
   if (ms_tile < ms_rows) {
-    if (!L.x32b && (rc = galloc(&L.x32b, L.n, 1, s))) return rc;
+    if (!L.x32b && (rc = galloc(m, &L.x32b, L.n, 1, s))) return rc;
     L.tile32 = shape;
     int pshape = -1;
     float ms_pair = 0;
@@ -806,7 +839,8 @@ int tune_tile64(const StencilView<double, double>& v, cudaStream_t s, int* best_
   }
   const size_t ps = plane_size(v.n);
   double* scratch = nullptr;   // x, x', f
-  if (int e = dalloc_zero(&scratch, 3 * ps, s)) return e;
+  Arena tmp;
+  if (int e = dalloc_zero(tmp, &scratch, 3 * ps, s)) return e;
   const double* f = scratch + 2 * ps;
   int best_shape = 0, rc = BMG_OK;
   float best = 1e30f;
@@ -821,7 +855,6 @@ int tune_tile64(const StencilView<double, double>& v, cudaStream_t s, int* best_
       best_shape = shape;
     }
   }
-  cudaFree(scratch);
   if (rc) return rc;
   cache[key] = {best_shape, best};
   tune_file_put(fkey, TuneRecord{{best_shape}, best});
@@ -832,13 +865,13 @@ int tune_tile64(const StencilView<double, double>& v, cudaStream_t s, int* best_
 
 // Row kernel vs the one-pass kernel for an FP64 level (the second iterate is
 // allocated when the one-pass kernel wins).
-int tune_level64(Level& L, cudaStream_t s) {
+int tune_level64(Arena& m, Level& L, cudaStream_t s) {
   float ms_rows = 0, ms_tile = 0;
   int shape = 0, rc = tune_rows(view64(L), s, &L.cl64, &ms_rows);
   if (!rc) rc = tune_tile64(view64(L), s, &shape, &ms_tile);
   if (rc) return rc;
   if (ms_tile < ms_rows) {
-    if (!L.x64b && (rc = dalloc_zero(&L.x64b, plane_size(L.n), s))) return rc;
+    if (!L.x64b && (rc = dalloc_zero(m, &L.x64b, plane_size(L.n), s))) return rc;
     L.tile64 = shape;
   }
   return BMG_OK;
@@ -875,7 +908,7 @@ int choose_level_halves(bmg_hierarchy* h) {
     if (h->tail_l >= 0 && l >= h->tail_l) break;
     L.lrows = level_rows(f64, L.n);
     if (L.lrows <= 0) continue;
-    int rc = f64 ? dalloc_zero(&L.x64b, plane_size(L.n), h->ws) : galloc(&L.x32b, L.n, 1, h->ws);
+    int rc = f64 ? dalloc_zero(h->mem, &L.x64b, plane_size(L.n), h->ws) : galloc(h->mem, &L.x32b, L.n, 1, h->ws);
     if (rc) return rc;
   }
   return BMG_OK;
@@ -912,8 +945,8 @@ int build_tail(bmg_hierarchy* h, int lmin) {
       d.lv[k] = LevelDesc<float, float>{view32(L), L.ci32, L.x32, L.f32, C ? C->x32 : nullptr,
                                         C ? C->f32 : nullptr, nullptr, h->Lfac, h->work};
   }
-  CK(dev_malloc((void**)&h->d_tail, sizeof(d)));
-  CK(cudaMemcpy(h->d_tail, &d, sizeof(d), cudaMemcpyHostToDevice));
+  if (int rc = h->mem.take(&h->d_tail, sizeof(d), false, h->ws)) return rc;
+  CK(cudaMemcpyAsync(h->d_tail, &d, sizeof(d), cudaMemcpyHostToDevice, h->ws));   // (pageable: returns once copied)
   h->tail_l = lt;
   return BMG_OK;
 }
@@ -926,11 +959,11 @@ int force_tile(bmg_hierarchy* h) {
     Level& L = h->lv[l];
     if (L.kind != 9) continue;
     if (h->precision == BMG_FP64) {
-      if (int rc = dalloc_zero(&L.x64b, plane_size(L.n), h->ws)) return rc;
+      if (int rc = dalloc_zero(h->mem, &L.x64b, plane_size(L.n), h->ws)) return rc;
       L.tile64 = h->smoother - BMG_SMOOTHER_TILE;
       continue;
     }
-    int rc = galloc(&L.x32b, L.n, 1, h->ws);
+    int rc = galloc(h->mem, &L.x32b, L.n, 1, h->ws);
     if (rc) return rc;
     if (h->smoother >= BMG_SMOOTHER_PAIR) {
       L.tile32 = 3;
@@ -955,7 +988,7 @@ int build_lines(bmg_hierarchy* h) {
     for (int axis = 0; axis < 2; ++axis) {
       if (dir == (axis == 0 ? LINE_Y : LINE_X)) continue;
       auto add = [&](auto& jobs, const auto& v, auto& F, int arrays) {
-        if (int rc = dalloc(&F.c, arrays * ps)) return rc;
+        if (int rc = dalloc(h->mem, &F.c, arrays * ps, h->ws)) return rc;
         F.m = F.c + ps;
         if (arrays == 4) {
           F.y = F.m + ps;
@@ -990,15 +1023,15 @@ int autotune_solo(bmg_hierarchy* h) {
     if (L.kind != 9 || L.n < 127 || (l > 0 && L.lrows > 0)) continue;
     int rc = BMG_OK;
     if (h->precision == BMG_FP64)
-      rc = h->smoother == BMG_SMOOTHER_AUTO ? tune_level64(L, h->ws)
+      rc = h->smoother == BMG_SMOOTHER_AUTO ? tune_level64(h->mem, L, h->ws)
            : L.tile64 >= 0                ? BMG_OK
                                           : tune_rows(view64(L), h->ws, &L.cl64);
     else if (h->smoother != BMG_SMOOTHER_AUTO)
       rc = L.tile32 >= 0 ? BMG_OK : L.bf16 ? tune_rows(viewbf(L), h->ws, &L.cl32) : tune_rows(view32(L), h->ws, &L.cl32);
     else if (L.bf16)
-      rc = tune_level32(L, viewbf(L), h->ws);
+      rc = tune_level32(h->mem, L, viewbf(L), h->ws);
     else
-      rc = tune_level32(L, view32(L), h->ws);
+      rc = tune_level32(h->mem, L, view32(L), h->ws);
     if (rc) return rc;
   }
   return BMG_OK;
@@ -1019,7 +1052,8 @@ int tune_pair_restrict(Level& L, Level& C, const StencilView<float, S>& v, cudaS
   }
   size_t ps = plane_stride32(v.n);
   float* scratch = nullptr;   // x, x', f laid out like a level's arrays
-  int rc = galloc(&scratch, v.n, 3, s);
+  Arena tmp;
+  int rc = galloc(tmp, &scratch, v.n, 3, s);
   if (rc) return rc;
   const float* f = scratch + 2 * ps;
   // the two candidates timed alternately, twice each (the clocks may still be
@@ -1041,7 +1075,6 @@ int tune_pair_restrict(Level& L, Level& C, const StencilView<float, S>& v, cudaS
       }, &ms);
     ms_fused = std::min(ms_fused, ms);
   }
-  gfree(scratch);
   if (!rc && strip_timeouts()) rc = set_error(BMG_ETIMEOUT, "two-sweep pass: bulk copies did not complete");
   if (rc) return rc;
   L.pair_rr = fused_ok && ms_fused < ms_sep ? 1 : 0;
@@ -1196,36 +1229,6 @@ int ensure_ctl(bmg_hierarchy* h, int maxit) {
   return BMG_OK;
 }
 
-void free_level(Level& L, bool shared_ops = false) {
-  if (shared_ops) {   // borrowed operator arrays stay with their owner
-    L.st = nullptr;
-    L.ci = nullptr;
-    L.st32 = nullptr;
-    L.off16 = nullptr;
-    L.od32 = nullptr;
-    L.ci32 = nullptr;
-    L.pk32 = nullptr;
-  }
-  cudaFree(L.st);
-  cudaFree(L.ci);
-  cudaFree(L.x);
-  cudaFree(L.f);
-  for (int axis = 0; axis < 2; ++axis) {
-    cudaFree(L.lfac[axis].c);
-    cudaFree(L.lfac32[axis].c);
-  }
-  gfree(L.st32);
-  gfree(L.off16);
-  gfree(L.od32);
-  gfree(L.pk32);
-  cudaFree(L.ci32);
-  gfree(L.x32);
-  gfree(L.x32b);
-  gfree(L.f32);
-  cudaFree(L.x64b);
-  L = Level{};
-}
-
 bool is_level_size(int n) { return n >= 3 && ((n + 1) & n) == 0; }
 
 // The smallest n = 2^m - 1 >= max(nx, ny, 3): the level-0 size of an nx x ny problem.
@@ -1249,34 +1252,28 @@ int setup_impl(bmg_hierarchy* h, const bmg_stencil* A, int n, const bmg_opts* o)
     L.kind = l == 0 ? A->kind : 9;
     L.fused = h->arith == BMG_ARITH_FUSED;
     size_t ps = plane_size(L.n);
-    if ((rc = dalloc(&L.st, 6 * ps))) return rc;
+    if ((rc = dalloc(h->mem, &L.st, 6 * ps, s))) return rc;
     if (l + 1 < h->nlev)
-      if ((rc = dalloc(&L.ci, 8 * plane_size(sizes[l + 1])))) return rc;
+      if ((rc = dalloc(h->mem, &L.ci, 8 * plane_size(sizes[l + 1]), s))) return rc;
     if (l > 0) {
-      if ((rc = dalloc(&L.x, ps))) return rc;
-      if ((rc = dalloc(&L.f, ps))) return rc;
-      CK(cudaMemsetAsync(L.x, 0, ps * sizeof(double), s));
-      CK(cudaMemsetAsync(L.f, 0, ps * sizeof(double), s));
+      if ((rc = dalloc_zero(h->mem, &L.x, ps, s))) return rc;
+      if ((rc = dalloc_zero(h->mem, &L.f, ps, s))) return rc;
     }
   }
   h->m = h->coarsest * h->coarsest;
-  if ((rc = dalloc(&h->Lfac, (size_t)h->m * h->m))) return rc;
-  if ((rc = dalloc(&h->work, (size_t)h->m * h->m + h->m))) return rc;
-  if ((rc = dalloc(&h->partials, 2 * (size_t)norm_partials_max()))) return rc;
+  if ((rc = dalloc(h->mem, &h->Lfac, (size_t)h->m * h->m, s))) return rc;
+  if ((rc = dalloc(h->mem, &h->work, (size_t)h->m * h->m + h->m, s))) return rc;
+  if ((rc = dalloc(h->mem, &h->partials, 2 * (size_t)norm_partials_max(), s))) return rc;
   if (h->krylov == BMG_KRYLOV_FCG) {
     size_t ps = plane_size(n);
-    if ((rc = dalloc(&h->kr, 4 * ps))) return rc;
-    CK(cudaMemsetAsync(h->kr, 0, 4 * ps * sizeof(double), s));
+    if ((rc = dalloc_zero(h->mem, &h->kr, 4 * ps, s))) return rc;
   }
-  if ((rc = dalloc(&h->err, 1))) return rc;
-  CK(cudaMemsetAsync(h->err, 0, sizeof(int), s));
+  if ((rc = dalloc_zero(h->mem, &h->err, 1, s))) return rc;
 
   launch_prepare(n, h->nx, h->ny, A->kind, A->coef, h->lv[0].st, h->err, s);
   if (h->nx != n || h->ny != n) {   // embedded problem: the solve's own f and x on the n x n grid
-    if ((rc = dalloc(&h->fpad, plane_size(n)))) return rc;
-    if ((rc = dalloc(&h->xpad, plane_size(n)))) return rc;
-    CK(cudaMemsetAsync(h->fpad, 0, plane_size(n) * sizeof(double), s));
-    CK(cudaMemsetAsync(h->xpad, 0, plane_size(n) * sizeof(double), s));
+    if ((rc = dalloc_zero(h->mem, &h->fpad, plane_size(n), s))) return rc;
+    if ((rc = dalloc_zero(h->mem, &h->xpad, plane_size(n), s))) return rc;
   }
   for (int l = 0; l + 1 < h->nlev; ++l) {
     Level& L = h->lv[l];
@@ -1297,26 +1294,24 @@ int setup_impl(bmg_hierarchy* h, const bmg_stencil* A, int n, const bmg_opts* o)
     int nbf = h->precision == BMG_BF16_IR ? (o && o->bf16_levels > 0 ? o->bf16_levels : 2) : 0;
     for (int l = 0; l < h->nlev; ++l) {
       Level& L = h->lv[l];
-      size_t ps = plane_size(L.n);
       L.bf16 = l < nbf && l + 1 < h->nlev;
       if (L.bf16) {
-        if ((rc = galloc(&L.off16, L.n, 4, s))) return rc;
-        if ((rc = galloc(&L.od32, L.n, 2, s))) return rc;
-        launch_lower_bf16(L.n, L.st, L.off16, L.od32, s);
+        if ((rc = galloc(h->mem, &L.off16, L.n, 4, s))) return rc;
+        if ((rc = galloc(h->mem, &L.od32, L.n, 2, s))) return rc;
       } else {
-        if ((rc = galloc(&L.st32, L.n, 6, s))) return rc;
+        if ((rc = galloc(h->mem, &L.st32, L.n, 6, s))) return rc;
       }
-      if (l + 1 < h->nlev && (rc = dalloc(&L.ci32, 8 * plane_size(h->lv[l + 1].n)))) return rc;
-      launch_lower32(L.n, L.bf16 ? nullptr : L.st, L.bf16 ? nullptr : L.st32, L.ci, L.ci32, s);
-      if (l + 1 < h->nlev) {   // the packed copy the bulk-copy sweeps stream (guard band after it too)
-        if ((rc = galloc(&L.pk32, L.n, L.bf16 ? PK_WORDS_BF16 : PK_WORDS_F32, s))) return rc;
-        if (L.bf16)
-          launch_pack_bf16(L.n, L.off16, L.od32, L.pk32, s);
-        else
-          launch_pack32(L.n, L.st32, L.pk32, s);
+      if (l + 1 < h->nlev) {   // weights, and the packed copy the bulk-copy sweeps stream (guard band after it too)
+        if ((rc = dalloc(h->mem, &L.ci32, 8 * plane_size(h->lv[l + 1].n), s))) return rc;
+        if ((rc = galloc(h->mem, &L.pk32, L.n, L.bf16 ? PK_WORDS_BF16 : PK_WORDS_F32, s))) return rc;
+        launch_round32(8 * plane_size(h->lv[l + 1].n), L.ci, L.ci32, s);
       }
-      if ((rc = galloc(&L.x32, L.n, 1, s))) return rc;
-      if ((rc = galloc(&L.f32, L.n, 1, s))) return rc;
+      if (L.bf16)
+        launch_lower_bf16(L.n, L.st, L.off16, L.od32, L.pk32, s);
+      else
+        launch_lower32(L.n, L.st, L.st32, L.pk32, s);
+      if ((rc = galloc(h->mem, &L.x32, L.n, 1, s))) return rc;
+      if ((rc = galloc(h->mem, &L.f32, L.n, 1, s))) return rc;
     }
   }
   CK(cudaGetLastError());
@@ -1424,7 +1419,7 @@ int setup_periodic(bmg_hierarchy* h, const bmg_stencil* A, int nx, int ny, int p
   if (!rc) rc = cuda_check(cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming), "event");
   if (!rc) rc = cuda_check(host_malloc((void**)&h->ctl_host, sizeof(Ctl)), "pinned");
   if (!rc) rc = order_after_user(h);
-  if (!rc) rc = dalloc(&h->partials, 2 * (size_t)norm_partials_max());
+  if (!rc) rc = dalloc(h->mem, &h->partials, 2 * (size_t)norm_partials_max(), h->ws);
   if (!rc) rc = per_setup(&h->per, A->kind, A->coef, nx, ny, periodic, h->arith == BMG_ARITH_FUSED, h->nu1, h->nu2,
                           h->smoother == BMG_SMOOTHER_ROWS   ? PER_SWEEP_ROWS
                           : h->smoother == BMG_SMOOTHER_TILE ? PER_SWEEP_STRIP
@@ -1455,6 +1450,7 @@ int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* o, bmg_hiera
   h->nx = nx;
   h->ny = ny;
   h->n = embed_size(nx, ny);
+  h->mem.size_for(h->n);
   if (o) {
     h->precision = o->precision;
     h->coarsest = o->coarsest ? o->coarsest : 3;
@@ -1768,24 +1764,13 @@ long long bmg_launch_count(const bmg_hierarchy* h) { return h ? h->launches : 0;
 void bmg_free(bmg_hierarchy* h) {
   if (!h) return;
   if (h->ws) cudaStreamSynchronize(h->ws);
-  for (Level& L : h->lv) free_level(L, h->shared_ops);
-  if (!h->shared_ops) {
-    cudaFree(h->Lfac);
-    cudaFree(h->work);
-  }
-  cudaFree(h->partials);
-  cudaFree(h->kr);
-  cudaFree(h->fpad);
-  cudaFree(h->xpad);
   per_free(h->per);
-  cudaFree(h->d_tail);
-  cudaFree(h->err);
   cudaFree(h->ctl);
   if (h->ctl_host) cudaFreeHost(h->ctl_host);
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->ev) cudaEventDestroy(h->ev);
   if (h->ws) cudaStreamDestroy(h->ws);
-  delete h;
+  delete h;   // with its arena
 }
 
 int bmg_inner_cycle(bmg_hierarchy* h, const float* r32, float* e32) {
@@ -2400,9 +2385,9 @@ int group_alloc_x2(bmg_batch* B, const bmg_batch::Group& g, int b) {
     if (lv.n != g.n || lv.kind != g.kind || storage != g.storage || lv.x32b || lv.x64b) continue;
     int rc = BMG_OK;
     if (storage == 0) {
-      rc = dalloc_zero(&lv.x64b, plane_size(lv.n), B->ws);
+      rc = dalloc_zero(h->mem, &lv.x64b, plane_size(lv.n), B->ws);
     } else {
-      rc = galloc(&lv.x32b, lv.n, 1, B->ws);
+      rc = galloc(h->mem, &lv.x32b, lv.n, 1, B->ws);
     }
     if (rc) return rc;
   }
@@ -2428,7 +2413,8 @@ int tune_group(bmg_batch* B, bmg_batch::Group& g, int b) {
     const int base = rows_cluster<T>(g.n);
     const size_t ps = plane_stride32(g.n);   // scratch x, x2, f per problem, laid out like level arrays
     T* scratch = nullptr;
-    int rc = galloc(&scratch, g.n, 3 * g.count, B->ws);
+    Arena tmp;
+    int rc = galloc(tmp, &scratch, g.n, 3 * g.count, B->ws);
     if (rc) return rc;
     std::vector<LevelDesc<T, S>> d((const LevelDesc<T, S>*)g.host.data(),
                                    (const LevelDesc<T, S>*)g.host.data() + g.count);
@@ -2519,8 +2505,7 @@ int tune_group(bmg_batch* B, bmg_batch::Group& g, int b) {
       }
     }
     cudaFree(dd);
-    gfree(scratch);
-    if (!rc && strip_timeouts_b()) rc = set_error(BMG_ETIMEOUT, "batched one-pass sweep: bulk copies did not complete");
+      if (!rc && strip_timeouts_b()) rc = set_error(BMG_ETIMEOUT, "batched one-pass sweep: bulk copies did not complete");
     if (rc) return rc;
     it = g_tuned.emplace(key, best).first;
     tune_file_put(fkey, TuneRecord{{best.cl, best.tile, best.pair, best.multi}, best_ms});
@@ -2640,8 +2625,9 @@ int batch_init(bmg_batch* B, const bmg_opts* o, bmg_opts* so) {
 // right-hand sides and norm partials.
 int clone_state(const bmg_hierarchy* h0, cudaStream_t s, bmg_hierarchy** out) {
   bmg_hierarchy* h = new bmg_hierarchy();
-  h->shared_ops = true;
+  h->member = true;
   h->n = h0->n;
+  h->mem.size_for(h->n);
   h->nlev = h0->nlev;
   h->precision = h0->precision;
   h->nu1 = h0->nu1;
@@ -2671,15 +2657,13 @@ int clone_state(const bmg_hierarchy* h0, cudaStream_t s, bmg_hierarchy** out) {
     L.ci32 = S.ci32;
     const size_t ps = plane_size(L.n);
     if (l >= 1) {
-      if (!(rc = dalloc(&L.x, ps))) rc = dalloc(&L.f, ps);
-      if (!rc) rc = cuda_check(cudaMemsetAsync(L.x, 0, ps * sizeof(double), s), "clone");
-      if (!rc) rc = cuda_check(cudaMemsetAsync(L.f, 0, ps * sizeof(double), s), "clone");
+      if (!(rc = dalloc_zero(h->mem, &L.x, ps, s))) rc = dalloc_zero(h->mem, &L.f, ps, s);
     }
     if (!rc && h->precision != BMG_FP64) {
-      if (!(rc = galloc(&L.x32, L.n, 1, s))) rc = galloc(&L.f32, L.n, 1, s);
+      if (!(rc = galloc(h->mem, &L.x32, L.n, 1, s))) rc = galloc(h->mem, &L.f32, L.n, 1, s);
     }
   }
-  if (!rc) rc = dalloc(&h->partials, 2 * (size_t)norm_partials_max());
+  if (!rc) rc = dalloc(h->mem, &h->partials, 2 * (size_t)norm_partials_max(), s);
   if (rc) {
     bmg_free(h);
     return rc;
@@ -2778,7 +2762,7 @@ int bmg_batch_rhs(const bmg_hierarchy* h0, int k, const bmg_opts* o, bmg_batch**
   if (!out) return set_error(BMG_EINVAL, "bmg_batch_rhs: out is NULL");
   *out = nullptr;
   if (!h0 || k < 1) return set_error(BMG_EINVAL, "bmg_batch_rhs: bad argument");
-  if (h0->shared_ops) return set_error(BMG_EINVAL, "bmg_batch_rhs: h is itself a batch member");
+  if (h0->member) return set_error(BMG_EINVAL, "bmg_batch_rhs: h is itself a batch member");
   if (h0->fpad) return set_error(BMG_EINVAL, "bmg_batch_rhs: h holds an embedded (general-size) problem");
   if (h0->per) return set_error(BMG_EINVAL, "bmg_batch_rhs: h has periodic sides");
   if (o && o->krylov != BMG_KRYLOV_NONE) return set_error(BMG_EINVAL, "bmg_batch_rhs: stationary cycles only");

@@ -38,13 +38,12 @@ void launch_dendy(int n, const double* st, double* ci, int* err, cudaStream_t s)
 void launch_rap(int n, const double* st, const double* ci, double* stc, cudaStream_t s);
 void launch_dinv(int n, double* st, int* err, cudaStream_t s);
 void launch_factor(int n, const double* st, double* L, double* work, int* err, cudaStream_t s);
-// st32 / off16 / od32: planes plane_stride32(n) elements apart.
-void launch_lower32(int n, const double* st, float* st32, const double* ci, float* ci32, cudaStream_t s);
-void launch_lower_bf16(int n, const double* st, __nv_bfloat16* off16, float* od32, cudaStream_t s);
-// The packed stencil of an FP32 level (words d, w, s, sw, nw per point) or a
-// BF16 level (words d, w|s, sw|nw) over all (n+2)^2 points, from its planes.
-void launch_pack32(int n, const float* st32, float* pk, cudaStream_t s);
-void launch_pack_bf16(int n, const __nv_bfloat16* off16, const float* od32, float* pk, cudaStream_t s);
+// st32 / off16 / od32: planes plane_stride32(n) elements apart; pk (may be NULL
+// in FP32): the packed stencil, words d, w, s, sw, nw per point of an FP32
+// level or d, w|s, sw|nw of a BF16 level, over all (n+2)^2 points.
+void launch_round32(size_t count, const double* in, float* out, cudaStream_t s);
+void launch_lower32(int n, const double* st, float* st32, float* pk, cudaStream_t s);
+void launch_lower_bf16(int n, const double* st, __nv_bfloat16* off16, float* od32, float* pk, cudaStream_t s);
 constexpr int PK_WORDS_F32 = 5, PK_WORDS_BF16 = 3;
 
 // ---- cycle (k_cycle.cu) ----
