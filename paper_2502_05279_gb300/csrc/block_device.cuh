@@ -258,7 +258,8 @@ __device__ __forceinline__ void block_interp(BlockX<T>& x, T e_sw, T e_se, T e_n
 }
 
 // ---- coarsest solve by one warp ---------------------------------------------------------
-// L L^T x = f.  m = 9 unknowns (the default coarsest level): lane i holds
+// L L^T x = f.  m = 9 unknowns (the default coarsest level; 12 or 16 with
+// periodic sides): lane i holds
 // unknown i's partial sum, a step's quotient goes to the others by shuffle.
 // Forward, right-looking: row i subtracts L_ik y_k as soon as y_k is known, the
 // increasing-k order of the row-by-row loop.  Backward: row i's terms are
@@ -267,11 +268,12 @@ __device__ __forceinline__ void block_interp(BlockX<T>& x, T e_sw, T e_se, T e_n
 // chain of 45 differences, 18 products and 18 quotients (quot, four operations
 // each), about 63 cycles an operation.
 constexpr int COARSE_LANES = 9;
-struct Coarse9 {            // lane i: L(i, k), L(k, i), L(i, i) and its reciprocal
-  double row[COARSE_LANES], col[COARSE_LANES], dg, y, yl;
+template <int M>
+struct CoarseFactor {       // lane i: L(i, k), L(k, i), L(i, i) and its reciprocal
+  double row[M], col[M], dg, y, yl;
 };
-__device__ __forceinline__ void coarse9_load(Coarse9& c, const double* L) {
-  constexpr int M = COARSE_LANES;
+template <int M>
+__device__ __forceinline__ void coarse_load(CoarseFactor<M>& c, const double* L) {
   const int lane = threadIdx.x & 31, i = lane < M ? lane : 0;
 #pragma unroll
   for (int k = 0; k < M; ++k) {
@@ -280,9 +282,9 @@ __device__ __forceinline__ void coarse9_load(Coarse9& c, const double* L) {
   }
   c.dg = L[i * M + i];
 }
-// lane i < 9: f_i in, x_i out (other lanes compute along and are ignored)
-__device__ __forceinline__ double coarse9_solve(const Coarse9& c, double f) {
-  constexpr int M = COARSE_LANES;
+// lane i < M: f_i in, x_i out (other lanes compute along and are ignored)
+template <int M>
+__device__ __forceinline__ double coarse_substitute(const CoarseFactor<M>& c, double f) {
   const int lane = threadIdx.x & 31;
   double s = f;
 #pragma unroll
@@ -343,11 +345,11 @@ __device__ __forceinline__ void coarse_body(int n, const double* __restrict__ L,
   __shared__ double y[COARSE_M_MAX];
   const int lane = threadIdx.x & 31;
   if (n * n == COARSE_LANES) {
-    Coarse9 c;
-    coarse9_load(c, L);
+    CoarseFactor<COARSE_LANES> c;
+    coarse_load(c, L);
     c.y = quot_recip(c.dg, &c.yl);
     const int p = lane < COARSE_LANES ? (lane / 3 + 1) * 5 + lane % 3 + 1 : 6;
-    const T v = (T)coarse9_solve(c, (double)f[p]);
+    const T v = (T)coarse_substitute(c, (double)f[p]);
     if (lane < COARSE_LANES) x[p] = v;
   } else {
     warp_coarse<T>(n, L, f, x, y);

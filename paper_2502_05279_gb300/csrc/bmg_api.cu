@@ -361,10 +361,19 @@ int galloc(Arena& m, T** p, int n, int planes, cudaStream_t s) {
   return BMG_OK;
 }
 
-// Level l >= 1 starts its part of the cycle from a zero iterate without reading one.
-bool zero_aware(const bmg_hierarchy* h, int l) { return l == h->tail_l || (h->lv[l].lrows > 0 && !h->prof); }
+// Level l, started from a zero iterate, does not read one (and nothing has to
+// write the zeros): the tail, a level that runs by halves, an FP64 level whose
+// first sweep is a one-pass sweep, an FP32 level whose first pass streams rows.
+bool zero_aware(const bmg_hierarchy* h, int l) {
+  const Level& L = h->lv[l];
+  if ((l > 0 && l == h->tail_l) || (L.lrows > 0 && !h->prof)) return true;
+  if (h->nu1 < 1 || is_line(h->smoother)) return false;
+  if (h->precision == BMG_FP64) return L.tile64 >= 0;
+  return L.tile32 >= 0 && (L.tile32 < 4 || (L.pair32 >= 0 && h->nu1 >= 2));
+}
 
-void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* done) {
+// zero: the iterate is zero on entry (every level below the first).
+void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* done, bool zero) {
   Level& L = h->lv[l];
   cudaStream_t s = h->ws;
   if (l == h->tail_l) {
@@ -379,9 +388,9 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
   auto v = view64(L);
   Level& C = h->lv[l + 1];
   if (L.lrows > 0 && !h->prof) {   // one launch down, one up; the result is in x as below
-    launch_level_down(v, L.kind, (const double*)L.ci, f, l > 0 ? (const double*)nullptr : (const double*)x, L.x64b,
+    launch_level_down(v, L.kind, (const double*)L.ci, f, zero ? (const double*)nullptr : (const double*)x, L.x64b,
                       C.f, zero_aware(h, l + 1) ? (double*)nullptr : C.x, h->nu1, L.lrows, done, s);
-    vcycle64(h, l + 1, C.x, C.f, done);
+    vcycle64(h, l + 1, C.x, C.f, done, true);
     launch_level_up(v, L.kind, (const double*)L.ci, (const double*)C.x, f, (const double*)L.x64b, x, h->nu2, L.lrows,
                     done, s);
     return;
@@ -396,15 +405,19 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
     else if (L.tile64 >= 0)
       for (int k = 0; k < sweeps; ++k) {
         double* nxt = cur == x ? L.x64b : x;
-        step(h, l, BMG_K_RELAX, 0, [&] { launch_gs_tile64(v, f, cur, nxt, L.tile64, done, s); });
+        step(h, l, BMG_K_RELAX, 0, [&] { launch_gs_tile64(v, f, zero ? nullptr : cur, nxt, L.tile64, done, s); });
         cur = nxt;
+        zero = false;
       }
     else
       step(h, l, BMG_K_RELAX, 0, [&] { launch_gs(v, L.kind, f, x, sweeps, done, s, L.cl64); });
   };
   relax64(h->nu1);
-  step(h, l, BMG_K_RESID_RESTRICT, 0, [&] { launch_resid_restrict(v, L.kind, L.ci, cur, f, C.f, C.x, done, s); });
-  vcycle64(h, l + 1, C.x, C.f, done);
+  zero = false;
+  step(h, l, BMG_K_RESID_RESTRICT, 0, [&] {
+    launch_resid_restrict(v, L.kind, L.ci, cur, f, C.f, zero_aware(h, l + 1) ? (double*)nullptr : C.x, done, s);
+  });
+  vcycle64(h, l + 1, C.x, C.f, done, true);
   double* dst = L.tile64 >= 0 && (h->nu2 & 1) ? L.x64b : x;
   step(h, l, BMG_K_INTERP, 0, [&] { launch_interp_to<double>(L.n, L.ci, C.x, cur, dst, done, s, L.fused); });
   cur = dst;
@@ -414,7 +427,8 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
 // Sweeps of an FP32 level.  Row kernel: in place on x32.  One-pass tile kernel:
 // each sweep reads *cur and writes the other of x32 / x32b, and *cur follows.
 template <typename S>
-void relax32(bmg_hierarchy* h, const StencilView<float, S>& v, int l, int sweeps, float** cur, const int* done) {
+void relax32(bmg_hierarchy* h, const StencilView<float, S>& v, int l, int sweeps, float** cur, const int* done,
+             bool zero = false) {
   Level& L = h->lv[l];
   if (is_line(h->smoother)) {
     step(h, l, BMG_K_RELAX, 1, [&] {
@@ -433,16 +447,18 @@ void relax32(bmg_hierarchy* h, const StencilView<float, S>& v, int l, int sweeps
     step(h, l, BMG_K_RELAX_PAIR, 1, [&] {
       for (int k = 0; k < pairs; ++k) {
         float* dst = *cur == L.x32 ? L.x32b : L.x32;
-        launch_gs_pair(v, (const float*)L.f32, (const float*)*cur, dst, L.pair32, done, h->ws);
+        launch_gs_pair(v, (const float*)L.f32, zero ? (const float*)nullptr : *cur, dst, L.pair32, done, h->ws);
         *cur = dst;
+        zero = false;
       }
     });
   if (sweeps > 2 * pairs)
     step(h, l, BMG_K_RELAX, 1, [&] {
       for (int k = 2 * pairs; k < sweeps; ++k) {
         float* dst = *cur == L.x32 ? L.x32b : L.x32;
-        launch_gs_tile(v, (const float*)L.f32, (const float*)*cur, dst, L.tile32, done, h->ws);
+        launch_gs_tile(v, (const float*)L.f32, zero ? (const float*)nullptr : *cur, dst, L.tile32, done, h->ws);
         *cur = dst;
+        zero = false;
       }
     });
 }
@@ -455,13 +471,15 @@ void restrict32(bmg_hierarchy* h, const StencilView<float, S>& v, int l, const f
   Level& L = h->lv[l];
   Level& C = h->lv[l + 1];
   step(h, l, BMG_K_RESID_RESTRICT, 1,
-       [&] { launch_resid_restrict(v, L.kind, (const float*)L.ci32, x, (const float*)L.f32, C.f32, C.x32, done,
-                                   h->ws); });
+       [&] { launch_resid_restrict(v, L.kind, (const float*)L.ci32, x, (const float*)L.f32, C.f32,
+                                   zero_aware(h, l + 1) ? (float*)nullptr : C.x32, done, h->ws); });
 }
 
 // The FP32 cycle leaves every level's result in x32.  On a tile-swept level the
 // interpolation writes the array from which nu2 alternating sweeps end in x32.
-void vcycle32(bmg_hierarchy* h, int l, const int* done) {
+// zero: the iterate is zero on entry (every level below the first, and the
+// first cycle of a step).
+void vcycle32(bmg_hierarchy* h, int l, const int* done, bool zero) {
   Level& L = h->lv[l];
   cudaStream_t s = h->ws;
   if (l == h->tail_l) {
@@ -478,9 +496,9 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done) {
   if (L.lrows > 0 && !h->prof) {   // one launch down, one up
     auto both = [&](const auto& v) {
       launch_level_down(v, L.kind, (const float*)L.ci32, (const float*)L.f32,
-                        l > 0 ? (const float*)nullptr : (const float*)L.x32, L.x32b, C.f32,
+                        zero ? (const float*)nullptr : (const float*)L.x32, L.x32b, C.f32,
                         zero_aware(h, l + 1) ? (float*)nullptr : C.x32, h->nu1, L.lrows, done, s);
-      vcycle32(h, l + 1, done);
+      vcycle32(h, l + 1, done, true);
       launch_level_up(v, L.kind, (const float*)L.ci32, (const float*)C.x32, (const float*)L.f32,
                       (const float*)L.x32b, L.x32, h->nu2, L.lrows, done, s);
     };
@@ -491,13 +509,15 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done) {
     return;
   }
   float* cur = L.x32;
+  zero = zero && zero_aware(h, l);   // else the array holds the zeros
   auto pre = [&](const auto& v) {
     if (L.pair_rr && h->nu1 == 2) {   // temporal blocking: sweeps, residual and restriction in one pass
       float* dst = cur == L.x32 ? L.x32b : L.x32;
       step(h, l, BMG_K_PAIR_RESTRICT, 1, [&] {
-        if (!launch_gs_pair_restrict(v, (const float*)L.f32, (const float*)cur, dst, (const float*)L.ci32, C.f32,
-                                     C.x32, L.pair32 == 1 ? 1 : 0, done, s)) {
-          launch_gs_pair(v, (const float*)L.f32, (const float*)cur, dst, L.pair32, done, s);
+        const float* from = zero ? nullptr : cur;
+        if (!launch_gs_pair_restrict(v, (const float*)L.f32, from, dst, (const float*)L.ci32, C.f32,
+                                     zero_aware(h, l + 1) ? (float*)nullptr : C.x32, L.pair32 == 1 ? 1 : 0, done, s)) {
+          launch_gs_pair(v, (const float*)L.f32, from, dst, L.pair32, done, s);
           launch_resid_restrict(v, L.kind, (const float*)L.ci32, (const float*)dst, (const float*)L.f32, C.f32,
                                 C.x32, done, s);
         }
@@ -505,14 +525,14 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done) {
       cur = dst;
       return;
     }
-    relax32(h, v, l, h->nu1, &cur, done);
+    relax32(h, v, l, h->nu1, &cur, done, zero);
     restrict32(h, v, l, cur, done);
   };
   if (L.bf16)
     pre(viewbf(L));
   else
     pre(view32(L));
-  vcycle32(h, l + 1, done);
+  vcycle32(h, l + 1, done, true);
   float* dst = L.tile32 >= 0 && (sweep_launches(L, h->nu2) & 1) ? L.x32b : L.x32;
   step(h, l, BMG_K_INTERP, 1, [&] { launch_interp_to<float>(L.n, L.ci32, C.x32, cur, dst, done, s, L.fused); });
   cur = dst;
@@ -877,21 +897,6 @@ int tune_level64(Arena& m, Level& L, cudaStream_t s) {
   return BMG_OK;
 }
 
-// Block rows per tile of a level whose halves of the cycle run as one launch
-// each (0: its steps are launched separately).  The change of a whole cycle
-// when one level runs by halves, us, fused arithmetic (8 / 16 / 32 rows):
-//   FP64  63: -15 / -6    127: -12 / -4    255: -3 / -10   511: 0 / -17   1023: +121 / +55
-//   FP32  127: -11 / -11 / -11   255: -14 / -13 / -11   511: -12 / -15 / -17
-//         1023: +4 / -13 / -9    2047: +66 / -2 / +12
-// (one rounding per operation: within a few us of these).  Small FP64 levels
-// want few warps per SM quarter, each of whose FP64 instructions takes 60
-// cycles; larger ones a small halo.  In FP32 32 rows pay while their tiles,
-// one to an SM, fit the chip at once.
-int level_rows(bool f64, int n) {
-  if (f64) return n > 511 || n < 31 ? 0 : n <= 127 ? 8 : 16;
-  return n > 1023 || n < 31 ? 0 : n == 511 ? 32 : 16;
-}
-
 // Whether levels of the hierarchy may run by halves: graphs on, nothing forced,
 // sweep counts that the tiles' halos allow.
 bool by_halves(const bmg_hierarchy* h) {
@@ -1142,25 +1147,26 @@ void enqueue_iteration(bmg_hierarchy* h, const double* rhs, double* x) {
     double *r = h->kr, *z = h->kr + ps, *pv = h->kr + 2 * ps, *q = h->kr + 3 * ps;
     bool mixed = h->precision != BMG_FP64;
     if (mixed)
-      for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, done);
+      for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, done, c == 0);
     else
-      vcycle64(h, 0, z, r, done);
+      vcycle64(h, 0, z, r, done, true);
     step(h, 0, BMG_K_FCG, 0, [&] {
       launch_fcg_step(view64(L0), L0.kind, x, r, mixed ? nullptr : z, mixed ? L0.x32 : nullptr, pv, q,
-                      mixed ? L0.f32 : nullptr, mixed ? L0.x32 : nullptr, mixed ? nullptr : z, h->partials, h->ctl,
-                      h->ws, nullptr, nullptr);
+                      mixed ? L0.f32 : nullptr, mixed && !zero_aware(h, 0) ? L0.x32 : nullptr,
+                      mixed || zero_aware(h, 0) ? nullptr : z, h->partials, h->ctl, h->ws, nullptr, nullptr);
     });
     np = L0.n < norm_partials_max() ? L0.n : norm_partials_max();
   } else if (h->precision == BMG_FP64) {
-    vcycle64(h, 0, x, rhs, done);
+    vcycle64(h, 0, x, rhs, done, false);
     step(h, 0, BMG_K_NORM, 0, [&] {
       np = launch_residual(view64(L0), L0.kind, (const double*)x, rhs, (double*)nullptr, h->partials, done, h->ws);
     });
   } else {
-    for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, done);
+    for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, done, c == 0);
     step(h, 0, BMG_K_IR_UPDATE, 0, [&] { launch_ir_update(L0.n, x, L0.x32, h->ctl, h->ws); });
     step(h, 0, BMG_K_IR_RESIDUAL, 0, [&] {
-      np = launch_ir_residual(view64(L0), L0.kind, x, rhs, L0.f32, L0.x32, h->partials, h->ctl, h->ws);
+      np = launch_ir_residual(view64(L0), L0.kind, x, rhs, L0.f32, zero_aware(h, 0) ? nullptr : L0.x32, h->partials,
+                              h->ctl, h->ws);
     });
   }
   step(h, 0, BMG_K_FINALIZE, 0, [&] { launch_norm_finalize(h->partials, np, h->ctl, 1, nullptr, h->ws); });
@@ -1424,7 +1430,7 @@ int setup_periodic(bmg_hierarchy* h, const bmg_stencil* A, int nx, int ny, int p
                           h->smoother == BMG_SMOOTHER_ROWS   ? PER_SWEEP_ROWS
                           : h->smoother == BMG_SMOOTHER_TILE ? PER_SWEEP_STRIP
                                                              : PER_SWEEP_AUTO,
-                          h->krylov == BMG_KRYLOV_FCG, h->ws);
+                          h->krylov == BMG_KRYLOV_FCG, h->use_graph != 0, h->ws);
   if (!rc) rc = ensure_ctl(h, 64);
   if (rc) {
     bmg_free(h);
@@ -1783,7 +1789,7 @@ int bmg_inner_cycle(bmg_hierarchy* h, const float* r32, float* e32) {
   size_t bytes = plane_size(L0.n) * sizeof(float);
   CK(cudaMemcpyAsync(L0.f32, r32, bytes, cudaMemcpyDeviceToDevice, h->ws));
   CK(cudaMemsetAsync(L0.x32, 0, bytes, h->ws));
-  for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, nullptr);
+  for (int c = 0; c < h->inner; ++c) vcycle32(h, 0, nullptr, c == 0);
   CK(cudaMemcpyAsync(e32, L0.x32, bytes, cudaMemcpyDeviceToDevice, h->ws));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->ws));

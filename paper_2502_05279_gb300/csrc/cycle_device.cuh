@@ -343,6 +343,48 @@ __device__ __forceinline__ void strip_row(const StripRowT<T, S>& L, StripRowT<T,
   }
 }
 
+// The same two colours of the first sweep from a zero iterate: the terms of
+// points that are still zero are left out (a term a * 0 changes no sum but the
+// sign of a zero one), 16 of the 32 of a 2 x 2 block.  ODD rows: the odd-i
+// points have no term, the even-i points W and E; even rows: the odd-i points
+// all but W and E, the even-i points all eight.
+template <bool ODD, typename T, typename S, bool FU>
+__device__ __forceinline__ void strip_row_zero(const StripRowT<T, S>& L, StripRowT<T, S>& M, const StripRowT<T, S>& U,
+                                               bool oka, bool okb) {
+  {
+    T s = M.fa;
+    if constexpr (!ODD) {
+      const T xsw = shfl_up1(L.xb), xnw = shfl_up1(U.xb);
+      s = msub<FU>(s, cvt<T>(M.sa), L.xa);
+      s = msub<FU>(s, cvt<T>(U.sa), U.xa);
+      s = msub<FU>(s, cvt<T>(M.swa), xsw);
+      s = msub<FU>(s, cvt<T>(U.swb), U.xb);
+      s = msub<FU>(s, cvt<T>(M.nwa), xnw);
+      s = msub<FU>(s, cvt<T>(L.nwb), L.xb);
+    }
+    const T xn = rmul(s, M.da);
+    M.xa = oka ? xn : T(0);
+  }
+  {
+    const T xe = shfl_dn1(M.xa), we = shfl_dn1(cvt<T>(M.wa));
+    T s = M.fb;
+    s = msub<FU>(s, cvt<T>(M.wb), M.xa);
+    s = msub<FU>(s, we, xe);
+    if constexpr (!ODD) {
+      const T xne = shfl_dn1(U.xa), swne = shfl_dn1(cvt<T>(U.swa));
+      const T xse = shfl_dn1(L.xa), nwse = shfl_dn1(cvt<T>(L.nwa));
+      s = msub<FU>(s, cvt<T>(M.sb), L.xb);
+      s = msub<FU>(s, cvt<T>(U.sb), U.xb);
+      s = msub<FU>(s, cvt<T>(M.swb), L.xa);
+      s = msub<FU>(s, swne, xne);
+      s = msub<FU>(s, cvt<T>(M.nwb), U.xa);
+      s = msub<FU>(s, nwse, xse);
+    }
+    const T xn = rmul(s, M.db);
+    M.xb = okb ? xn : T(0);
+  }
+}
+
 template <typename T, typename S>
 __device__ __forceinline__ void strip_store(T* __restrict__ xout, int n, int ld, int ic, int j, bool own,
                                             const StripRowT<T, S>& R) {
@@ -473,19 +515,20 @@ struct StripSrc {           // the 3 arrays the walk reads
 
 // Request row j into `slot`, called by the whole warp: lane 0 arms the slot's
 // mbarrier for the row's bytes, then lanes 0, 1, 2 copy the row segments of
-// x, f and the packed stencil.  The caller's __syncwarp orders the warp's
+// x (not with ZERO: a zero iterate is not read), f and the packed stencil.  The
+// caller's __syncwarp orders the warp's
 // earlier reads of the slot before the fences.
-template <typename S>
+template <typename S, bool ZERO = false>
 __device__ __forceinline__ void ring_issue_warp(const StripSrc& A, int ld, int icol, int j, unsigned char* slot,
                                                 unsigned long long* bar) {
   using RG = StripRing<S>;
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    mbar_expect_tx(bar, RG::SLOT);
+    mbar_expect_tx(bar, RG::SLOT - (ZERO ? RG::BF : 0));
   }
   __syncwarp();
-  if (lane < 3) {
+  if (lane < 3 && !(ZERO && lane == 0)) {
     const long long e = (long long)j * ld + icol;   // first point of the row segment
     const long long e4 = e - (e & 3);
     // (debug builds: a segment outside the array's guarded extent is read from its start instead)
@@ -530,7 +573,7 @@ __device__ __forceinline__ void packed_read_wide(const float* q, bool bf16, floa
 // A row of the walk with every value in FP32 (BF16 coefficients widened).
 using StripRowW = StripRowT<float, float>;
 
-template <typename S>
+template <typename S, bool ZERO = false>
 __device__ __forceinline__ void ring_read(const unsigned char* slot, int ld, int icol, int ic, int j, StripRowW& R) {
   using RG = StripRing<S>;
   const long long e = (long long)j * ld + icol;
@@ -539,8 +582,8 @@ __device__ __forceinline__ void ring_read(const unsigned char* slot, int ld, int
   const float* ff = reinterpret_cast<const float*>(slot + RG::BF);
   const float* pq = reinterpret_cast<const float*>(slot + 2 * RG::BF) + RG::PK * o;
   constexpr bool BF = sizeof(S) == 2;
-  R.xa = xf[o];
-  R.xb = xf[o + 1];
+  R.xa = ZERO ? 0.0f : xf[o];
+  R.xb = ZERO ? 0.0f : xf[o + 1];
   R.fa = ff[o];
   R.fb = ff[o + 1];
   packed_read_wide(pq, BF, R.da, R.wa, R.sa, R.swa, R.nwa);
@@ -548,8 +591,19 @@ __device__ __forceinline__ void ring_read(const unsigned char* slot, int ld, int
 }
 
 
+// A row's two colours of a sweep, the first sweep of a zero iterate with ZERO.
+template <bool ODD, bool FU, bool ZERO>
+__device__ __forceinline__ void strip_sweep_row(const StripRowW& L, StripRowW& M, const StripRowW& U, bool oka,
+                                                bool okb) {
+  if constexpr (ZERO)
+    strip_row_zero<ODD, float, float, FU>(L, M, U, oka, okb);
+  else
+    strip_row<float, float, FU>(L, M, U, oka, okb);
+}
+
 // The strip height ty (even, >= 2) is a launch argument, as in the FP64 sweep.
-template <typename S, int RING, bool FU = false>
+// ZERO: from a zero iterate (xin is not read).
+template <typename S, int RING, bool FU = false, bool ZERO = false>
 __device__ __forceinline__ bool gs_strip_ring_body(const StencilView<float, S>& v, const float* __restrict__ f,
                                                    const float* __restrict__ xin, float* __restrict__ xout,
                                                    int sx, int sy, int ty, unsigned char* ring,
@@ -574,7 +628,7 @@ __device__ __forceinline__ bool gs_strip_ring_body(const StencilView<float, S>& 
   }
   __syncwarp();
   for (int q = 0; q < RING; ++q)
-    if (valid(q)) ring_issue_warp<S>(A, ld, icol, j0 - 1 + q, ring + q * RG::SLOT, &bars[q]);
+    if (valid(q)) ring_issue_warp<S, ZERO>(A, ld, icol, j0 - 1 + q, ring + q * RG::SLOT, &bars[q]);
   bool ok = true;
   int taken = 0;                                  // rows 0 .. taken-1 read; rows < taken + RING requested
   // read band row q into R (waiting for its slot), then hand the slot to row q + RING
@@ -582,18 +636,18 @@ __device__ __forceinline__ bool gs_strip_ring_body(const StencilView<float, S>& 
     const int slot = q % RING;
     if (valid(q) && ok) ok = mbar_wait(&bars[slot], (unsigned)((q / RING) & 1));
     if (!ok) return;
-    ring_read<S>(ring + slot * RG::SLOT, ld, icol, ic, j0 - 1 + q, R);
+    ring_read<S, ZERO>(ring + slot * RG::SLOT, ld, icol, ic, j0 - 1 + q, R);
     taken = q + 1;
     __syncwarp();
     if (valid(q) && valid(q + RING))
-      ring_issue_warp<S>(A, ld, icol, j0 - 1 + q + RING, ring + slot * RG::SLOT, &bars[slot]);
+      ring_issue_warp<S, ZERO>(A, ld, icol, j0 - 1 + q + RING, ring + slot * RG::SLOT, &bars[slot]);
   };
   StripRowW P0, P1, Q0, Q1;                     // two row pairs in alternating roles
   take(0, P1);
   take(1, Q0);
   take(2, Q1);
   if (ok && j0 <= n) {
-    strip_row<float, float, FU>(P1, Q0, Q1, c1, c2);                // row j0: c1, c2
+    strip_sweep_row<true, FU, ZERO>(P1, Q0, Q1, c1, c2);                // row j0: c1, c2
     strip_store(xout, n, ld, ic, j0, own, Q0);
   }
   // step m: old pair = rows a - 2, a - 1; new pair = rows a, a + 1 (band rows 2m + 1, 2m + 2)
@@ -603,11 +657,11 @@ __device__ __forceinline__ bool gs_strip_ring_body(const StencilView<float, S>& 
     take(2 * m + 2, E3);
     if (!ok) return;
     if (a <= n) {
-      strip_row<float, float, FU>(E1, E2, E3, c1, c2);              // row a: c1, c2
+      strip_sweep_row<true, FU, ZERO>(E1, E2, E3, c1, c2);              // row a: c1, c2
       if (a < j1) strip_store(xout, n, ld, ic, a, own, E2);
     }
     if (a - 1 <= n) {
-      strip_row<float, float, FU>(E0, E1, E2, c3, c4);              // row a - 1: c3, c4
+      strip_sweep_row<false, FU, ZERO>(E0, E1, E2, c3, c4);              // row a - 1: c3, c4
       strip_store(xout, n, ld, ic, a - 1, own, E1);
     }
   };
@@ -639,7 +693,7 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <typename S, int RING, bool FU = false>
+template <typename S, int RING, bool FU = false, bool ZERO = false>
 __device__ __forceinline__ bool gs_strip2_ring_body(const StencilView<float, S>& v, const float* __restrict__ f,
                                                     const float* __restrict__ xin, float* __restrict__ xout,
                                                     int sx, int sy, int ty, unsigned char* ring,
@@ -665,7 +719,7 @@ __device__ __forceinline__ bool gs_strip2_ring_body(const StencilView<float, S>&
   auto issue = [&](int q) {
     if (q >= NR) return;
     if (rowok(q))
-      ring_issue_warp<S>(A, ld, icol, j0 - 3 + q, ring + (q % RING) * RG::SLOT, &bars[q % RING]);
+      ring_issue_warp<S, ZERO>(A, ld, icol, j0 - 3 + q, ring + (q % RING) * RG::SLOT, &bars[q % RING]);
     else if (lane == 0)
       mbar_arrive(&bars[q % RING]);
   };
@@ -681,7 +735,7 @@ __device__ __forceinline__ bool gs_strip2_ring_body(const StencilView<float, S>&
     const int slot = q % RING;
     if (ok) ok = mbar_wait(&bars[slot], (unsigned)((q / RING) & 1));
     if (!ok) return;
-    ring_read<S>(ring + slot * RG::SLOT, ld, icol, ic, j0 - 3 + q, R);
+    ring_read<S, ZERO>(ring + slot * RG::SLOT, ld, icol, ic, j0 - 3 + q, R);
     taken = q + 1;
     __syncwarp();
     issue(q + RING);
@@ -697,8 +751,8 @@ __device__ __forceinline__ bool gs_strip2_ring_body(const StencilView<float, S>&
       take(2 * m + 2, R5);
       if (!ok) return;
     }
-    if (a >= 1 && a <= n) strip_row<float, float, FU>(R3, R4, R5, p1, q1);                 // sweep 1, row a
-    if (m >= 1 && a - 1 >= 1 && a - 1 <= n) strip_row<float, float, FU>(R2, R3, R4, r1, t1);   // sweep 1, row a - 1
+    if (a >= 1 && a <= n) strip_sweep_row<true, FU, ZERO>(R3, R4, R5, p1, q1);                 // sweep 1, row a
+    if (m >= 1 && a - 1 >= 1 && a - 1 <= n) strip_sweep_row<false, FU, ZERO>(R2, R3, R4, r1, t1);   // sweep 1, row a - 1
     if (m >= 2 && b <= n) {                                               // sweep 2, row a - 2
       strip_row<float, float, FU>(R1, R2, R3, p2, q2);
       if (b < j1) strip_store(xout, n, ld, ic, b, own, R2);
@@ -978,17 +1032,17 @@ __device__ __forceinline__ void strip_resid(const StripRowW& L, const StripRowR&
   }
 }
 
-template <typename S>
+template <typename S, bool ZERO>
 __device__ __forceinline__ void ring_issue_warp_r(const StripSrc& A, const float* O, int ld, int icol, int j,
                                                   unsigned char* slot, unsigned long long* bar) {
   using RG = StripRing<S>;
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    mbar_expect_tx(bar, StripRingR<S>::SLOT);
+    mbar_expect_tx(bar, StripRingR<S>::SLOT - (ZERO ? RG::BF : 0));
   }
   __syncwarp();
-  if (lane < 4) {
+  if (lane < 4 && !(ZERO && lane == 0)) {
     const long long e = (long long)j * ld + icol;
     const long long e4 = e - (e & 3);
     // (debug builds: a segment outside the array's guarded extent is read from its start instead)
@@ -1004,9 +1058,9 @@ __device__ __forceinline__ void ring_issue_warp_r(const StripSrc& A, const float
   }
 }
 
-template <typename S>
+template <typename S, bool ZERO>
 __device__ __forceinline__ void ring_read_r(const unsigned char* slot, int ld, int icol, int ic, int j, StripRowR& R) {
-  ring_read<S>(slot, ld, icol, ic, j, R);
+  ring_read<S, ZERO>(slot, ld, icol, ic, j, R);
   const long long e = (long long)j * ld + icol;
   const int o = (int)(e & 3) + (ic - icol);
   const float* of = reinterpret_cast<const float*>(slot + StripRing<S>::SLOT);
@@ -1017,7 +1071,7 @@ __device__ __forceinline__ void ring_read_r(const unsigned char* slot, int ld, i
 // ci: the level's FP32 interpolation weights (8 planes of the coarse level);
 // fc, xc: the coarse right-hand side (written on owned coarse points) and
 // iterate (zeroed there).
-template <typename S, int RING, bool FU = false>
+template <typename S, int RING, bool FU = false, bool ZERO = false>
 __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>& v, const float* __restrict__ f,
                                                      const float* __restrict__ xin, float* __restrict__ xout,
                                                      const float* __restrict__ ci, float* __restrict__ fc,
@@ -1044,7 +1098,7 @@ __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>
   auto issue = [&](int q) {
     if (q >= NR) return;
     if (rowok(q))
-      ring_issue_warp_r<S>(A, v.O, ld, icol, j0 - 5 + q, ring + (q % RING) * SLOT, &bars[q % RING]);
+      ring_issue_warp_r<S, ZERO>(A, v.O, ld, icol, j0 - 5 + q, ring + (q % RING) * SLOT, &bars[q % RING]);
     else if (lane == 0)
       mbar_arrive(&bars[q % RING]);
   };
@@ -1060,7 +1114,7 @@ __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>
     const int slot = q % RING;
     if (ok) ok = mbar_wait(&bars[slot], (unsigned)((q / RING) & 1));
     if (!ok) return;
-    ring_read_r<S>(ring + slot * SLOT, ld, icol, ic, j0 - 5 + q, R);
+    ring_read_r<S, ZERO>(ring + slot * SLOT, ld, icol, ic, j0 - 5 + q, R);
     taken = q + 1;
     __syncwarp();
     issue(q + RING);
@@ -1076,8 +1130,8 @@ __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>
       take(2 * m + 2, R5);
       if (!ok) return;
     }
-    if (a >= 1 && a <= n) strip_row<float, float, FU>(R3, R4, R5, p1, q1);                   // sweep 1, row a
-    if (m >= 1 && a - 1 >= 1 && a - 1 <= n) strip_row<float, float, FU>(R2, R3, R4, r1, t1);   // sweep 1, row a - 1
+    if (a >= 1 && a <= n) strip_sweep_row<true, FU, ZERO>(R3, R4, R5, p1, q1);                   // sweep 1, row a
+    if (m >= 1 && a - 1 >= 1 && a - 1 <= n) strip_sweep_row<false, FU, ZERO>(R2, R3, R4, r1, t1);   // sweep 1, row a - 1
     if (m >= 2 && b >= 1 && b <= n) {                                                        // sweep 2, row b
       strip_row<float, float, FU>(R1, R2, R3, p2, q2);
       if (b >= j0 && b < j1) strip_store(xout, n, ld, ic, b, own, R2);
@@ -1113,7 +1167,7 @@ __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>
           const size_t pc = (size_t)jc * ldc + icc;
           if (BMG_IN(DBG_RESTRICT_STORE, pc, (size_t)ldc * ldc)) {
             fc[pc] = t;
-            xc[pc] = 0.f;
+            if (xc) xc[pc] = 0.f;
           }
         }
       }
@@ -1169,6 +1223,7 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool in) {
 }
 
 // this lane's columns ic, ic + 1 of row j into its part of `slot`, as one commit group
+template <bool ZERO>
 __device__ __forceinline__ void row64_issue(const StripSrc64& A, int n, int ld, int ic, int j, unsigned char* slot,
                                             int lane) {
   const bool rowin = j >= 0 && j <= n + 1;
@@ -1180,16 +1235,18 @@ __device__ __forceinline__ void row64_issue(const StripSrc64& A, int n, int ld, 
   double* d = reinterpret_cast<double*>(slot) + 2 * lane;
   const double* src[7] = {A.x, A.f, A.d, A.w, A.s, A.sw, A.nw};
 #pragma unroll
-  for (int k = 0; k < 7; ++k) {
+  for (int k = ZERO ? 1 : 0; k < 7; ++k) {   // a zero iterate is not read
     cp_async8(d + 64 * k, src[k] + (oka ? pa : 0), oka);
     cp_async8(d + 64 * k + 1, src[k] + (okb ? pb : 0), okb);
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
+template <bool ZERO>
 __device__ __forceinline__ void row64_read(const unsigned char* slot, int lane, StripRowT<double, double>& R) {
   const double2* d = reinterpret_cast<const double2*>(slot) + lane;
-  double2 v = d[0];
+  double2 v = make_double2(0.0, 0.0);
+  if constexpr (!ZERO) v = d[0];
   R.xa = v.x, R.xb = v.y;
   v = d[32];
   R.fa = v.x, R.fb = v.y;
@@ -1205,7 +1262,8 @@ __device__ __forceinline__ void row64_read(const unsigned char* slot, int lane, 
   R.nwa = v.x, R.nwb = v.y;
 }
 
-template <int RING, bool FU = false>
+// ZERO: the sweep starts from a zero iterate (xin is not read).
+template <int RING, bool FU = false, bool ZERO = false>
 __device__ __forceinline__ void gs_strip64_body(const StencilView<double, double>& v, const double* __restrict__ f,
                                                 const double* __restrict__ xin, double* __restrict__ xout, int sx,
                                                 int sy, int ty, unsigned char* ring) {
@@ -1224,7 +1282,7 @@ __device__ __forceinline__ void gs_strip64_body(const StencilView<double, double
   // every lane: request band row q (an empty group past the band keeps one group per row)
   auto issue = [&](int q) {
     if (q < NR)
-      row64_issue(A, n, ld, ic, j0 - 1 + q, ring + (q % RING) * STRIP64_SLOT, lane);
+      row64_issue<ZERO>(A, n, ld, ic, j0 - 1 + q, ring + (q % RING) * STRIP64_SLOT, lane);
     else
       asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
@@ -1233,15 +1291,27 @@ __device__ __forceinline__ void gs_strip64_body(const StencilView<double, double
   // band row q into R: its group is the oldest of the RING outstanding ones
   auto take = [&](int q, Row& R) {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 1) : "memory");
-    row64_read(ring + (q % RING) * STRIP64_SLOT, lane, R);
+    row64_read<ZERO>(ring + (q % RING) * STRIP64_SLOT, lane, R);
     issue(q + RING);
+  };
+  auto odd = [&](const Row& L, Row& M, const Row& U) {
+    if constexpr (ZERO)
+      strip_row_zero<true, double, double, FU>(L, M, U, c1, c2);
+    else
+      strip_row<double, double, FU>(L, M, U, c1, c2);
+  };
+  auto even = [&](const Row& L, Row& M, const Row& U) {
+    if constexpr (ZERO)
+      strip_row_zero<false, double, double, FU>(L, M, U, c3, c4);
+    else
+      strip_row<double, double, FU>(L, M, U, c3, c4);
   };
   Row P0, P1, Q0, Q1;                             // two row pairs in alternating roles
   take(0, P1);
   take(1, Q0);
   take(2, Q1);
   if (j0 <= n) {
-    strip_row<double, double, FU>(P1, Q0, Q1, c1, c2);     // row j0: c1, c2
+    odd(P1, Q0, Q1);     // row j0: c1, c2
     strip_store(xout, n, ld, ic, j0, own, Q0);
   }
   // step m: old pair = rows a - 2, a - 1; new pair = rows a, a + 1 (band rows 2m + 1, 2m + 2)
@@ -1250,11 +1320,11 @@ __device__ __forceinline__ void gs_strip64_body(const StencilView<double, double
     take(2 * m + 1, E2);
     take(2 * m + 2, E3);
     if (a <= n) {
-      strip_row<double, double, FU>(E1, E2, E3, c1, c2);   // row a: c1, c2
+      odd(E1, E2, E3);   // row a: c1, c2
       if (a < j1) strip_store(xout, n, ld, ic, a, own, E2);
     }
     if (a - 1 <= n) {
-      strip_row<double, double, FU>(E0, E1, E2, c3, c4);   // row a - 1: c3, c4
+      even(E0, E1, E2);   // row a - 1: c3, c4
       strip_store(xout, n, ld, ic, a - 1, own, E1);
     }
   };
@@ -1545,7 +1615,7 @@ __device__ __forceinline__ void ir_residual_body(const StencilView<double, doubl
                        : row_residual<double, double, false, true, FU>(v, x, p, f[p]);
       if (BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * ld)) {
         r32[p] = narrow_scaled(rr, inv, inv32);
-        e32[p] = 0.0f;
+        if (e32) e32[p] = 0.0f;
       }
       acc = madd<FU>(acc, rr, rr);
     }

@@ -5,6 +5,7 @@
 // flexible-CG outer loop.  The arithmetic lives in cycle_device.cuh, shared with
 // the batched kernels.
 #include <cstdint>
+#include <type_traits>
 
 #include "block_device.cuh"
 
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip(StencilView<float
 // Bulk-copy form: warp w of the CTA owns ring slots [w RING, (w + 1) RING) and
 // mbarriers [w RING, (w + 1) RING) of the dynamic shared memory.
 __device__ int g_strip_timeout = 0;
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip_ring(StencilView<float, S> v,
                                                                     const float* __restrict__ f,
                                                                     const float* __restrict__ xin,
@@ -66,12 +67,12 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip_ring(StencilView<
   unsigned char* ring = strip_smem + (size_t)w * RING * StripRing<S>::SLOT;
   unsigned long long* bars =
       reinterpret_cast<unsigned long long*>(strip_smem + (size_t)STRIP_WARPS * RING * StripRing<S>::SLOT) + w * RING;
-  if (!gs_strip_ring_body<S, RING, FU>(v, f, xin, xout, g % nbx, g / nbx, ty, ring, bars) && (threadIdx.x & 31) == 0)
+  if (!gs_strip_ring_body<S, RING, FU, ZERO>(v, f, xin, xout, g % nbx, g / nbx, ty, ring, bars) && (threadIdx.x & 31) == 0)
     atomicExch(&g_strip_timeout, 1);
 }
 
 // Two sweeps in one pass: warps take 48-column strips, otherwise as above.
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip2_ring(StencilView<float, S> v,
                                                                      const float* __restrict__ f,
                                                                      const float* __restrict__ xin,
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip2_ring(StencilView
   unsigned char* ring = strip_smem + (size_t)w * RING * StripRing<S>::SLOT;
   unsigned long long* bars =
       reinterpret_cast<unsigned long long*>(strip_smem + (size_t)STRIP_WARPS * RING * StripRing<S>::SLOT) + w * RING;
-  if (!gs_strip2_ring_body<S, RING, FU>(v, f, xin, xout, g % nbx, g / nbx, ty, ring, bars) &&
+  if (!gs_strip2_ring_body<S, RING, FU, ZERO>(v, f, xin, xout, g % nbx, g / nbx, ty, ring, bars) &&
       (threadIdx.x & 31) == 0)
     atomicExch(&g_strip_timeout, 1);
 }
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip2_ring(StencilView
 // Two sweeps, residual and restriction in one pass: warps take 44-column
 // strips; the coarse right-hand side and iterate of the next level are written
 // at the strip's coarse points.
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip2r_ring(StencilView<float, S> v,
                                                                       const float* __restrict__ f,
                                                                       const float* __restrict__ xin,
@@ -111,14 +112,14 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip2r_ring(StencilVie
   unsigned char* ring = strip_smem + (size_t)w * RING * StripRingR<S>::SLOT;
   unsigned long long* bars =
       reinterpret_cast<unsigned long long*>(strip_smem + (size_t)STRIP_WARPS * RING * StripRingR<S>::SLOT) + w * RING;
-  if (!gs_strip2r_ring_body<S, RING, FU>(v, f, xin, xout, ci, fc, xc, g % nbx, g / nbx, ty, ring, bars) &&
+  if (!gs_strip2r_ring_body<S, RING, FU, ZERO>(v, f, xin, xout, ci, fc, xc, g % nbx, g / nbx, ty, ring, bars) &&
       (threadIdx.x & 31) == 0)
     atomicExch(&g_strip_timeout, 1);
 }
 
 // FP64 one-pass sweep with strips of 56 x ty points: warp w of the CTA owns
 // ring slots [w RING, (w + 1) RING).
-template <int RING, bool FU>
+template <int RING, bool FU, bool ZERO>
 __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip64(StencilView<double, double> v,
                                                                  const double* __restrict__ f,
                                                                  const double* __restrict__ xin,
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS) k_gs_strip64(StencilView<dou
   const int nbx = (v.n + 55) / 56, nby = (v.n + ty - 1) / ty;
   const int w = threadIdx.x >> 5, g = blockIdx.x * STRIP_WARPS + w;
   if (g >= nbx * nby) return;                     // whole warps only
-  gs_strip64_body<RING, FU>(v, f, xin, xout, g % nbx, g / nbx, ty, strip_smem + (size_t)w * RING * STRIP64_SLOT);
+  gs_strip64_body<RING, FU, ZERO>(v, f, xin, xout, g % nbx, g / nbx, ty, strip_smem + (size_t)w * RING * STRIP64_SLOT);
 }
 
 // Zebra x-lines: one thread per row of the parity (first row 1 or 2).
@@ -358,11 +359,11 @@ static int resident_strip_warps(K kernel, size_t bytes) {
 
 // ty = 0: the smallest even strip height whose strips fit into one wave of
 // the kernel's resident warps.
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 static void strip_ring_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                               const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRing<S>::SLOT + 8);
-  static const int resident_warps = resident_strip_warps(k_gs_strip_ring<S, RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps(k_gs_strip_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 55) / 56;
   if (ty <= 0) {
     const int nby_max = resident_warps / nbx > 1 ? resident_warps / nbx : 1;
@@ -370,23 +371,23 @@ static void strip_ring_launch(const StencilView<float, S>& v, const float* f, co
     ty = 2 * (half > 1 ? half : 1);
   }
   const int warps = nbx * ((v.n + ty - 1) / ty);
-  pdl_launch(k_gs_strip_ring<S, RING, FU>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
+  pdl_launch(k_gs_strip_ring<S, RING, FU, ZERO>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
              v, f, xin, xout, done, ty);
   count_launch();
 }
 
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
-template <typename S, bool FU>
+template <typename S, bool FU, bool ZERO>
 static void gs_tile(const StencilView<float, S>& v, const float* f, const float* xin, float* xout, int shape,
                     const int* done, cudaStream_t s) {
   switch (shape) {
-    case 1: strip_ring_launch<S, 6, FU>(v, f, xin, xout, done, s, 0); break;   // one wave, deeper rings
-    case 2: strip_ring_launch<S, 8, FU>(v, f, xin, xout, done, s, 0); break;
-    case 3: strip_ring_launch<S, 4, FU>(v, f, xin, xout, done, s, 32); break;
+    case 1: strip_ring_launch<S, 6, FU, ZERO>(v, f, xin, xout, done, s, 0); break;   // one wave, deeper rings
+    case 2: strip_ring_launch<S, 8, FU, ZERO>(v, f, xin, xout, done, s, 0); break;
+    case 3: strip_ring_launch<S, 4, FU, ZERO>(v, f, xin, xout, done, s, 32); break;
     case 4: strip_launch<S, 32, FU>(v, f, xin, xout, done, s); break;
     case 5: strip_launch<S, 16, FU>(v, f, xin, xout, done, s); break;
-    default: strip_ring_launch<S, 4, FU>(v, f, xin, xout, done, s, 0); break;   // one wave
+    default: strip_ring_launch<S, 4, FU, ZERO>(v, f, xin, xout, done, s, 0); break;   // one wave
   }
 }
 
@@ -396,18 +397,19 @@ void launch_gs_tile(const StencilView<float, S>& v, const float* f, const float*
   const bool ring_ok = aligned16(f) && aligned16(xin) && v.pk && aligned16(v.pk);
   if (shape < 4 && !ring_ok) shape = 4;           // bulk copies need 16-byte aligned arrays and the packed stencil
   if (v.fused)
-    gs_tile<S, true>(v, f, xin, xout, shape, done, s);
+    xin ? gs_tile<S, true, false>(v, f, xin, xout, shape, done, s) : gs_tile<S, true, true>(v, f, xin, xout, shape, done, s);
   else
-    gs_tile<S, false>(v, f, xin, xout, shape, done, s);
+    xin ? gs_tile<S, false, false>(v, f, xin, xout, shape, done, s)
+        : gs_tile<S, false, true>(v, f, xin, xout, shape, done, s);
 }
 
 // ty = 0: the smallest even height whose strips fit into one wave of the
 // kernel's resident warps (occupancy x SMs x warps per CTA).
-template <int RING, bool FU>
+template <int RING, bool FU, bool ZERO>
 static void strip64_launch(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                            const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * STRIP64_SLOT;
-  static const int resident_warps = resident_strip_warps(k_gs_strip64<RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps(k_gs_strip64<RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 55) / 56;
   if (ty <= 0) {
     const int nby_max = resident_warps / nbx > 1 ? resident_warps / nbx : 1;
@@ -415,28 +417,29 @@ static void strip64_launch(const StencilView<double, double>& v, const double* f
     ty = 2 * (half > 1 ? half : 1);
   }
   const int warps = nbx * ((v.n + ty - 1) / ty);
-  pdl_launch(k_gs_strip64<RING, FU>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s, v, f,
+  pdl_launch(k_gs_strip64<RING, FU, ZERO>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s, v, f,
              xin, xout, done, ty);
   count_launch();
 }
 
-template <bool FU>
+template <bool FU, bool ZERO>
 static void gs_tile64(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                       int shape, const int* done, cudaStream_t s) {
   switch (shape) {
-    case 1: strip64_launch<4, FU>(v, f, xin, xout, done, s, 16); break;
-    case 2: strip64_launch<6, FU>(v, f, xin, xout, done, s, 0); break;
-    case 3: strip64_launch<4, FU>(v, f, xin, xout, done, s, 8); break;
-    default: strip64_launch<4, FU>(v, f, xin, xout, done, s, 0); break;
+    case 1: strip64_launch<4, FU, ZERO>(v, f, xin, xout, done, s, 16); break;
+    case 2: strip64_launch<6, FU, ZERO>(v, f, xin, xout, done, s, 0); break;
+    case 3: strip64_launch<4, FU, ZERO>(v, f, xin, xout, done, s, 8); break;
+    default: strip64_launch<4, FU, ZERO>(v, f, xin, xout, done, s, 0); break;
   }
 }
 
 void launch_gs_tile64(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                       int shape, const int* done, cudaStream_t s) {
   if (v.fused)
-    gs_tile64<true>(v, f, xin, xout, shape, done, s);
+    xin ? gs_tile64<true, false>(v, f, xin, xout, shape, done, s) : gs_tile64<true, true>(v, f, xin, xout, shape, done, s);
   else
-    gs_tile64<false>(v, f, xin, xout, shape, done, s);
+    xin ? gs_tile64<false, false>(v, f, xin, xout, shape, done, s)
+        : gs_tile64<false, true>(v, f, xin, xout, shape, done, s);
 }
 
 // One warp waits, through the same bounded wait as the bulk-copy sweep, on an
@@ -454,11 +457,11 @@ void launch_wait_selftest(cudaStream_t s) {
 }
 
 // ty = 0: the one-wave strip height, as strip_ring_launch.
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 static void strip2_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                           const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRing<S>::SLOT + 8);
-  static const int resident_warps = resident_strip_warps(k_gs_strip2_ring<S, RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps(k_gs_strip2_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 47) / 48;
   if (ty <= 0) {
     const int nby_max = resident_warps / nbx > 1 ? resident_warps / nbx : 1;
@@ -466,34 +469,34 @@ static void strip2_launch(const StencilView<float, S>& v, const float* f, const 
     ty = 2 * (half > 1 ? half : 1);
   }
   const int warps = nbx * ((v.n + ty - 1) / ty);
-  pdl_launch(k_gs_strip2_ring<S, RING, FU>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
+  pdl_launch(k_gs_strip2_ring<S, RING, FU, ZERO>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
              v, f, xin, xout, done, ty);
   count_launch();
 }
 
-template <typename S, bool FU>
+template <typename S, bool FU, bool ZERO>
 static void gs_pair(const StencilView<float, S>& v, const float* f, const float* xin, float* xout, int shape,
                     const int* done, cudaStream_t s) {
   switch (shape) {
-    case 1: strip2_launch<S, 6, FU>(v, f, xin, xout, done, s, 0); break;   // one wave, deeper rings
-    case 2: strip2_launch<S, 8, FU>(v, f, xin, xout, done, s, 0); break;
-    case 3: strip2_launch<S, 4, FU>(v, f, xin, xout, done, s, 26); break;
-    default: strip2_launch<S, 4, FU>(v, f, xin, xout, done, s, 0); break;   // one wave
+    case 1: strip2_launch<S, 6, FU, ZERO>(v, f, xin, xout, done, s, 0); break;   // one wave, deeper rings
+    case 2: strip2_launch<S, 8, FU, ZERO>(v, f, xin, xout, done, s, 0); break;
+    case 3: strip2_launch<S, 4, FU, ZERO>(v, f, xin, xout, done, s, 26); break;
+    default: strip2_launch<S, 4, FU, ZERO>(v, f, xin, xout, done, s, 0); break;   // one wave
   }
 }
 
 // ty = 0: the one-wave strip height, as strip_ring_launch.
-template <typename S, int RING, bool FU>
+template <typename S, int RING, bool FU, bool ZERO>
 static void strip2r_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                            const float* ci, float* fc, float* xc, const int* done, cudaStream_t s) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRingR<S>::SLOT + 8);
-  static const int resident_warps = resident_strip_warps(k_gs_strip2r_ring<S, RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps(k_gs_strip2r_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 43) / 44;
   const int nby_max = resident_warps / nbx > 1 ? resident_warps / nbx : 1;
   const int half = (v.n + 2 * nby_max - 1) / (2 * nby_max);
   const int ty = 2 * (half > 1 ? half : 1);
   const int warps = nbx * ((v.n + ty - 1) / ty);
-  pdl_launch(k_gs_strip2r_ring<S, RING, FU>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
+  pdl_launch(k_gs_strip2r_ring<S, RING, FU, ZERO>, (warps + STRIP_WARPS - 1) / STRIP_WARPS, 32 * STRIP_WARPS, bytes, s,
              v, f, xin, xout, ci, fc, xc, done, ty);
   count_launch();
 }
@@ -501,20 +504,18 @@ static void strip2r_launch(const StencilView<float, S>& v, const float* f, const
 template <typename S>
 bool launch_gs_pair_restrict(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                              const float* ci, float* fc, float* xc, int shape, const int* done, cudaStream_t s) {
-  if (!(aligned16(f) && aligned16(xin) && v.pk && aligned16(v.pk) && aligned16(v.O) && ci && fc && xc))
+  if (!(aligned16(f) && aligned16(xin) && v.pk && aligned16(v.pk) && aligned16(v.O) && ci && fc))
     return false;
-  const bool deep = shape == 1;
-  if (v.fused) {
-    if (deep)
-      strip2r_launch<S, 6, true>(v, f, xin, xout, ci, fc, xc, done, s);
+  auto go = [&](auto fused, auto zero) {
+    if (shape == 1)
+      strip2r_launch<S, 6, decltype(fused)::value, decltype(zero)::value>(v, f, xin, xout, ci, fc, xc, done, s);
     else
-      strip2r_launch<S, 4, true>(v, f, xin, xout, ci, fc, xc, done, s);
-  } else {
-    if (deep)
-      strip2r_launch<S, 6, false>(v, f, xin, xout, ci, fc, xc, done, s);
-    else
-      strip2r_launch<S, 4, false>(v, f, xin, xout, ci, fc, xc, done, s);
-  }
+      strip2r_launch<S, 4, decltype(fused)::value, decltype(zero)::value>(v, f, xin, xout, ci, fc, xc, done, s);
+  };
+  if (v.fused)
+    xin ? go(std::true_type{}, std::false_type{}) : go(std::true_type{}, std::true_type{});
+  else
+    xin ? go(std::false_type{}, std::false_type{}) : go(std::false_type{}, std::true_type{});
   return true;
 }
 template bool launch_gs_pair_restrict<float>(const StencilView<float, float>&, const float*, const float*, float*,
@@ -528,9 +529,10 @@ bool launch_gs_pair(const StencilView<float, S>& v, const float* f, const float*
                     const int* done, cudaStream_t s) {
   if (!(aligned16(f) && aligned16(xin) && v.pk && aligned16(v.pk))) return false;
   if (v.fused)
-    gs_pair<S, true>(v, f, xin, xout, shape, done, s);
+    xin ? gs_pair<S, true, false>(v, f, xin, xout, shape, done, s) : gs_pair<S, true, true>(v, f, xin, xout, shape, done, s);
   else
-    gs_pair<S, false>(v, f, xin, xout, shape, done, s);
+    xin ? gs_pair<S, false, false>(v, f, xin, xout, shape, done, s)
+        : gs_pair<S, false, true>(v, f, xin, xout, shape, done, s);
   return true;
 }
 template bool launch_gs_pair<float>(const StencilView<float, float>&, const float*, const float*, float*, int,
@@ -830,8 +832,9 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_matvec(StencilView<double,
   }
 }
 
-// x += alpha p, r -= alpha q, partial r.r; zero the preconditioner output and,
-// in mixed precision, write r32 = fl32(r / scale_next).
+// x += alpha p, r -= alpha q, partial r.r; zero the preconditioner's output z or
+// z32 (NULL: its cycle starts from zero without reading it) and, in mixed
+// precision, write r32 = fl32(r / scale_next).
 template <bool FU>
 __global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __restrict__ x, double* __restrict__ r,
                                                              const double* __restrict__ pv,
@@ -865,12 +868,9 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __re
         x[p] = madd<FU>(xv[c], alpha, pw[c]);
         const double rr = msub<FU>(rv[c], alpha, qv[c]);
         r[p] = rr;
-        if (r32) {
-          r32[p] = __double2float_rn(rmul(rr, inv));
-          z32[p] = 0.0f;
-        } else {
-          z[p] = 0.0;
-        }
+        if (r32) r32[p] = __double2float_rn(rmul(rr, inv));
+        if (z32) z32[p] = 0.0f;
+        if (z) z[p] = 0.0;
         acc = madd<FU>(acc, rr, rr);
       }
     }
@@ -904,12 +904,9 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
                        : row_residual<double, double, false, true, FU>(v, x, p, f[p]);
       if (!BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * ld)) continue;
       r[p] = rr;
-      if (r32) {
-        r32[p] = __double2float_rn(rmul(rr, inv));
-        z32[p] = 0.0f;
-      } else {
-        z[p] = 0.0;
-      }
+      if (r32) r32[p] = __double2float_rn(rmul(rr, inv));
+      if (z32) z32[p] = 0.0f;
+      if (z) z[p] = 0.0;
       acc = madd<FU>(acc, rr, rr);
     }
   double tot = block_sum(acc);

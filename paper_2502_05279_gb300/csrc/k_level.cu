@@ -35,25 +35,59 @@ struct LevelBlock {
   BlockCoef<T> k;
   BlockPlanes<T> q;
   size_t p;                     // its point A
-  int ld, ty;
+  int ld, ty, ic, jc;           // ic, jc: its coarse cell
   bool va, vb, vc, vd;
 };
 
-template <typename T, typename S>
-__device__ __forceinline__ void level_block(LevelBlock<T>& B, const StencilView<T, S>& v, int bi, int bj, T* planes) {
-  const int nb = (v.n + 1) / 2, rows = blockDim.y;
-  B.ld = v.ld;
+// A level's blocks: Dirichlet axes of n = 2 blocks - 1 points, whose last block
+// lacks its even points, and (PER) periodic axes of 2 blocks points, whose
+// block, point and coarse indexes wrap around; a tile wider than such an axis
+// holds copies of its blocks, of which the first is the one that owns.
+template <bool PER>
+struct LevelMap {
+  LevelGrid g;
+  int nbx, nby, ncx, ncy;
+  __device__ __forceinline__ explicit LevelMap(const LevelGrid& grid) : g(grid) {
+    nbx = (g.nx + 1) / 2, nby = (g.ny + 1) / 2;
+    ncx = PER && g.px ? g.nx / 2 : (g.nx - 1) / 2, ncy = PER && g.py ? g.ny / 2 : (g.ny - 1) / 2;
+  }
+  static __device__ __forceinline__ int wrap(int k, int n) { return k < 1 ? k + n : (k > n ? k - n : k); }   // 1 .. n
+  __device__ __forceinline__ int bx(int b) const { return PER && g.px ? (b % nbx + nbx) % nbx : b; }
+  __device__ __forceinline__ int by(int b) const { return PER && g.py ? (b % nby + nby) % nby : b; }
+  __device__ __forceinline__ bool last_x(int b) const { return !(PER && g.px) && b == nbx - 1; }
+  __device__ __forceinline__ bool last_y(int b) const { return !(PER && g.py) && b == nby - 1; }
+  __device__ __forceinline__ size_t at(int i, int j) const {
+    if (PER && g.px) i = wrap(i, g.nx);
+    if (PER && g.py) j = wrap(j, g.ny);
+    return (size_t)j * (g.nx + 2) + i;
+  }
+  __device__ __forceinline__ size_t coarse(int ic, int jc) const {
+    if (PER && g.px) ic = wrap(ic, ncx);
+    if (PER && g.py) jc = wrap(jc, ncy);
+    return (size_t)jc * (ncx + 2) + ic;
+  }
+  __device__ __forceinline__ size_t psc() const { return (size_t)(ncx + 2) * (ncy + 2); }
+};
+
+// ux, uy: the thread's block before wrapping.
+template <bool PER, typename T, typename S>
+__device__ __forceinline__ void level_block(LevelBlock<T>& B, const StencilView<T, S>& v, const LevelMap<PER>& m,
+                                            int ux, int uy, T* planes) {
+  const int bi = m.bx(ux), bj = m.by(uy);
+  B.ld = m.g.nx + 2;
   B.ty = threadIdx.y;
-  B.va = bi >= 0 && bi < nb && bj >= 0 && bj < nb;
-  B.vb = B.va && bi < nb - 1;
-  B.vc = B.va && bj < nb - 1;
+  B.va = bi >= 0 && bi < m.nbx && bj >= 0 && bj < m.nby;
+  B.vb = B.va && !m.last_x(bi);
+  B.vc = B.va && !m.last_y(bj);
   B.vd = B.vb && B.vc;
+  B.ic = bi + 1;
+  B.jc = bj + 1;
   const int i = 2 * bi + 1, j = 2 * bj + 1;
-  B.p = B.va ? (size_t)j * v.ld + i : 0;
-  B.q = block_planes(planes, LEVEL_NBX + 2, rows + 2, (int)threadIdx.x, (int)threadIdx.y);
+  B.p = B.va ? (size_t)j * B.ld + i : 0;
+  B.q = block_planes(planes, LEVEL_NBX + 2, (int)blockDim.y + 2, (int)threadIdx.x, (int)threadIdx.y);
   const S* const off[5] = {nullptr, v.W, v.S_, v.SW, v.NW};
   block_coef(B.k, i, j, B.va, B.vb, B.vc, B.vd, [&](int plane, int a, int b) -> T {
-    const size_t e = (size_t)b * v.ld + a;
+    const size_t e = m.at(a, b);
     return plane == 5 ? v.D[e] : cvt<T>(off[plane][e]);
   });
 }
@@ -77,8 +111,7 @@ __device__ __forceinline__ void level_planes(const LevelBlock<T>& B, const Block
 }
 
 template <typename T>
-__device__ __forceinline__ void level_store(const LevelBlock<T>& B, const BlockX<T>& x, T* out) {
-  const size_t ext = (size_t)B.ld * B.ld;
+__device__ __forceinline__ void level_store(const LevelBlock<T>& B, const BlockX<T>& x, T* out, size_t ext) {
   (void)ext;
   if (B.va && BMG_IN(DBG_STRIP_STORE, B.p, ext)) out[B.p] = x.a;
   if (B.vb && BMG_IN(DBG_STRIP_STORE, B.p + 1, ext)) out[B.p + 1] = x.b;
@@ -100,16 +133,18 @@ __device__ __forceinline__ void level_sweep(const LevelBlock<T>& B, const BlockX
                                  B.vd && B.ty >= lo - 1 && B.ty <= hi, sync);
 }
 
-template <typename T, typename S, bool NINE, bool FU>
+template <typename T, typename S, bool NINE, bool FU, bool PER>
 __global__ void __launch_bounds__(level_threads<T>())
-    k_level_down(StencilView<T, S> v, const T* __restrict__ ci, const T* __restrict__ f, const T* __restrict__ xin,
-                 T* __restrict__ xout, T* __restrict__ fc, T* __restrict__ xc, int nu1, const int* done) {
+    k_level_down(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* __restrict__ f,
+                 const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ fc, T* __restrict__ xc, int nu1,
+                 const int* done) {
   extern __shared__ __align__(16) unsigned char level_smem[];
+  const LevelMap<PER> m(grid);
   const int hx = 2 * nu1 + 1, hy = nu1 + 1, rows = blockDim.y;
-  const int bi = (int)blockIdx.x * (LEVEL_NBX - 2 * hx) + (int)threadIdx.x - hx;
-  const int bj = (int)blockIdx.y * (rows - 2 * hy) + (int)threadIdx.y - hy;
+  const int ux = (int)blockIdx.x * (LEVEL_NBX - 2 * hx) + (int)threadIdx.x - hx;
+  const int uy = (int)blockIdx.y * (rows - 2 * hy) + (int)threadIdx.y - hy;
   LevelBlock<T> B;
-  level_block(B, v, bi, bj, reinterpret_cast<T*>(level_smem));
+  level_block(B, v, m, ux, uy, reinterpret_cast<T*>(level_smem));
   BlockX<T> o = level_values(B, v.O);
   pdl_enter();
   if (stopped(done)) return;
@@ -125,37 +160,38 @@ __global__ void __launch_bounds__(level_threads<T>())
     else
       level_sweep<NINE, FU, false>(B, fb, x, lo, hi);
   }
-  const bool own = (int)threadIdx.x >= hx && (int)threadIdx.x < LEVEL_NBX - hx && B.ty >= hy && B.ty < rows - hy;
-  const int nc = (v.n - 1) / 2, ldc = nc + 2;
-  const size_t psc = plane_size(nc), pc = (size_t)(bj + 1) * ldc + bi + 1;
+  const bool own = (int)threadIdx.x >= hx && (int)threadIdx.x < LEVEL_NBX - hx && B.ty >= hy && B.ty < rows - hy &&
+                   ux < m.nbx && uy < m.nby;
+  const size_t psc = m.psc(), pc = (size_t)B.jc * (m.ncx + 2) + B.ic;
   const bool rab = B.ty >= hy && B.ty <= rows - hy, rcd = B.ty >= hy && B.ty < rows - hy;
   const BlockX<T> r = block_resid<NINE, FU>(B.k, o, fb, x, B.q, B.va && rab, B.vb && rab, B.vc && rcd, B.vd && rcd);
-  if (own) level_store(B, x, xout);
+  if (own) level_store(B, x, xout, (size_t)B.ld * (grid.ny + 2));
   __syncthreads();
   *B.q.a = r.a;
   *B.q.b = r.b;
   *B.q.c = r.c;
   __syncthreads();
-  if (own && B.vd && BMG_IN(DBG_RESTRICT_STORE, pc, (size_t)ldc * ldc)) {
+  if (own && B.vd && BMG_IN(DBG_RESTRICT_STORE, pc, psc)) {
     fc[pc] = block_restrict<FU>(r, B.q, [&](int k, int dic, int djc) {
-      return ci[k * psc + pc + (size_t)djc * ldc + dic];
+      return ci[k * psc + m.coarse(B.ic + dic, B.jc + djc)];
     });
     if (xc) xc[pc] = T(0);
   }
 }
 
-template <typename T, typename S, bool NINE, bool FU>
+template <typename T, typename S, bool NINE, bool FU, bool PER>
 __global__ void __launch_bounds__(level_threads<T>())
-    k_level_up(StencilView<T, S> v, const T* __restrict__ ci, const T* ec, const T* __restrict__ f,
+    k_level_up(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* ec, const T* __restrict__ f,
                const T* __restrict__ xin, T* __restrict__ xout, int nu2, const int* done) {
   extern __shared__ __align__(16) unsigned char level_smem[];
+  const LevelMap<PER> m(grid);
   const int hx = 2 * nu2, hy = nu2, rows = blockDim.y;
-  const int bi = (int)blockIdx.x * (LEVEL_NBX - 2 * hx) + (int)threadIdx.x - hx;
-  const int bj = (int)blockIdx.y * (rows - 2 * hy) + (int)threadIdx.y - hy;
+  const int ux = (int)blockIdx.x * (LEVEL_NBX - 2 * hx) + (int)threadIdx.x - hx;
+  const int uy = (int)blockIdx.y * (rows - 2 * hy) + (int)threadIdx.y - hy;
   LevelBlock<T> B;
-  level_block(B, v, bi, bj, reinterpret_cast<T*>(level_smem));
-  const int nc = (v.n - 1) / 2, ldc = nc + 2;
-  const size_t psc = plane_size(nc), pc = B.va ? (size_t)(bj + 1) * ldc + bi + 1 : (size_t)ldc + 1;
+  level_block(B, v, m, ux, uy, reinterpret_cast<T*>(level_smem));
+  const int ic = B.va ? B.ic : 1, jc = B.va ? B.jc : 1;
+  const size_t psc = m.psc(), pc = (size_t)jc * (m.ncx + 2) + ic;
   T w[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) w[k] = ci[k * psc + pc];
@@ -163,58 +199,92 @@ __global__ void __launch_bounds__(level_threads<T>())
   BlockX<T> x = level_values(B, xin);
   pdl_enter();
   if (stopped(done)) return;
-  block_interp<FU>(x, ec[pc - ldc - 1], ec[pc - ldc], ec[pc - 1], ec[pc], B.va, B.vb, B.vc, B.vd,
-                   [&](int k) { return w[k]; });
+  block_interp<FU>(x, ec[m.coarse(ic - 1, jc - 1)], ec[m.coarse(ic, jc - 1)], ec[m.coarse(ic - 1, jc)],
+                   ec[m.coarse(ic, jc)], B.va, B.vb, B.vc, B.vd, [&](int k) { return w[k]; });
   level_planes(B, x);
   __syncthreads();
   for (int s = 0; s < nu2; ++s) {
     const int rem = nu2 - 1 - s;
     level_sweep<NINE, FU, false>(B, fb, x, hy - rem, rows - 1 - hy + rem);
   }
-  if ((int)threadIdx.x >= hx && (int)threadIdx.x < LEVEL_NBX - hx && B.ty >= hy && B.ty < rows - hy)
-    level_store(B, x, xout);
+  if ((int)threadIdx.x >= hx && (int)threadIdx.x < LEVEL_NBX - hx && B.ty >= hy && B.ty < rows - hy && ux < m.nbx &&
+      uy < m.nby)
+    level_store(B, x, xout, (size_t)B.ld * (grid.ny + 2));
 }
 
 template <typename T>
 size_t level_bytes(int rows) { return (size_t)4 * (LEVEL_NBX + 2) * (rows + 2) * sizeof(T); }
 
-dim3 level_grid(int n, int rows, int hx, int hy) {
-  const int nb = (n + 1) / 2, ox = LEVEL_NBX - 2 * hx, oy = rows - 2 * hy;
-  return dim3((nb + ox - 1) / ox, (nb + oy - 1) / oy);
+dim3 level_grid(const LevelGrid& g, int rows, int hx, int hy) {
+  const int nbx = (g.nx + 1) / 2, nby = (g.ny + 1) / 2, ox = LEVEL_NBX - 2 * hx, oy = rows - 2 * hy;
+  return dim3((nbx + ox - 1) / ox, (nby + oy - 1) / oy);
+}
+
+template <typename T, typename S, bool PER>
+void down(const StencilView<T, S>& v, const LevelGrid& grid, int kind, const T* ci, const T* f, const T* xin, T* xout,
+          T* fc, T* xc, int nu1, int rows, const int* done, cudaStream_t s) {
+  const dim3 g = level_grid(grid, rows, 2 * nu1 + 1, nu1 + 1), b(LEVEL_NBX, rows);
+  const size_t bytes = level_bytes<T>(rows);
+  auto go = [&](auto kernel) { pdl_launch(kernel, g, b, bytes, s, v, grid, ci, f, xin, xout, fc, xc, nu1, done); };
+  if (kind == 9)
+    v.fused ? go(k_level_down<T, S, true, true, PER>) : go(k_level_down<T, S, true, false, PER>);
+  else
+    v.fused ? go(k_level_down<T, S, false, true, PER>) : go(k_level_down<T, S, false, false, PER>);
+  count_launch();
+}
+
+template <typename T, typename S, bool PER>
+void up(const StencilView<T, S>& v, const LevelGrid& grid, int kind, const T* ci, const T* ec, const T* f,
+        const T* xin, T* xout, int nu2, int rows, const int* done, cudaStream_t s) {
+  const dim3 g = level_grid(grid, rows, 2 * nu2, nu2), b(LEVEL_NBX, rows);
+  const size_t bytes = level_bytes<T>(rows);
+  auto go = [&](auto kernel) { pdl_launch(kernel, g, b, bytes, s, v, grid, ci, ec, f, xin, xout, nu2, done); };
+  if (kind == 9)
+    v.fused ? go(k_level_up<T, S, true, true, PER>) : go(k_level_up<T, S, true, false, PER>);
+  else
+    v.fused ? go(k_level_up<T, S, false, true, PER>) : go(k_level_up<T, S, false, false, PER>);
+  count_launch();
 }
 
 }  // namespace
 
+// Block rows per tile of a level whose halves of the cycle run as one launch
+// each (0: its steps are launched separately).  The change of a whole cycle
+// when one level runs by halves, us, fused arithmetic (8 / 16 / 32 rows):
+//   FP64  63: -15 / -6    127: -12 / -4    255: -3 / -10   511: 0 / -17   1023: +121 / +55
+//   FP32  127: -11 / -11 / -11   255: -14 / -13 / -11   511: -12 / -15 / -17
+//         1023: +4 / -13 / -9    2047: +66 / -2 / +12
+// (one rounding per operation: within a few us of these).  Small FP64 levels
+// want few warps per SM quarter, each of whose FP64 instructions takes 60
+// cycles; larger ones a small halo.  In FP32 32 rows pay while their tiles,
+// one to an SM, fit the chip at once.
+int level_rows(bool f64, int n) {
+  if (f64) return n > 512 ? 0 : n <= 128 ? 8 : 16;
+  return n > 1023 ? 0 : n == 511 ? 32 : 16;
+}
+
 template <typename T, typename S>
 void launch_level_down(const StencilView<T, S>& v, int kind, const T* ci, const T* f, const T* xin, T* xout, T* fc,
                        T* xc, int nu1, int rows, const int* done, cudaStream_t s) {
-  const dim3 g = level_grid(v.n, rows, 2 * nu1 + 1, nu1 + 1), b(LEVEL_NBX, rows);
-  const size_t bytes = level_bytes<T>(rows);
-  auto go = [&](auto kernel) { pdl_launch(kernel, g, b, bytes, s, v, ci, f, xin, xout, fc, xc, nu1, done); };
-  if (kind == 9) {
-    if (v.fused) go(k_level_down<T, S, true, true>);
-    else go(k_level_down<T, S, true, false>);
-  } else {
-    if (v.fused) go(k_level_down<T, S, false, true>);
-    else go(k_level_down<T, S, false, false>);
-  }
-  count_launch();
+  down<T, S, false>(v, LevelGrid{v.n, v.n, 0, 0}, kind, ci, f, xin, xout, fc, xc, nu1, rows, done, s);
 }
 
 template <typename T, typename S>
 void launch_level_up(const StencilView<T, S>& v, int kind, const T* ci, const T* ec, const T* f, const T* xin,
                      T* xout, int nu2, int rows, const int* done, cudaStream_t s) {
-  const dim3 g = level_grid(v.n, rows, 2 * nu2, nu2), b(LEVEL_NBX, rows);
-  const size_t bytes = level_bytes<T>(rows);
-  auto go = [&](auto kernel) { pdl_launch(kernel, g, b, bytes, s, v, ci, ec, f, xin, xout, nu2, done); };
-  if (kind == 9) {
-    if (v.fused) go(k_level_up<T, S, true, true>);
-    else go(k_level_up<T, S, true, false>);
-  } else {
-    if (v.fused) go(k_level_up<T, S, false, true>);
-    else go(k_level_up<T, S, false, false>);
-  }
-  count_launch();
+  up<T, S, false>(v, LevelGrid{v.n, v.n, 0, 0}, kind, ci, ec, f, xin, xout, nu2, rows, done, s);
+}
+
+void launch_level_down_p(const StencilView<double, double>& v, const LevelGrid& grid, int kind, const double* ci,
+                         const double* f, const double* xin, double* xout, double* fc, double* xc, int nu1, int rows,
+                         const int* done, cudaStream_t s) {
+  down<double, double, true>(v, grid, kind, ci, f, xin, xout, fc, xc, nu1, rows, done, s);
+}
+
+void launch_level_up_p(const StencilView<double, double>& v, const LevelGrid& grid, int kind, const double* ci,
+                       const double* ec, const double* f, const double* xin, double* xout, int nu2, int rows,
+                       const int* done, cudaStream_t s) {
+  up<double, double, true>(v, grid, kind, ci, ec, f, xin, xout, nu2, rows, done, s);
 }
 
 #define BMG_INST(T, S)                                                                                               \

@@ -265,11 +265,11 @@ __global__ void __launch_bounds__(tail_blocks<T>() * tail_blocks<T>(), 1)
     __syncwarp();
     if (nine_unknowns) {
       const int p = lane < COARSE_LANES ? (lane / 3 + 1) * 5 + lane % 3 + 1 : 6;
-      Coarse9 c9;
-      coarse9_load(c9, S.L9);
+      CoarseFactor<COARSE_LANES> c9;
+      coarse_load(c9, S.L9);
       c9.y = S.y9[lane < COARSE_LANES ? lane : 0];
       c9.yl = S.yl9[lane < COARSE_LANES ? lane : 0];
-      const T x = (T)coarse9_solve(c9, (double)f[p]);
+      const T x = (T)coarse_substitute(c9, (double)f[p]);
       __syncwarp();
       if (lane < COARSE_LANES) f[p] = x;
       __syncwarp();

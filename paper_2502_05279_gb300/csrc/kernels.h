@@ -107,7 +107,8 @@ void launch_wait_selftest(cudaStream_t s);
 // 0 .. 3 stream rows by bulk copies into 4 row slots (TY = W, 8, 16, 32, W the
 // smallest even height whose strips fit into one wave of resident warps),
 // shapes 4, 5 load them into registers (TY 32, 16).  The bulk-copy
-// shapes need the array layout above (else they run as shape 4).
+// shapes need the array layout above (else they run as shape 4).  xin NULL
+// (shapes 0 .. 3): from a zero iterate, which is not read.
 constexpr int GS_TILE_SHAPES = 6;
 template <typename S>
 void launch_gs_tile(const StencilView<float, S>& v, const float* f, const float* xin, float* xout, int shape,
@@ -117,10 +118,12 @@ void launch_gs_tile(const StencilView<float, S>& v, const float* f, const float*
 // intermediate array.  One warp per strip of 48 x TY points, rows by bulk
 // copies: shapes 0 .. 3 = TY W (one wave), 16, 32, 26 with 4, 4, 6, 4 row slots.  Needs
 // the guarded, aligned array layout; returns false (nothing launched) without it.
+// xin NULL: from a zero iterate.
 constexpr int GS_PAIR_SHAPES = 4;
 // The two pre-smoothing sweeps, the residual and its restriction in one pass
 // (44-column strips): fc, xc are the next level's right-hand side and iterate
-// (written / zeroed at its interior points).  Shape 0 or 1 (4- or 6-slot row
+// (written / zeroed at its interior points; xc may be NULL).  xin NULL: from a
+// zero iterate.  Shape 0 or 1 (4- or 6-slot row
 // rings).  Returns false when the arrays do not allow the bulk copies.
 template <typename S>
 bool launch_gs_pair_restrict(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
@@ -134,7 +137,7 @@ bool launch_gs_pair(const StencilView<float, S>& v, const float* f, const float*
 // 56 x TY points, rows copied per lane into RING row slots; shapes 0 .. 3 =
 // (TY, RING) = (one wave, 4), (16, 4), (one wave, 6), (8, 4), where "one
 // wave" is the smallest even TY whose strips all fit into the resident warps.
-// Needs v.D.
+// Needs v.D.  xin NULL: from a zero iterate (5 of the 9 FP64 operations a point).
 constexpr int GS_TILE64_SHAPES = 4;
 void launch_gs_tile64(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                       int shape, const int* done, cudaStream_t s);
@@ -146,12 +149,26 @@ void launch_gs_tile64(const StencilView<double, double>& v, const double* f, con
 // v, ci, and for up also f and xin, must have been written before the launch
 // that precedes on the stream started.
 constexpr int LEVEL_NU_MAX = 2;
+// Points of a level along x and y, and which of the axes are periodic.
+struct LevelGrid {
+  int nx, ny, px, py;
+};
 template <typename T, typename S>
 void launch_level_down(const StencilView<T, S>& v, int kind, const T* ci, const T* f, const T* xin, T* xout, T* fc,
                        T* xc, int nu1, int rows, const int* done, cudaStream_t s);
 template <typename T, typename S>
 void launch_level_up(const StencilView<T, S>& v, int kind, const T* ci, const T* ec, const T* f, const T* xin,
                      T* xout, int nu2, int rows, const int* done, cudaStream_t s);
+// The same for a level with periodic sides (v.n is not used, v.ld = nx + 2).
+void launch_level_down_p(const StencilView<double, double>& v, const LevelGrid& grid, int kind, const double* ci,
+                         const double* f, const double* xin, double* xout, double* fc, double* xc, int nu1, int rows,
+                         const int* done, cudaStream_t s);
+void launch_level_up_p(const StencilView<double, double>& v, const LevelGrid& grid, int kind, const double* ci,
+                       const double* ec, const double* f, const double* xin, double* xout, int nu2, int rows,
+                       const int* done, cudaStream_t s);
+// Block rows per tile of a level of about n points a side whose halves of the
+// cycle run as one launch each (0: its steps are launched separately).
+int level_rows(bool f64, int n);
 template <typename T, typename S>
 void launch_resid_restrict(const StencilView<T, S>& v, int kind, const T* ci, const T* x, const T* f, T* fc,
                            T* xc, const int* done, cudaStream_t s);

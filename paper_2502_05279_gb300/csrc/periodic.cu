@@ -20,7 +20,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "cycle_device.cuh"
+#include "block_device.cuh"
 #include "kernels.h"
 #include "periodic.h"
 
@@ -390,7 +390,8 @@ __global__ void __launch_bounds__(256) k_p_gs_rows(PGeom g, const double* __rest
 // row 1, computed from copies of the old values and never stored.  Every point
 // takes the operands of the colour-by-colour sweep in the same order, so the
 // result is bit-identical to it.
-template <int RING, bool FU>
+// ZERO: from a zero iterate, which is not read.
+template <int RING, bool FU, bool ZERO>
 __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __restrict__ st,
                                                const double* __restrict__ f, const double* __restrict__ xin,
                                                double* __restrict__ xout, int sx, int sy, int ty,
@@ -431,7 +432,7 @@ __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __r
       const bool oka = rin && cpa && BMG_IN(DBG_PERIODIC, pa, ps), okb = rin && cpb && BMG_IN(DBG_PERIODIC, pb, ps);
       double* d = reinterpret_cast<double*>(ring + (q % RING) * dev::STRIP64_SLOT) + 2 * lane;
 #pragma unroll
-      for (int k = 0; k < 7; ++k) {
+      for (int k = ZERO ? 1 : 0; k < 7; ++k) {
         const double* a = k == 0 ? xin : k == 1 ? f : st + (size_t)plane[k] * ps;
         dev::cp_async8(d + 64 * k, a + (oka ? pa : 0), oka);
         dev::cp_async8(d + 64 * k + 1, a + (okb ? pb : 0), okb);
@@ -443,7 +444,7 @@ __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __r
   for (int q = 0; q < RING; ++q) issue(q);
   auto take = [&](int q, Row& R) {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 1) : "memory");
-    dev::row64_read(ring + (q % RING) * dev::STRIP64_SLOT, lane, R);
+    dev::row64_read<ZERO>(ring + (q % RING) * dev::STRIP64_SLOT, lane, R);
     issue(q + RING);
   };
   auto store = [&](int j, const Row& R) {
@@ -452,12 +453,24 @@ __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __r
     if (ic <= nx && BMG_IN(DBG_PERIODIC, p, ps)) xout[p] = R.xa;
     if (ic + 1 <= nx && BMG_IN(DBG_PERIODIC, p + 1, ps)) xout[p + 1] = R.xb;
   };
+  auto odd = [&](const Row& L, Row& M, const Row& U) {     // colours 1, 2
+    if constexpr (ZERO)
+      dev::strip_row_zero<true, double, double, FU>(L, M, U, c1, c2);
+    else
+      dev::strip_row<double, double, FU>(L, M, U, c1, c2);
+  };
+  auto even = [&](const Row& L, Row& M, const Row& U) {    // colours 3, 4
+    if constexpr (ZERO)
+      dev::strip_row_zero<false, double, double, FU>(L, M, U, c3, c4);
+    else
+      dev::strip_row<double, double, FU>(L, M, U, c3, c4);
+  };
   Row P0, P1, Q0, Q1;
   take(0, P1);
   take(1, Q0);
   take(2, Q1);
   if (j0 <= rlim) {
-    dev::strip_row<double, double, FU>(P1, Q0, Q1, c1, c2);   // row j0: colours 1, 2
+    odd(P1, Q0, Q1);                              // row j0
     store(j0, Q0);
   }
   auto step = [&](int m, Row& E0, Row& E1, Row& E2, Row& E3) {
@@ -465,11 +478,11 @@ __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __r
     take(2 * m + 1, E2);
     take(2 * m + 2, E3);
     if (a <= rlim) {
-      dev::strip_row<double, double, FU>(E1, E2, E3, c1, c2); // row a: colours 1, 2
+      odd(E1, E2, E3);                            // row a
       if (a < j1) store(a, E2);
     }
     if (a - 1 <= ny) {
-      dev::strip_row<double, double, FU>(E0, E1, E2, c3, c4); // row a - 1: colours 3, 4
+      even(E0, E1, E2);                           // row a - 1
       store(a - 1, E1);
     }
   };
@@ -484,7 +497,7 @@ __device__ __forceinline__ void p_strip64_body(const PGeom& g, const double* __r
 constexpr int P_STRIP_WARPS = 4, P_STRIP_RING = 4;
 constexpr size_t P_STRIP_SMEM = (size_t)P_STRIP_WARPS * P_STRIP_RING * dev::STRIP64_SLOT;
 
-template <bool FU>
+template <bool FU, bool ZERO>
 __global__ void __launch_bounds__(32 * P_STRIP_WARPS, 4) k_p_gs_strip(PGeom g, const double* __restrict__ st,
                                                                    const double* __restrict__ f,
                                                                    const double* __restrict__ xin,
@@ -495,7 +508,7 @@ __global__ void __launch_bounds__(32 * P_STRIP_WARPS, 4) k_p_gs_strip(PGeom g, c
   const int nbx = (g.nx + 55) / 56, nby = (g.ny + ty - 1) / ty;
   const int w = threadIdx.x >> 5, s = blockIdx.x * P_STRIP_WARPS + w;
   if (s >= nbx * nby) return;                     // whole warps only
-  p_strip64_body<P_STRIP_RING, FU>(g, st, f, xin, xout, s % nbx, s / nbx, ty,
+  p_strip64_body<P_STRIP_RING, FU, ZERO>(g, st, f, xin, xout, s % nbx, s / nbx, ty,
                                    p_strip_smem + (size_t)w * P_STRIP_RING * dev::STRIP64_SLOT);
 }
 
@@ -550,7 +563,7 @@ __global__ void k_p_restrict(PGeom g, const double* __restrict__ ci, const doubl
   const size_t pc = (size_t)jc * (c.ncx + 2) + ic;
   if (BMG_IN(DBG_PERIODIC, pc, psc)) {
     fc[pc] = t;
-    xc[pc] = 0.0;   // the coarse iterate starts from zero (its ghost lines stay zero)
+    if (xc) xc[pc] = 0.0;   // the coarse iterate starts from zero (its ghost lines stay zero)
   }
 }
 
@@ -614,25 +627,20 @@ __global__ void k_p_interp(PGeom g, const double* __restrict__ ci, const double*
   }
 }
 
-// L L^T x = f on the coarsest level (one thread, m <= 16): forward then backward
-// substitution, inner sums in increasing index order.
+// L L^T x = f on the coarsest level, m = 9, 12 or 16 unknowns, one warp
+// (the row-by-row order of every sum).
+template <int M>
 __global__ void k_p_coarse_solve(PGeom g, const double* __restrict__ L, const double* __restrict__ f,
                                  double* __restrict__ x, const int* done) {
+  const int lane = threadIdx.x, k = lane < M ? lane : 0;
+  dev::CoarseFactor<M> c;
+  dev::coarse_load(c, L);
+  c.y = quot_recip(c.dg, &c.yl);
+  pdl_enter();
   if (dev::stopped(done)) return;
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  const int m = g.nx * g.ny;
-  double y[16], z[16];
-  for (int i = 0; i < m; ++i) {
-    double s = f[(size_t)(i / g.nx + 1) * (g.nx + 2) + (i % g.nx + 1)];
-    for (int k = 0; k < i; ++k) s = rsub(s, rmul(L[(size_t)i * m + k], y[k]));
-    y[i] = rdiv(s, L[(size_t)i * m + i]);
-  }
-  for (int i = m - 1; i >= 0; --i) {
-    double s = y[i];
-    for (int k = i + 1; k < m; ++k) s = rsub(s, rmul(L[(size_t)k * m + i], z[k]));
-    z[i] = rdiv(s, L[(size_t)i * m + i]);
-  }
-  for (int i = 0; i < m; ++i) x[(size_t)(i / g.nx + 1) * (g.nx + 2) + (i % g.nx + 1)] = z[i];
+  const size_t p = (size_t)(k / g.nx + 1) * (g.nx + 2) + (k % g.nx + 1);
+  const double v = dev::coarse_substitute(c, f[p]);
+  if (lane < M && BMG_IN(DBG_PERIODIC, p, g.ps())) x[p] = v;
 }
 
 // ---- flexible CG (FCG(1)) on level 0, preconditioned by the periodic V-cycle ----
@@ -749,7 +757,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_update(PGeom g, dou
       x[p] = madd<FU>(x[p], alpha, pv[p]);
       const double rr = msub<FU>(r[p], alpha, q[p]);
       r[p] = rr;
-      z[p] = 0.0;
+      if (z) z[p] = 0.0;
       acc = madd<FU>(acc, rr, rr);
     }
   const double tot = dev::block_sum(acc);
@@ -785,6 +793,7 @@ struct PerLevel {
   double* xb = nullptr;   // second iterate for strip sweeps (9-point levels above the coarsest)
   int ty = 0;             // strip height
   bool strip = false;     // swept by the strip kernel (else by the row-parity pair, in place)
+  int rows = 0;           // > 0: runs by halves of the cycle (launch_level_down_p), tiles of this many block rows
 };
 
 struct PerHier {
@@ -800,8 +809,10 @@ struct PerHier {
 // kernel's resident warps (a warp walks its strip serially; a partial second
 // wave would leave most FP64 pipes idle).
 static int strip_height(const PGeom& g, int fused) {
-  auto k = fused ? k_p_gs_strip<true> : k_p_gs_strip<false>;
+  auto k = fused ? k_p_gs_strip<true, false> : k_p_gs_strip<false, false>;
+  auto k0 = fused ? k_p_gs_strip<true, true> : k_p_gs_strip<false, true>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P_STRIP_SMEM);
+  cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P_STRIP_SMEM);
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -847,7 +858,8 @@ void per_free(PerHier* P) {
 
 namespace {
 template <bool FU>
-double* per_sweep(const PerLevel& L, const double* f, double* x, double* home, const int* done, cudaStream_t s);
+double* per_sweep(const PerLevel& L, const double* f, double* x, double* home, const int* done, cudaStream_t s,
+                  bool zero = false);
 
 // The sweep of each 9-point level: the strip walk or the row-parity pair,
 // whichever takes less time here over 3 sweeps (after one untimed), run on
@@ -858,7 +870,7 @@ int tune_sweeps(PerHier* P, cudaStream_t s) {
   int rc = cuda_check(cudaEventCreate(&e0), "periodic setup: event");
   if (!rc) rc = cuda_check(cudaEventCreate(&e1), "periodic setup: event");
   for (PerLevel& L : P->lv) {
-    if (rc || !L.xb) continue;
+    if (rc || !L.xb || L.rows > 0) continue;
     float t[2] = {0.f, 0.f};
     for (int k = 0; k < 2 && !rc; ++k) {
       L.strip = k == 0;
@@ -881,7 +893,7 @@ int tune_sweeps(PerHier* P, cudaStream_t s) {
 }  // namespace
 
 int per_setup(PerHier** out, int kind, const double* coef, int nx, int ny, int periodic, int fused, int nu1,
-              int nu2, int sweep, int krylov, cudaStream_t s) {
+              int nu2, int sweep, int krylov, bool halves, cudaStream_t s) {
   *out = nullptr;
   const int nlev = per_levels_for(nx, ny, periodic);
   if (nlev < 1)
@@ -909,7 +921,10 @@ int per_setup(PerHier** out, int kind, const double* coef, int nx, int ny, int p
       rc = palloc(&L.ci, 8 * psc, s);
       if (!rc) rc = palloc(&L.r, ps, s);
     }
-    if (!rc && sweep != PER_SWEEP_ROWS && l + 1 < nlev && L.kind == 9) rc = palloc(&L.xb, ps, s);
+    if (halves && sweep == PER_SWEEP_AUTO && nu1 >= 1 && nu2 >= 1 && nu1 <= LEVEL_NU_MAX && nu2 <= LEVEL_NU_MAX &&
+        l + 1 < nlev)
+      L.rows = level_rows(true, L.g.nx > L.g.ny ? L.g.nx : L.g.ny);
+    if (!rc && ((sweep != PER_SWEEP_ROWS && l + 1 < nlev && L.kind == 9) || L.rows > 0)) rc = palloc(&L.xb, ps, s);
     if (!rc && l > 0) rc = palloc(&L.x, ps, s);
     if (!rc && l > 0) rc = palloc(&L.f, ps, s);
   }
@@ -925,7 +940,7 @@ int per_setup(PerHier** out, int kind, const double* coef, int nx, int ny, int p
     return rc;
   }
   for (PerLevel& L : P->lv)
-    if (L.xb) {
+    if (L.xb && L.kind == 9) {
       L.ty = strip_height(L.g, fused);
       L.strip = true;
     }
@@ -978,12 +993,14 @@ struct Bracket {
 // One sweep starting from x, which is the level's iterate `home` or its
 // second iterate L.xb; returns the array holding the result: the other one of
 // the two for a level swept by strips (one launch), x itself otherwise.
+// zero: x holds zeros (the strips then do not read it).
 template <bool FU>
-double* per_sweep(const PerLevel& L, const double* f, double* x, double* home, const int* done, cudaStream_t s) {
+double* per_sweep(const PerLevel& L, const double* f, double* x, double* home, const int* done, cudaStream_t s,
+                  bool zero) {
   if (L.strip) {
     double* out = x == L.xb ? home : L.xb;
     const int warps = ((L.g.nx + 55) / 56) * ((L.g.ny + L.ty - 1) / L.ty);
-    k_p_gs_strip<FU><<<(warps + P_STRIP_WARPS - 1) / P_STRIP_WARPS, 32 * P_STRIP_WARPS, P_STRIP_SMEM, s>>>(
+    (zero ? k_p_gs_strip<FU, true> : k_p_gs_strip<FU, false>)<<<(warps + P_STRIP_WARPS - 1) / P_STRIP_WARPS, 32 * P_STRIP_WARPS, P_STRIP_SMEM, s>>>(
         L.g, L.st, f, x, out, L.ty, done);
     count_launch();
     return out;
@@ -1021,29 +1038,52 @@ int per_residual(const PerLevel& L, const double* x, const double* f, double* r,
   return G;
 }
 
+StencilView<double, double> per_view(const PerHier* P, const PerLevel& L) {
+  const size_t ps = L.g.ps();
+  return {L.st, L.st + ps, L.st + 2 * ps, L.st + 3 * ps, L.st + 4 * ps, L.st + 5 * ps, 0, L.g.nx + 2, P->fused};
+}
+
+// Level l, started from a zero iterate, does not read one.
+bool per_zero_aware(const PerHier* P, int l, const PerMarks* mk) {
+  const PerLevel& L = P->lv[l];
+  return (L.rows > 0 && !mk) || (L.strip && P->nu1 > 0);
+}
+
+// zero: the iterate is zero on entry.
 template <bool FU>
 void per_vcycle(PerHier* P, int l, double* x, const double* f, const int* done, cudaStream_t s,
-                const PerMarks* mk) {
+                const PerMarks* mk, bool zero) {
   PerLevel& L = P->lv[l];
   if (l + 1 == (int)P->lv.size()) {
     Bracket b(mk, l, BMG_K_COARSE);
-    k_p_coarse_solve<<<1, 1, 0, s>>>(L.g, P->L, f, x, done);
+    const int m = L.g.nx * L.g.ny;
+    pdl_launch(m == 9 ? k_p_coarse_solve<9> : m == 12 ? k_p_coarse_solve<12> : k_p_coarse_solve<16>, 1, 32, 0, s, L.g,
+               P->L, f, x, done);
     count_launch();
     return;
   }
   PerLevel& C = P->lv[l + 1];
+  double* const xc = per_zero_aware(P, l + 1, mk) ? nullptr : C.x;   // zeroed unless nothing reads it
+  if (L.rows > 0 && !mk) {
+    const LevelGrid g{L.g.nx, L.g.ny, L.g.px, L.g.py};
+    const StencilView<double, double> v = per_view(P, L);
+    launch_level_down_p(v, g, L.kind, L.ci, f, zero ? nullptr : x, L.xb, C.f, xc, P->nu1, L.rows, done, s);
+    per_vcycle<FU>(P, l + 1, C.x, C.f, done, s, mk, true);
+    launch_level_up_p(v, g, L.kind, L.ci, C.x, f, L.xb, x, P->nu2, L.rows, done, s);
+    return;
+  }
   double* cur = x;                                // where the iterate is
   for (int k = 0; k < P->nu1; ++k) {
     Bracket b(mk, l, BMG_K_RELAX);
-    cur = per_sweep<FU>(L, f, cur, x, done, s);
+    cur = per_sweep<FU>(L, f, cur, x, done, s, zero && k == 0);
   }
   {
     Bracket b(mk, l, BMG_K_RESID_RESTRICT);
     per_residual<FU>(L, cur, f, L.r, nullptr, done, s);
-    k_p_restrict<FU><<<pgrid(C.g.nx, C.g.ny), dim3(PBX, PBY), 0, s>>>(L.g, L.ci, L.r, C.f, C.x, done);
+    k_p_restrict<FU><<<pgrid(C.g.nx, C.g.ny), dim3(PBX, PBY), 0, s>>>(L.g, L.ci, L.r, C.f, xc, done);
     count_launch();
   }
-  per_vcycle<FU>(P, l + 1, C.x, C.f, done, s, mk);
+  per_vcycle<FU>(P, l + 1, C.x, C.f, done, s, mk, true);
   {
     // corrected iterate into the array from which the nu2 post-sweeps end in x
     Bracket b(mk, l, BMG_K_INTERP);
@@ -1082,7 +1122,7 @@ namespace {
 // One FCG step after the preconditioner z = V(r): z.q and beta, p, q = A p with
 // p.q and p.r, then the x / r update with the r.r partial sums; returns G.
 template <bool FU>
-int per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t s) {
+int per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t s, bool zero_z) {
   const PerLevel& L = P->lv[0];
   const size_t ps = L.g.ps();
   double *r = P->kr, *z = P->kr + ps, *pv = P->kr + 2 * ps, *q = P->kr + 3 * ps;
@@ -1098,7 +1138,7 @@ int per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t
     k_p_fcg_matvec<false, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, pv, r, q, partials, ctl);
   count_launch();
   launch_fcg_reduce(partials, G, ctl, 1, s);
-  k_p_fcg_update<FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, x, r, pv, q, z, partials, ctl);
+  k_p_fcg_update<FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, x, r, pv, q, zero_z ? z : nullptr, partials, ctl);
   count_launch();
   return G;
 }
@@ -1113,16 +1153,18 @@ void per_enqueue_iteration(PerHier* P, const double* rhs, double* x, double* par
     const size_t ps = P->lv[0].g.ps();
     double *r = P->kr, *z = P->kr + ps;
     if (P->fused)
-      per_vcycle<true>(P, 0, z, r, done, s, mk);
+      per_vcycle<true>(P, 0, z, r, done, s, mk, true);
     else
-      per_vcycle<false>(P, 0, z, r, done, s, mk);
+      per_vcycle<false>(P, 0, z, r, done, s, mk, true);
     Bracket b(mk, 0, BMG_K_FCG);
-    G = P->fused ? per_fcg_step<true>(P, x, partials, ctl, s) : per_fcg_step<false>(P, x, partials, ctl, s);
+    const bool zero_z = !per_zero_aware(P, 0, mk);
+    G = P->fused ? per_fcg_step<true>(P, x, partials, ctl, s, zero_z)
+                 : per_fcg_step<false>(P, x, partials, ctl, s, zero_z);
   } else {
     if (P->fused)
-      per_vcycle<true>(P, 0, x, rhs, done, s, mk);
+      per_vcycle<true>(P, 0, x, rhs, done, s, mk, false);
     else
-      per_vcycle<false>(P, 0, x, rhs, done, s, mk);
+      per_vcycle<false>(P, 0, x, rhs, done, s, mk, false);
     Bracket b(mk, 0, BMG_K_NORM);
     G = P->fused ? per_residual<true>(P->lv[0], x, rhs, nullptr, partials, done, s)
                  : per_residual<false>(P->lv[0], x, rhs, nullptr, partials, done, s);

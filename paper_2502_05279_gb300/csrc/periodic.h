@@ -30,11 +30,13 @@ int per_levels_for(int nx, int ny, int periodic);
 // row-parity launches in place (PER_SWEEP_ROWS), by the one-pass strip kernel
 // into a second iterate (PER_SWEEP_STRIP), or per level by whichever of the
 // two is faster, timed during setup (PER_SWEEP_AUTO).
+// halves: with PER_SWEEP_AUTO, the smaller levels run by halves of the cycle
+// (launch_level_down_p) outside profiling.
 // krylov: the solve runs flexible CG (FCG(1)) preconditioned by one V(nu1, nu2)
 // cycle per step instead of stationary cycles.
 enum { PER_SWEEP_AUTO = 0, PER_SWEEP_ROWS = 1, PER_SWEEP_STRIP = 2 };
 int per_setup(PerHier** out, int kind, const double* coef, int nx, int ny, int periodic, int fused, int nu1,
-              int nu2, int sweep, int krylov, cudaStream_t s);
+              int nu2, int sweep, int krylov, bool halves, cudaStream_t s);
 void per_free(PerHier* P);
 
 // Profiling brackets around each step's launches (begin: level and BMG_K_*
