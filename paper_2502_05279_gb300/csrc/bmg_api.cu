@@ -2009,6 +2009,7 @@ struct bmg_batch {
     int tile = -1, pair = -1;   // one-pass / two-sweep shapes chosen for an FP32 group (-1: row kernel / none)
     int multi = 0;              // 2 or 4: one-pass sweeps with that many members per warp (shared operator)
     int dir = 0;                // while a cycle is enqueued: 0 = iterate in x, 1 = in x2
+    int rows = 0;               // > 0: the stage runs by halves of the cycle, tiles of this many block rows
     size_t elem = 0;
     void* d = nullptr;
     std::vector<char> host;
@@ -2133,15 +2134,15 @@ int build_batch_tables(bmg_batch* B, const double* const* rhs, double* const* x)
       }
       if (storage == 0) {
         LevelDesc<double, double> d{view64(lv), lv.ci, l == 0 ? x[p] : lv.x, l == 0 ? rhs[p] : lv.f,
-                                    C ? C->x : nullptr, C ? C->f : nullptr, done, h->Lfac, h->work, lv.x64b};
+                                    C ? C->x : nullptr, C ? C->f : nullptr, done, h->Lfac, h->work, lv.x64b, l > 0};
         append_desc(g, d);
       } else if (storage == 2) {
         LevelDesc<float, __nv_bfloat16> d{viewbf(lv), lv.ci32, lv.x32, lv.f32, C ? C->x32 : nullptr,
-                                          C ? C->f32 : nullptr, done, h->Lfac, h->work, lv.x32b};
+                                          C ? C->f32 : nullptr, done, h->Lfac, h->work, lv.x32b, l > 0};
         append_desc(g, d);
       } else {
         LevelDesc<float, float> d{view32(lv), lv.ci32, lv.x32, lv.f32, C ? C->x32 : nullptr, C ? C->f32 : nullptr,
-                                  done, h->Lfac, h->work, lv.x32b};
+                                  done, h->Lfac, h->work, lv.x32b, l > 0};
         append_desc(g, d);
       }
     }
@@ -2234,12 +2235,29 @@ void group_coarse(bmg_batch* B, bmg_batch::Group& g) {
   else launch_coarse_b(gdesc<float, __nv_bfloat16>(g), g.count, B->ws);
 }
 
+// One half of the cycle on a stage that runs by halves.
+void group_half(bmg_batch* B, bmg_batch::Group& g, bool up) {
+  auto go = [&](const auto* d) {
+    if (up)
+      launch_level_up_b(d, g.count, g.n, g.kind, B->nu2, g.rows, B->ws, B->arith);
+    else
+      launch_level_down_b(d, g.count, g.n, g.kind, B->nu1, g.rows, B->ws, B->arith);
+  };
+  if (g.storage == 0) go(gdesc<double, double>(g));
+  else if (g.storage == 1) go(gdesc<float, float>(g));
+  else go(gdesc<float, __nv_bfloat16>(g));
+}
+
 // One V(nu1, nu2) cycle of every problem: down the stages (largest first), the
 // coarsest solves, back up.
 void batch_vcycle(bmg_batch* B) {
   for (int b = B->bmax; b >= 1; --b) {
     for (auto& g : B->stages[b]) {
       g.dir = 0;
+      if (g.count && g.rows > 0) {
+        group_half(B, g, false);
+        continue;
+      }
       group_relax(B, g, B->nu1);
       group_restrict(B, g);
     }
@@ -2255,6 +2273,10 @@ void batch_vcycle(bmg_batch* B) {
   for (auto& g : B->stages[0]) group_coarse(B, g);
   for (int b = 1; b <= B->bmax; ++b)
     for (auto& g : B->stages[b]) {
+      if (g.count && g.rows > 0) {
+        group_half(B, g, true);
+        continue;
+      }
       group_interp(B, g);
       group_relax(B, g, B->nu2);
     }
@@ -2559,6 +2581,35 @@ int force_rhs_block(bmg_batch* B) {
   return BMG_OK;
 }
 
+// Block rows per tile of a batched stage that runs by halves (0: step by step).
+// The change of a whole batch iteration when one stage runs by halves, us,
+// fused arithmetic, 16 rows (FP64 also 8), at 127 / 255 / 511 / 1023:
+//   40 problems FP32: -8 / -5 / -22 / +44    10 problems FP32: -13 / -15 / -8 / -7
+//   10 problems BF16: -28 / -28 / -9 / -1
+//   16 right-hand sides of 1023^2 FP32: -13 / -8 / +17 / +148 (block sweeps read the shared stencil once)
+//   FP64 at 63 / 127: 40 problems -4 / +13, 10 problems -5 (8 rows) / -1, 8 right-hand sides -8 (8 rows) / -2:
+//   the halos' FP64 work costs more than the launches as soon as the problems fill the chip
+int batch_rows(bool f64, int n, int count, bool shared) {
+  if (f64) return n > 63 ? 0 : count <= 16 ? 8 : 16;
+  return n <= 255 || (n <= 511 && !shared) ? 16 : 0;
+}
+
+// The stages that run by halves, and their second iterates: graphs on, no
+// smoother or right-hand-side blocking forced, sweep counts the tiles allow.
+int choose_batch_halves(bmg_batch* B) {
+  if (!B->use_graph || B->smoother != BMG_SMOOTHER_AUTO || B->rhs_block > BMG_RHS_BLOCK_OFF || B->nu1 < 1 ||
+      B->nu2 < 1 || B->nu1 > LEVEL_NU_MAX || B->nu2 > LEVEL_NU_MAX)
+    return BMG_OK;
+  for (int b = 1; b <= B->bmax; ++b)
+    for (auto& g : B->stages[b]) {
+      if (!g.count) continue;
+      g.rows = batch_rows(B->precision == BMG_FP64, g.n, g.count, group_shared(B, g, b));
+      if (g.rows > 0)
+        if (int rc = group_alloc_x2(B, g, b)) return rc;
+    }
+  return BMG_OK;
+}
+
 int autotune_batch(bmg_batch* B) {
   std::lock_guard<std::mutex> guard(tune_lock());
   // descriptor contents are needed: build the tables with the internal level
@@ -2720,6 +2771,7 @@ int batch_finish(bmg_batch* B, int rc) {
   if (!rc) rc = batch_ensure_ctl(B, 64);
   if (!rc && B->smoother >= BMG_SMOOTHER_TILE) rc = force_batch_onepass(B);
   if (!rc && B->use_graph) rc = autotune_batch(B);
+  if (!rc) rc = choose_batch_halves(B);
   if (!rc) rc = force_rhs_block(B);
   if (!rc) rc = cuda_check(cudaStreamSynchronize(B->ws), "batched setup");
   return rc;

@@ -163,6 +163,7 @@ struct Ctl {
   // flexible CG scalars
   double zq, pq, pr, pq_prev;
   double beta;           // -zq / pq_prev of the current step, formed once by the zq reduction
+  double alpha;          // pr / pq of the current step, formed once by the pq, pr reduction
   int first;             // 1 until the first direction is formed
   int pad2;
   double hist[1];        // [maxit + 1] residual norms (allocated past the struct)

@@ -1557,8 +1557,22 @@ static __device__ __noinline__ float narrow_scaled_slow(double r, double inv) {
   return __double2float_rn(rmul(r, inv));
 }
 
+// 1 / s for the refinement scales, powers of two: formed from the exponent (a
+// division takes ten FP64 operations of every thread, as much as the residual
+// of one point; a block of a 1023-column row has four points a thread).
+__device__ __forceinline__ double pow2_inverse(double s) {
+  const unsigned hi = (unsigned)__double2hiint(s), e = hi >> 20;
+  if (e - 1u < 2045u && (hi & 0xfffffu) == 0 && __double2loint(s) == 0)
+    return __hiloint2double((int)((2046u - e) << 20), 0);
+  return rdiv(1.0, s);
+}
+
+// (on the bit pattern: inv is a power of two, or takes the FP64 product)
 __device__ __forceinline__ float narrow_scale32(double inv) {
-  return inv >= 0x1p-125 && inv <= 0x1p125 ? (float)inv : 0.0f;
+  const unsigned hi = (unsigned)__double2hiint(inv);
+  const int e = (int)(hi >> 20) - 1023;
+  return (hi & 0xfffffu) == 0 && __double2loint(inv) == 0 && e >= -125 && e <= 125 ? __uint_as_float((unsigned)(e + 127) << 23)
+                                                                                 : 0.0f;
 }
 
 __device__ __forceinline__ float narrow_scaled(double r, double inv, float inv32) {
@@ -1605,7 +1619,7 @@ __device__ __forceinline__ void ir_residual_body(const StencilView<double, doubl
                                                  double* __restrict__ partials, Ctl* ctl, int b, int G) {
   const int n = v.n, ld = v.ld;
   const double s = ctl->scale_next;
-  const double inv = 1.0 / s;   // exact: s is a power of two
+  const double inv = pow2_inverse(s);
   const float inv32 = narrow_scale32(inv);
   double acc = 0.0;
   for (int j = 1 + b; j <= n; j += G)

@@ -764,6 +764,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_reduce(const double* __res
     if (threadIdx.x == 0) {
       ctl->pq = a;
       ctl->pr = b;
+      ctl->alpha = rdiv(b, a);   // one division per step, not per thread
     }
   }
 }
@@ -844,9 +845,9 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __re
   pdl_enter();
   if (ctl->done) return;
   const int ld = n + 2;
-  const double alpha = rdiv(ctl->pr, ctl->pq);
+  const double alpha = ctl->alpha;
   const double s = ctl->scale_next;
-  const double inv = 1.0 / s;
+  const double inv = pow2_inverse(s);
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS * FCG_COLS) {
@@ -895,7 +896,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
   pdl_enter();
   const int n = v.n, ld = v.ld;
   const double s = ctl->scale_next;
-  const double inv = 1.0 / s;
+  const double inv = pow2_inverse(s);
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS) {

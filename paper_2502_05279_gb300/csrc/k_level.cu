@@ -134,10 +134,9 @@ __device__ __forceinline__ void level_sweep(const LevelBlock<T>& B, const BlockX
 }
 
 template <typename T, typename S, bool NINE, bool FU, bool PER>
-__global__ void __launch_bounds__(level_threads<T>())
-    k_level_down(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* __restrict__ f,
-                 const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ fc, T* __restrict__ xc, int nu1,
-                 const int* done) {
+__device__ __forceinline__ void down_body(const StencilView<T, S>& v, const LevelGrid& grid, const T* __restrict__ ci,
+                                          const T* __restrict__ f, const T* __restrict__ xin, T* __restrict__ xout,
+                                          T* __restrict__ fc, T* __restrict__ xc, int nu1, const int* done) {
   extern __shared__ __align__(16) unsigned char level_smem[];
   const LevelMap<PER> m(grid);
   const int hx = 2 * nu1 + 1, hy = nu1 + 1, rows = blockDim.y;
@@ -180,9 +179,9 @@ __global__ void __launch_bounds__(level_threads<T>())
 }
 
 template <typename T, typename S, bool NINE, bool FU, bool PER>
-__global__ void __launch_bounds__(level_threads<T>())
-    k_level_up(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* ec, const T* __restrict__ f,
-               const T* __restrict__ xin, T* __restrict__ xout, int nu2, const int* done) {
+__device__ __forceinline__ void up_body(const StencilView<T, S>& v, const LevelGrid& grid, const T* __restrict__ ci,
+                                        const T* ec, const T* __restrict__ f, const T* __restrict__ xin,
+                                        T* __restrict__ xout, int nu2, const int* done) {
   extern __shared__ __align__(16) unsigned char level_smem[];
   const LevelMap<PER> m(grid);
   const int hx = 2 * nu2, hy = nu2, rows = blockDim.y;
@@ -210,6 +209,35 @@ __global__ void __launch_bounds__(level_threads<T>())
   if ((int)threadIdx.x >= hx && (int)threadIdx.x < LEVEL_NBX - hx && B.ty >= hy && B.ty < rows - hy && ux < m.nbx &&
       uy < m.nby)
     level_store(B, x, xout, (size_t)B.ld * (grid.ny + 2));
+}
+
+template <typename T, typename S, bool NINE, bool FU, bool PER>
+__global__ void __launch_bounds__(level_threads<T>())
+    k_level_down(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* __restrict__ f,
+                 const T* __restrict__ xin, T* __restrict__ xout, T* __restrict__ fc, T* __restrict__ xc, int nu1,
+                 const int* done) {
+  down_body<T, S, NINE, FU, PER>(v, grid, ci, f, xin, xout, fc, xc, nu1, done);
+}
+
+template <typename T, typename S, bool NINE, bool FU, bool PER>
+__global__ void __launch_bounds__(level_threads<T>())
+    k_level_up(StencilView<T, S> v, LevelGrid grid, const T* __restrict__ ci, const T* ec, const T* __restrict__ f,
+               const T* __restrict__ xin, T* __restrict__ xout, int nu2, const int* done) {
+  up_body<T, S, NINE, FU, PER>(v, grid, ci, ec, f, xin, xout, nu2, done);
+}
+
+// One problem of a batched stage per blockIdx.z; the iterate goes x -> x2 -> x.
+template <typename T, typename S, bool NINE, bool FU>
+__global__ void __launch_bounds__(level_threads<T>()) k_level_down_b(const LevelDesc<T, S>* __restrict__ d, int nu1) {
+  const LevelDesc<T, S>& q = d[blockIdx.z];
+  down_body<T, S, NINE, FU, false>(q.v, LevelGrid{q.v.n, q.v.n, 0, 0}, q.ci, q.f, q.zero ? nullptr : q.x, q.x2, q.fc,
+                                   q.xc, nu1, q.done);
+}
+
+template <typename T, typename S, bool NINE, bool FU>
+__global__ void __launch_bounds__(level_threads<T>()) k_level_up_b(const LevelDesc<T, S>* __restrict__ d, int nu2) {
+  const LevelDesc<T, S>& q = d[blockIdx.z];
+  up_body<T, S, NINE, FU, false>(q.v, LevelGrid{q.v.n, q.v.n, 0, 0}, q.ci, q.xc, q.f, q.x2, q.x, nu2, q.done);
 }
 
 template <typename T>
@@ -287,11 +315,39 @@ void launch_level_up_p(const StencilView<double, double>& v, const LevelGrid& gr
   up<double, double, true>(v, grid, kind, ci, ec, f, xin, xout, nu2, rows, done, s);
 }
 
+template <typename T, typename S>
+void launch_level_down_b(const LevelDesc<T, S>* d, int count, int n, int kind, int nu1, int rows, cudaStream_t s,
+                         int fused) {
+  dim3 g = level_grid(LevelGrid{n, n, 0, 0}, rows, 2 * nu1 + 1, nu1 + 1);
+  g.z = count;
+  auto go = [&](auto kernel) { pdl_launch(kernel, g, dim3(LEVEL_NBX, rows), level_bytes<T>(rows), s, d, nu1); };
+  if (kind == 9)
+    fused ? go(k_level_down_b<T, S, true, true>) : go(k_level_down_b<T, S, true, false>);
+  else
+    fused ? go(k_level_down_b<T, S, false, true>) : go(k_level_down_b<T, S, false, false>);
+  count_launch();
+}
+
+template <typename T, typename S>
+void launch_level_up_b(const LevelDesc<T, S>* d, int count, int n, int kind, int nu2, int rows, cudaStream_t s,
+                       int fused) {
+  dim3 g = level_grid(LevelGrid{n, n, 0, 0}, rows, 2 * nu2, nu2);
+  g.z = count;
+  auto go = [&](auto kernel) { pdl_launch(kernel, g, dim3(LEVEL_NBX, rows), level_bytes<T>(rows), s, d, nu2); };
+  if (kind == 9)
+    fused ? go(k_level_up_b<T, S, true, true>) : go(k_level_up_b<T, S, true, false>);
+  else
+    fused ? go(k_level_up_b<T, S, false, true>) : go(k_level_up_b<T, S, false, false>);
+  count_launch();
+}
+
 #define BMG_INST(T, S)                                                                                               \
   template void launch_level_down<T, S>(const StencilView<T, S>&, int, const T*, const T*, const T*, T*, T*, T*, int, \
                                         int, const int*, cudaStream_t);                                              \
   template void launch_level_up<T, S>(const StencilView<T, S>&, int, const T*, const T*, const T*, const T*, T*,      \
-                                      int, int, const int*, cudaStream_t);
+                                      int, int, const int*, cudaStream_t);                                           \
+  template void launch_level_down_b<T, S>(const LevelDesc<T, S>*, int, int, int, int, int, cudaStream_t, int);        \
+  template void launch_level_up_b<T, S>(const LevelDesc<T, S>*, int, int, int, int, int, cudaStream_t, int);
 BMG_INST(double, double)
 BMG_INST(float, float)
 BMG_INST(float, __nv_bfloat16)

@@ -233,7 +233,8 @@ struct LevelDesc {
   const int* done;    // the problem's control flag
   const double* L;    // coarsest level: Cholesky factor and substitution workspace
   double* y;
-  T* x2 = nullptr;    // second iterate of a level swept by the one-pass kernels (else NULL)
+  T* x2 = nullptr;    // second iterate of a level swept by the one-pass kernels or run by halves (else NULL)
+  int zero = 0;       // 1: a coarse level of its problem, whose iterate is zero when the cycle comes down to it
 };
 
 // A problem's finest level, for the FP64 outer loop.
@@ -279,6 +280,14 @@ void launch_gs_pair_b(const LevelDesc<float, S>* d, int count, int n, int shape,
 // launch_gs_tile64, with the one-wave height taken over all `count` problems.
 void launch_gs_tile64_b(const LevelDesc<double, double>* d, int count, int n, int shape, int dir, cudaStream_t s,
                         int fused = 0);
+// Batched halves of the cycle (launch_level_down / _up over every problem of a
+// stage): down reads x (zero: nothing) and writes x2, up reads x2 and writes x.
+template <typename T, typename S>
+void launch_level_down_b(const LevelDesc<T, S>* d, int count, int n, int kind, int nu1, int rows, cudaStream_t s,
+                         int fused);
+template <typename T, typename S>
+void launch_level_up_b(const LevelDesc<T, S>* d, int count, int n, int kind, int nu2, int rows, cudaStream_t s,
+                       int fused);
 int strip_timeouts_b();
 template <typename T, typename S>
 void launch_coarse_b(const LevelDesc<T, S>* d, int count, cudaStream_t s);

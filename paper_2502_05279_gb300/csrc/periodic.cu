@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_update(PGeom g, dou
                                                                     double* __restrict__ z,
                                                                     double* __restrict__ partials, Ctl* ctl) {
   if (ctl->done) return;
-  const double alpha = rdiv(ctl->pr, ctl->pq);
+  const double alpha = ctl->alpha;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= g.ny; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= g.nx; i += dev::NORM_THREADS) {
