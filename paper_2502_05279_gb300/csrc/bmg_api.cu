@@ -2288,7 +2288,7 @@ void batch_iteration(bmg_batch* B) {
     launch_residual_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws, B->arith);
   } else {
     for (int c = 0; c < B->inner; ++c) batch_vcycle(B);
-    launch_ir_update_b(B->d_top, B->nprob, B->maxn, B->ws);
+    launch_ir_update_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws);
     launch_ir_residual_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws, B->arith);
   }
   launch_finalize_b(B->d_top, B->nprob, 1, B->ws);

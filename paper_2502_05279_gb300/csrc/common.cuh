@@ -156,7 +156,7 @@ struct Ctl {
   int done;
   int it;
   int maxit;
-  int pad;
+  unsigned ticket;       // blocks of the running reduction launch that have stored their partial sums
   double tol;
   double scale_next;     // power-of-two scale for the next FP32 residual
   double scale_applied;  // the scale the current FP32 residual carries

@@ -1487,14 +1487,39 @@ __device__ __forceinline__ double scale_of(double rho) {
   return ldexp(1.0, e);
 }
 
+// True in the last block of a launch to get here (every block calls it once,
+// after its thread 0 has stored its partial sums): that block sums the
+// partials, in the same order as a launch of one block would, and that launch
+// is saved.  Used by the periodic hierarchy, whose kernels are launched plainly
+// (three launches of an iteration, 17 us at 2048 x 2047); behind programmatic
+// launches the small launch costs no more than the tickets (84 us a cycle
+// either way at 127^2).  The ticket is left at zero.
+__device__ __forceinline__ bool last_block(unsigned* ticket, unsigned blocks) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == blocks - 1;
+    if (last) {
+      *ticket = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last != 0;
+}
+
+// (partials are read from L2, where the other blocks' stores are)
+__device__ __forceinline__ double reduce_partials(const double* partials, int np) {
+  double acc = 0.0;
+  for (int k = threadIdx.x; k < np; k += NORM_THREADS) acc = __dadd_rn(acc, __ldcg(partials + k));
+  return block_sum(acc);
+}
+
 // One block: sum the partials in index order per thread, fixed tree, sqrt;
 // record the norm in ctl (phase 0 = initial residual, 1 = after a cycle).
-__device__ __forceinline__ void finalize_body(const double* __restrict__ partials, int np, Ctl* ctl, int phase,
-                                              double* out) {
+__device__ __forceinline__ void finalize_body(const double* partials, int np, Ctl* ctl, int phase, double* out) {
   if (phase == 1 && ctl && ctl->done) return;
-  double acc = 0.0;
-  for (int k = threadIdx.x; k < np; k += NORM_THREADS) acc = __dadd_rn(acc, partials[k]);
-  double tot = block_sum(acc);
+  const double tot = reduce_partials(partials, np);
   if (threadIdx.x != 0) return;
   double rho = __dsqrt_rn(tot);
   if (out) *out = rho;
@@ -1513,6 +1538,28 @@ __device__ __forceinline__ void finalize_body(const double* __restrict__ partial
     else if (it >= ctl->maxit) ctl->done = 2;
   }
   ctl->scale_next = scale_of(rho);
+}
+
+// The scalars of a flexible-CG step from its partial sums, by one block: z.q and
+// beta = -(z.q) / (p.q)_prev after the first step; then p.q, p.r (the second
+// partial array NORM_BLOCKS_MAX entries after the first) and alpha.  One
+// division per step each.
+__device__ __forceinline__ void fcg_beta_body(const double* partials, int np, Ctl* ctl) {
+  const double v = reduce_partials(partials, np);
+  if (threadIdx.x == 0) {
+    ctl->zq = v;
+    if (!ctl->first) ctl->beta = -rdiv(v, ctl->pq_prev);
+  }
+}
+__device__ __forceinline__ void fcg_alpha_body(const double* partials, int np, Ctl* ctl) {
+  const double a = reduce_partials(partials, np);
+  __syncthreads();
+  const double b = reduce_partials(partials + NORM_BLOCKS_MAX, np);
+  if (threadIdx.x == 0) {
+    ctl->pq = a;
+    ctl->pr = b;
+    ctl->alpha = rdiv(b, a);
+  }
 }
 
 constexpr int COARSE_M_MAX = 225;   // coarsest level n <= 15

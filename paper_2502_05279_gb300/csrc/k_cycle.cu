@@ -740,33 +740,15 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_zq(int n, const double* __
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
 }
 
-__device__ __forceinline__ double reduce_partials(const double* partials, int np) {
-  double acc = 0.0;
-  for (int k = threadIdx.x; k < np; k += NORM_THREADS) acc = __dadd_rn(acc, partials[k]);
-  return block_sum(acc);
-}
-
 // slot 0: zq; slot 1: pq and pr (second partial array right after the first)
 __global__ void __launch_bounds__(NORM_THREADS) k_fcg_reduce(const double* __restrict__ partials, int np, Ctl* ctl,
                                                              int which) {
   pdl_enter();
   if (ctl->done) return;
-  if (which == 0) {
-    double v = reduce_partials(partials, np);
-    if (threadIdx.x == 0) {
-      ctl->zq = v;
-      if (!ctl->first) ctl->beta = -rdiv(v, ctl->pq_prev);   // one division per step, not per point
-    }
-  } else {
-    double a = reduce_partials(partials, np);
-    __syncthreads();
-    double b = reduce_partials(partials + NORM_BLOCKS_MAX, np);
-    if (threadIdx.x == 0) {
-      ctl->pq = a;
-      ctl->pr = b;
-      ctl->alpha = rdiv(b, a);   // one division per step, not per thread
-    }
-  }
+  if (which == 0)
+    fcg_beta_body(partials, np, ctl);
+  else
+    fcg_alpha_body(partials, np, ctl);
 }
 
 // FCG_COLS points of a row per thread, FBX apart, every load before the first store
@@ -960,11 +942,6 @@ static void fcg_step(const StencilView<double, double>& v, int kind, double* x, 
   pdl_launch(k_fcg_update<FU>, g, NORM_THREADS, 0, s, n, x, r, pv, q, r32, z32_zero, z_zero, partials, c);
   count_launch();
   if (mark) mark(mark_arg, 3);
-}
-
-void launch_fcg_reduce(const double* partials, int np, void* ctl, int which, cudaStream_t s) {
-  pdl_launch(k_fcg_reduce, 1, NORM_THREADS, 0, s, partials, np, (Ctl*)ctl, which);
-  count_launch();
 }
 
 void launch_fcg_step(const StencilView<double, double>& v, int kind, double* x, double* r, const double* z,

@@ -205,12 +205,6 @@ int launch_fcg_init(const StencilView<double, double>& v, int kind, const double
 void launch_fcg_step(const StencilView<double, double>& v, int kind, double* x, double* r, const double* z,
                      const float* z32, double* p, double* q, float* r32, float* z32_zero, double* z_zero,
                      double* partials, void* ctl, cudaStream_t s, void (*mark)(void*, int), void* mark_arg);
-// The step's scalar reductions over np partial sums in the canonical order:
-// which = 0: z.q into ctl (and beta = -(z.q) / (p.q)_prev after the first
-// step); which = 1: p.q and p.r (the second partial array NORM_BLOCKS_MAX
-// entries after the first).
-void launch_fcg_reduce(const double* partials, int np, void* ctl, int which, cudaStream_t s);
-
 // FP64 throughput probe.
 double measure_fp64_rate(cudaStream_t s);
 
@@ -295,7 +289,7 @@ void launch_coarse_b(const LevelDesc<T, S>* d, int count, cudaStream_t s);
 // min(n, 1024) canonical reduction blocks in turn.
 void launch_residual_b(const TopDesc* d, const int2* bmap, int nblocks, cudaStream_t s, int fused = 0);
 void launch_finalize_b(const TopDesc* d, int count, int phase, cudaStream_t s);
-void launch_ir_update_b(const TopDesc* d, int count, int maxn, cudaStream_t s);
+void launch_ir_update_b(const TopDesc* d, const int2* bmap, int nblocks, cudaStream_t s);
 void launch_ir_residual_b(const TopDesc* d, const int2* bmap, int nblocks, cudaStream_t s, int fused = 0);
 void launch_all_done(const char* ctls, size_t stride, int count, int* out, cudaStream_t s);
 template <typename T>

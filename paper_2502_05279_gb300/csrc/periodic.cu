@@ -519,7 +519,8 @@ template <bool NINE, bool FU>
 __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_residual(PGeom g, const double* __restrict__ st,
                                                                   const double* __restrict__ x,
                                                                   const double* __restrict__ f, double* __restrict__ r,
-                                                                  double* __restrict__ partials, const int* done) {
+                                                                  double* __restrict__ partials, const int* done,
+                                                                  Ctl* ctl, int phase) {
   if (dev::stopped(done)) return;
   const int b = blockIdx.x, G = gridDim.x;
   double acc = 0.0;
@@ -533,6 +534,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_residual(PGeom g, const
   if (partials) {
     const double tot = dev::block_sum(acc);
     if (threadIdx.x == 0) partials[b] = tot;
+    if (ctl && dev::last_block(&ctl->ticket, G)) dev::finalize_body(partials, G, ctl, phase, nullptr);
   }
 }
 
@@ -673,13 +675,14 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_init(PGeom g, const
     partials[blockIdx.x] = tot;
     if (blockIdx.x == 0) ctl->first = 1;
   }
+  if (dev::last_block(&ctl->ticket, gridDim.x)) dev::finalize_body(partials, gridDim.x, ctl, 0, nullptr);
 }
 
 // partial z.q
 template <bool FU>
 __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_zq(PGeom g, const double* __restrict__ z,
                                                                 const double* __restrict__ q,
-                                                                double* __restrict__ partials, const Ctl* ctl) {
+                                                                double* __restrict__ partials, Ctl* ctl) {
   if (ctl->done) return;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= g.ny; j += gridDim.x)
@@ -689,6 +692,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_zq(PGeom g, const d
     }
   const double tot = dev::block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
+  if (dev::last_block(&ctl->ticket, gridDim.x)) dev::fcg_beta_body(partials, gridDim.x, ctl);
 }
 
 // p = z (first step) or z + beta p
@@ -709,7 +713,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_matvec(PGeom g, con
                                                                     const double* __restrict__ pv,
                                                                     const double* __restrict__ r,
                                                                     double* __restrict__ q,
-                                                                    double* __restrict__ partials, const Ctl* ctl) {
+                                                                    double* __restrict__ partials, Ctl* ctl) {
   if (ctl->done) return;
   double apq = 0.0, apr = 0.0;
   for (int j = 1 + blockIdx.x; j <= g.ny; j += gridDim.x)
@@ -737,6 +741,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_matvec(PGeom g, con
     partials[blockIdx.x] = t1;
     partials[dev::NORM_BLOCKS_MAX + blockIdx.x] = t2;
   }
+  if (dev::last_block(&ctl->ticket, gridDim.x)) dev::fcg_alpha_body(partials, gridDim.x, ctl);
 }
 
 // x += alpha p, r -= alpha q (alpha = (p.r) / (p.q)), z = 0, partial r.r
@@ -768,6 +773,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_update(PGeom g, dou
       ctl->first = 0;
     }
   }
+  if (dev::last_block(&ctl->ticket, gridDim.x)) dev::finalize_body(partials, gridDim.x, ctl, 1, nullptr);
 }
 
 dim3 pgrid(int nx, int ny) { return dim3((unsigned)((nx + PBX - 1) / PBX), (unsigned)((ny + PBY - 1) / PBY)); }
@@ -1028,12 +1034,12 @@ double* per_sweep(const PerLevel& L, const double* f, double* x, double* home, c
 
 template <bool FU>
 int per_residual(const PerLevel& L, const double* x, const double* f, double* r, double* partials, const int* done,
-                 cudaStream_t s) {
+                 cudaStream_t s, Ctl* ctl = nullptr, int phase = 0) {
   const int G = L.g.ny < dev::NORM_BLOCKS_MAX ? L.g.ny : dev::NORM_BLOCKS_MAX;
   if (L.kind == 9)
-    k_p_residual<true, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, x, f, r, partials, done);
+    k_p_residual<true, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, x, f, r, partials, done, ctl, phase);
   else
-    k_p_residual<false, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, x, f, r, partials, done);
+    k_p_residual<false, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, x, f, r, partials, done, ctl, phase);
   count_launch();
   return G;
 }
@@ -1110,26 +1116,25 @@ void per_enqueue_initial(PerHier* P, const double* rhs, double* x, double* parti
                       : (L.kind == 9 ? k_p_fcg_init<true, false> : k_p_fcg_init<false, false>);
     k<<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, x, rhs, P->kr, P->kr + ps, partials, ctl);
     count_launch();
-    launch_norm_finalize(partials, G, ctl, 0, nullptr, s);
     return;
   }
-  const int G = P->fused ? per_residual<true>(P->lv[0], x, rhs, nullptr, partials, nullptr, s)
-                         : per_residual<false>(P->lv[0], x, rhs, nullptr, partials, nullptr, s);
-  launch_norm_finalize(partials, G, ctl, 0, nullptr, s);
+  if (P->fused)
+    per_residual<true>(P->lv[0], x, rhs, nullptr, partials, nullptr, s, ctl, 0);
+  else
+    per_residual<false>(P->lv[0], x, rhs, nullptr, partials, nullptr, s, ctl, 0);
 }
 
 namespace {
 // One FCG step after the preconditioner z = V(r): z.q and beta, p, q = A p with
 // p.q and p.r, then the x / r update with the r.r partial sums; returns G.
 template <bool FU>
-int per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t s, bool zero_z) {
+void per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t s, bool zero_z) {
   const PerLevel& L = P->lv[0];
   const size_t ps = L.g.ps();
   double *r = P->kr, *z = P->kr + ps, *pv = P->kr + 2 * ps, *q = P->kr + 3 * ps;
   const int G = L.g.ny < dev::NORM_BLOCKS_MAX ? L.g.ny : dev::NORM_BLOCKS_MAX;
   k_p_fcg_zq<FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, z, q, partials, ctl);
   count_launch();
-  launch_fcg_reduce(partials, G, ctl, 0, s);
   k_p_fcg_direction<FU><<<pgrid(L.g.nx, L.g.ny), dim3(PBX, PBY), 0, s>>>(L.g, z, pv, ctl);
   count_launch();
   if (L.kind == 9)
@@ -1137,17 +1142,14 @@ int per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_t
   else
     k_p_fcg_matvec<false, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, pv, r, q, partials, ctl);
   count_launch();
-  launch_fcg_reduce(partials, G, ctl, 1, s);
   k_p_fcg_update<FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, x, r, pv, q, zero_z ? z : nullptr, partials, ctl);
   count_launch();
-  return G;
 }
 }  // namespace
 
 void per_enqueue_iteration(PerHier* P, const double* rhs, double* x, double* partials, Ctl* ctl, cudaStream_t s,
                            const PerMarks* mk) {
   const int* done = &ctl->done;
-  int G;
   if (P->krylov) {
     // z = V(r) from z = 0 (zeroed by the previous update or the initial step), then the FCG step
     const size_t ps = P->lv[0].g.ps();
@@ -1158,19 +1160,21 @@ void per_enqueue_iteration(PerHier* P, const double* rhs, double* x, double* par
       per_vcycle<false>(P, 0, z, r, done, s, mk, true);
     Bracket b(mk, 0, BMG_K_FCG);
     const bool zero_z = !per_zero_aware(P, 0, mk);
-    G = P->fused ? per_fcg_step<true>(P, x, partials, ctl, s, zero_z)
-                 : per_fcg_step<false>(P, x, partials, ctl, s, zero_z);
+    if (P->fused)
+      per_fcg_step<true>(P, x, partials, ctl, s, zero_z);
+    else
+      per_fcg_step<false>(P, x, partials, ctl, s, zero_z);
   } else {
     if (P->fused)
       per_vcycle<true>(P, 0, x, rhs, done, s, mk, false);
     else
       per_vcycle<false>(P, 0, x, rhs, done, s, mk, false);
     Bracket b(mk, 0, BMG_K_NORM);
-    G = P->fused ? per_residual<true>(P->lv[0], x, rhs, nullptr, partials, done, s)
-                 : per_residual<false>(P->lv[0], x, rhs, nullptr, partials, done, s);
+    if (P->fused)
+      per_residual<true>(P->lv[0], x, rhs, nullptr, partials, done, s, ctl, 1);
+    else
+      per_residual<false>(P->lv[0], x, rhs, nullptr, partials, done, s, ctl, 1);
   }
-  Bracket b(mk, 0, BMG_K_FINALIZE);
-  launch_norm_finalize(partials, G, ctl, 1, nullptr, s);
 }
 
 int per_num_levels(const PerHier* P) { return (int)P->lv.size(); }
