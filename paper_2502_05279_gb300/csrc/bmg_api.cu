@@ -1046,7 +1046,9 @@ int autotune_solo(bmg_hierarchy* h) {
 // that also forms the residual and restricts it (temporal blocking) against
 // the two-sweep pass plus the separate residual + restriction, timed on
 // scratch iterates with the level's stencil; the coarse level's right-hand
-// side and iterate are written by both (they are rewritten every cycle).
+// side and iterate are written by both (they are rewritten every cycle). FP32
+// points, fused pass against the two: 842 / 907 us at 8191^2, 212 / 253 at
+// 4095^2, 66 / 84 at 2047^2.
 template <typename S>
 int tune_pair_restrict(Level& L, Level& C, const StencilView<float, S>& v, cudaStream_t s) {
   const std::string fkey = tune_key("pair_restrict", {v.n, (int)sizeof(S), v.fused, L.pair32});
