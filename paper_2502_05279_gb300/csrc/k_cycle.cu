@@ -703,8 +703,24 @@ namespace {
 
 constexpr int FBX = 32, FBY = 8;
 
-__device__ __forceinline__ double zval(const double* z, const float* z32, double s, size_t p) {
-  return z32 ? pow2_times_widened(s, z32[p]) : z[p];   // s * fl64(z32) is exact: s is a power of two
+// The preconditioned residual as stored: FP64, or FP32 (MIXED) with the cycle's
+// power-of-two scale, widened only after all of a thread's loads are issued (the
+// widening branches on the value: done as each was loaded it left one load of a
+// thread in flight, and z.q at 4095^2 took 97 us for 200 MB instead of 38, z + beta p
+// 79 instead of 44).
+template <bool MIXED>
+struct ZRaw { double v; };
+template <>
+struct ZRaw<true> { float v; };
+template <bool MIXED>
+__device__ __forceinline__ void zload(ZRaw<MIXED>& q, const double* z, const float* z32, size_t p) {
+  if constexpr (MIXED) q.v = z32[p];
+  else q.v = z[p];
+}
+template <bool MIXED>
+__device__ __forceinline__ double zvalue(const ZRaw<MIXED>& q, double s) {
+  if constexpr (MIXED) return pow2_times_widened(s, q.v);   // s * fl64(z32) is exact: s is a power of two
+  else return q.v;
 }
 
 // FCG_COLS columns of a row per thread iteration (NORM_THREADS apart): their
@@ -712,29 +728,34 @@ __device__ __forceinline__ double zval(const double* z, const float* z32, double
 // the canonical order.
 constexpr int FCG_COLS = 4;
 
-template <bool FU>
-__global__ void __launch_bounds__(NORM_THREADS) k_fcg_zq(int n, const double* __restrict__ z,
+// Every block of the grid resident at once (seven to an SM, 32 registers, so two
+// FP64 columns in flight): at six the last 112 blocks ran alone, most SMs idle
+// (8191^2 FP64: 230 us, now 173 for 1.07 GB).
+template <bool FU, bool MIXED>
+__global__ void __launch_bounds__(NORM_THREADS, 8) k_fcg_zq(int n, const double* __restrict__ z,
                                                          const float* __restrict__ z32, const double* __restrict__ q,
                                                          double* __restrict__ partials, const Ctl* ctl) {
   pdl_enter();
   if (ctl->done) return;
   const double s = ctl->scale_applied;
+  constexpr int COLS = MIXED ? FCG_COLS : 2;
   const int ld = n + 2;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
-    for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS * FCG_COLS) {
-      double zv[FCG_COLS], qv[FCG_COLS];
+    for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS * COLS) {
+      ZRaw<MIXED> zv[COLS];
+      double qv[COLS];
 #pragma unroll
-      for (int c = 0; c < FCG_COLS; ++c) {
+      for (int c = 0; c < COLS; ++c) {
         const size_t p = (size_t)j * ld + i + c * NORM_THREADS;
         if (i + c * NORM_THREADS <= n) {
-          zv[c] = zval(z, z32, s, p);
+          zload(zv[c], z, z32, p);
           qv[c] = q[p];
         }
       }
 #pragma unroll
-      for (int c = 0; c < FCG_COLS; ++c)
-        if (i + c * NORM_THREADS <= n) acc = madd<FU>(acc, zv[c], qv[c]);
+      for (int c = 0; c < COLS; ++c)
+        if (i + c * NORM_THREADS <= n) acc = madd<FU>(acc, zvalue(zv[c], s), qv[c]);
     }
   double tot = block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
@@ -752,7 +773,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_reduce(const double* __res
 }
 
 // FCG_COLS points of a row per thread, FBX apart, every load before the first store
-template <bool FU>
+template <bool FU, bool MIXED>
 __global__ void k_fcg_direction(int n, const double* __restrict__ z, const float* __restrict__ z32,
                                 double* __restrict__ pv, const Ctl* ctl) {
   pdl_enter();
@@ -761,29 +782,36 @@ __global__ void k_fcg_direction(int n, const double* __restrict__ z, const float
   if (j > n) return;
   const double s = ctl->scale_applied, beta = ctl->beta;
   const bool first = ctl->first;
-  double zp[FCG_COLS], pp[FCG_COLS];
+  ZRaw<MIXED> zp[FCG_COLS];
+  double pp[FCG_COLS];
 #pragma unroll
   for (int c = 0; c < FCG_COLS; ++c) {
     const size_t p = (size_t)j * (n + 2) + i0 + c * FBX;
     if (i0 + c * FBX <= n) {
-      zp[c] = zval(z, z32, s, p);
+      zload(zp[c], z, z32, p);
       pp[c] = first ? 0.0 : pv[p];
     }
   }
 #pragma unroll
   for (int c = 0; c < FCG_COLS; ++c) {
     const size_t p = (size_t)j * (n + 2) + i0 + c * FBX;
-    if (i0 + c * FBX <= n && BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * (n + 2)))
-      pv[p] = first ? zp[c] : madd<FU>(zp[c], beta, pp[c]);
+    if (i0 + c * FBX <= n && BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * (n + 2))) {
+      const double zc = zvalue(zp[c], s);
+      pv[p] = first ? zc : madd<FU>(zc, beta, pp[c]);
+    }
   }
 }
 
-// q = A p (row sum a_O p + a_W p_W + ... in canonical order), partial p.q and p.r
-template <bool FU>
-__global__ void __launch_bounds__(NORM_THREADS) k_fcg_matvec(StencilView<double, double> v, int nine,
-                                                             const double* __restrict__ pv, const double* __restrict__ r,
-                                                             double* __restrict__ q, double* __restrict__ partials,
-                                                             const Ctl* ctl) {
+// q = A p (row sum a_O p + a_W p_W + ... in canonical order), partial p.q and p.r.
+// Bound by its eleven FP64 operations a point (298 us at 4095^2). The partial sums
+// tie the grid to 1024 blocks, seven to an SM: four resident (64 registers) run
+// them as four and three; three (79 registers, unbounded) left the seventh alone
+// on its SM, too few warps to hide its loads (377 us at 4095^2, now 338).
+template <bool NINE, bool FU>
+__global__ void __launch_bounds__(NORM_THREADS, 4) k_fcg_matvec(StencilView<double, double> v,
+                                                                const double* __restrict__ pv,
+                                                                const double* __restrict__ r, double* __restrict__ q,
+                                                                double* __restrict__ partials, const Ctl* ctl) {
   pdl_enter();
   if (ctl->done) return;
   const int n = v.n, ld = v.ld;
@@ -796,7 +824,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_matvec(StencilView<double,
       acc = madd<FU>(acc, v.W[p + 1], pv[p + 1]);
       acc = madd<FU>(acc, v.S_[p], pv[p - ld]);
       acc = madd<FU>(acc, v.S_[p + ld], pv[p + ld]);
-      if (nine) {
+      if constexpr (NINE) {
         acc = madd<FU>(acc, v.SW[p], pv[p - ld - 1]);
         acc = madd<FU>(acc, v.SW[p + ld + 1], pv[p + ld + 1]);
         acc = madd<FU>(acc, v.NW[p], pv[p + ld - 1]);
@@ -817,19 +845,21 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_matvec(StencilView<double,
 
 // x += alpha p, r -= alpha q, partial r.r; zero the preconditioner's output z or
 // z32 (NULL: its cycle starts from zero without reading it) and, in mixed
-// precision, write r32 = fl32(r / scale_next).
-template <bool FU>
-__global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __restrict__ x, double* __restrict__ r,
-                                                             const double* __restrict__ pv,
-                                                             const double* __restrict__ q, float* __restrict__ r32,
-                                                             float* __restrict__ z32, double* __restrict__ z,
-                                                             double* __restrict__ partials, Ctl* ctl) {
+// precision (MIXED), write r32 = fl32(r / scale_next), narrowed before it is
+// scaled (the FP64 product and its conversion were half the update's FP64 work):
+// 4095^2 mixed 171 -> 148 us for 0.87 GB, 8191^2 FP64 504 -> 490 for 3.2 GB.
+template <bool FU, bool MIXED>
+__global__ void __launch_bounds__(NORM_THREADS, 4) k_fcg_update(int n, double* __restrict__ x, double* __restrict__ r,
+                                                                const double* __restrict__ pv,
+                                                                const double* __restrict__ q, float* __restrict__ r32,
+                                                                float* __restrict__ z32, double* __restrict__ z,
+                                                                double* __restrict__ partials, Ctl* ctl) {
   pdl_enter();
   if (ctl->done) return;
   const int ld = n + 2;
   const double alpha = ctl->alpha;
-  const double s = ctl->scale_next;
-  const double inv = pow2_inverse(s);
+  const double inv = MIXED ? pow2_inverse(ctl->scale_next) : 1.0;
+  const float inv32 = MIXED ? narrow_scale32(inv) : 1.0f;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS * FCG_COLS) {
@@ -851,9 +881,12 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __re
         x[p] = madd<FU>(xv[c], alpha, pw[c]);
         const double rr = msub<FU>(rv[c], alpha, qv[c]);
         r[p] = rr;
-        if (r32) r32[p] = __double2float_rn(rmul(rr, inv));
-        if (z32) z32[p] = 0.0f;
-        if (z) z[p] = 0.0;
+        if constexpr (MIXED) {
+          r32[p] = narrow_scaled(rr, inv, inv32);
+          if (z32) z32[p] = 0.0f;
+        } else {
+          if (z) z[p] = 0.0;
+        }
         acc = madd<FU>(acc, rr, rr);
       }
     }
@@ -861,7 +894,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_update(int n, double* __re
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = tot;
     if (blockIdx.x == 0) {
-      ctl->scale_applied = s;
+      ctl->scale_applied = ctl->scale_next;
       ctl->pq_prev = ctl->pq;
       ctl->first = 0;
     }
@@ -879,6 +912,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
   const int n = v.n, ld = v.ld;
   const double s = ctl->scale_next;
   const double inv = pow2_inverse(s);
+  const float inv32 = narrow_scale32(inv);
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS) {
@@ -887,7 +921,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
                        : row_residual<double, double, false, true, FU>(v, x, p, f[p]);
       if (!BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * ld)) continue;
       r[p] = rr;
-      if (r32) r32[p] = __double2float_rn(rmul(rr, inv));
+      if (r32) r32[p] = narrow_scaled(rr, inv, inv32);
       if (z32) z32[p] = 0.0f;
       if (z) z[p] = 0.0;
       acc = madd<FU>(acc, rr, rr);
@@ -926,20 +960,23 @@ static void fcg_step(const StencilView<double, double>& v, int kind, double* x, 
   int g = norm_blocks(n);
   Ctl* c = (Ctl*)ctl;
   if (mark) mark(mark_arg, 0);
-  pdl_launch(k_fcg_zq<FU>, g, NORM_THREADS, 0, s, n, z, z32, q, partials, c);
+  pdl_launch(z32 ? k_fcg_zq<FU, true> : k_fcg_zq<FU, false>, g, NORM_THREADS, 0, s, n, z, z32, q, partials, c);
   count_launch();
   pdl_launch(k_fcg_reduce, 1, NORM_THREADS, 0, s, partials, g, c, 0);
   count_launch();
-  pdl_launch(k_fcg_direction<FU>, dim3((n + FBX * FCG_COLS - 1) / (FBX * FCG_COLS), (n + FBY - 1) / FBY),
+  pdl_launch(z32 ? k_fcg_direction<FU, true> : k_fcg_direction<FU, false>,
+             dim3((n + FBX * FCG_COLS - 1) / (FBX * FCG_COLS), (n + FBY - 1) / FBY),
              dim3(FBX, FBY), 0, s, n, z, z32, pv, c);
   count_launch();
   if (mark) mark(mark_arg, 1);
-  pdl_launch(k_fcg_matvec<FU>, g, NORM_THREADS, 0, s, v, kind == 9, pv, r, q, partials, c);
+  pdl_launch(kind == 9 ? k_fcg_matvec<true, FU> : k_fcg_matvec<false, FU>, g, NORM_THREADS, 0, s, v, pv, r, q,
+             partials, c);
   count_launch();
   pdl_launch(k_fcg_reduce, 1, NORM_THREADS, 0, s, partials, g, c, 1);
   count_launch();
   if (mark) mark(mark_arg, 2);
-  pdl_launch(k_fcg_update<FU>, g, NORM_THREADS, 0, s, n, x, r, pv, q, r32, z32_zero, z_zero, partials, c);
+  pdl_launch(r32 ? k_fcg_update<FU, true> : k_fcg_update<FU, false>, g, NORM_THREADS, 0, s, n, x, r, pv, q, r32,
+             z32_zero, z_zero, partials, c);
   count_launch();
   if (mark) mark(mark_arg, 3);
 }

@@ -695,15 +695,32 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_zq(PGeom g, const d
   if (dev::last_block(&ctl->ticket, gridDim.x)) dev::fcg_beta_body(partials, gridDim.x, ctl);
 }
 
-// p = z (first step) or z + beta p
+// Columns of a row per thread, every load before the first store (direction and
+// update, bound by memory: 16 and 38 us at 2048 x 2047).
+constexpr int P_FCG_COLS = 4;
+
+// p = z (first step) or z + beta p, columns PBX apart
 template <bool FU>
 __global__ void k_p_fcg_direction(PGeom g, const double* __restrict__ z, double* __restrict__ pv, const Ctl* ctl) {
   if (ctl->done) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + 1, j = blockIdx.y * blockDim.y + threadIdx.y + 1;
-  if (i > g.nx || j > g.ny) return;
-  const size_t p = (size_t)j * (g.nx + 2) + i;
-  if (!BMG_IN(DBG_PERIODIC, p, g.ps())) return;
-  pv[p] = ctl->first ? z[p] : madd<FU>(z[p], ctl->beta, pv[p]);
+  const int i0 = blockIdx.x * (PBX * P_FCG_COLS) + threadIdx.x + 1, j = blockIdx.y * blockDim.y + threadIdx.y + 1;
+  if (j > g.ny) return;
+  const bool first = ctl->first;
+  const double beta = ctl->beta;
+  double zv[P_FCG_COLS], pw[P_FCG_COLS];
+#pragma unroll
+  for (int c = 0; c < P_FCG_COLS; ++c) {
+    const size_t p = (size_t)j * (g.nx + 2) + i0 + c * PBX;
+    if (i0 + c * PBX <= g.nx) {
+      zv[c] = z[p];
+      pw[c] = first ? 0.0 : pv[p];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < P_FCG_COLS; ++c) {
+    const size_t p = (size_t)j * (g.nx + 2) + i0 + c * PBX;
+    if (i0 + c * PBX <= g.nx && BMG_IN(DBG_PERIODIC, p, g.ps())) pv[p] = first ? zv[c] : madd<FU>(zv[c], beta, pw[c]);
+  }
 }
 
 // q = A p (a_O p first, then the neighbours in the canonical order, wrapped),
@@ -746,7 +763,7 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_matvec(PGeom g, con
 
 // x += alpha p, r -= alpha q (alpha = (p.r) / (p.q)), z = 0, partial r.r
 template <bool FU>
-__global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_update(PGeom g, double* __restrict__ x,
+__global__ void __launch_bounds__(dev::NORM_THREADS, 4) k_p_fcg_update(PGeom g, double* __restrict__ x,
                                                                     double* __restrict__ r,
                                                                     const double* __restrict__ pv,
                                                                     const double* __restrict__ q,
@@ -756,14 +773,28 @@ __global__ void __launch_bounds__(dev::NORM_THREADS) k_p_fcg_update(PGeom g, dou
   const double alpha = ctl->alpha;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= g.ny; j += gridDim.x)
-    for (int i = 1 + threadIdx.x; i <= g.nx; i += dev::NORM_THREADS) {
-      const size_t p = (size_t)j * (g.nx + 2) + i;
-      if (!BMG_IN(DBG_PERIODIC, p, g.ps())) continue;
-      x[p] = madd<FU>(x[p], alpha, pv[p]);
-      const double rr = msub<FU>(r[p], alpha, q[p]);
-      r[p] = rr;
-      if (z) z[p] = 0.0;
-      acc = madd<FU>(acc, rr, rr);
+    for (int i = 1 + threadIdx.x; i <= g.nx; i += dev::NORM_THREADS * P_FCG_COLS) {
+      double xv[P_FCG_COLS], rv[P_FCG_COLS], pw[P_FCG_COLS], qv[P_FCG_COLS];
+#pragma unroll
+      for (int c = 0; c < P_FCG_COLS; ++c) {
+        const size_t p = (size_t)j * (g.nx + 2) + i + c * dev::NORM_THREADS;
+        if (i + c * dev::NORM_THREADS <= g.nx) {
+          xv[c] = x[p];
+          rv[c] = r[p];
+          pw[c] = pv[p];
+          qv[c] = q[p];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < P_FCG_COLS; ++c) {
+        const size_t p = (size_t)j * (g.nx + 2) + i + c * dev::NORM_THREADS;
+        if (i + c * dev::NORM_THREADS > g.nx || !BMG_IN(DBG_PERIODIC, p, g.ps())) continue;
+        x[p] = madd<FU>(xv[c], alpha, pw[c]);
+        const double rr = msub<FU>(rv[c], alpha, qv[c]);
+        r[p] = rr;
+        if (z) z[p] = 0.0;
+        acc = madd<FU>(acc, rr, rr);
+      }
     }
   const double tot = dev::block_sum(acc);
   if (threadIdx.x == 0) {
@@ -1135,7 +1166,7 @@ void per_fcg_step(PerHier* P, double* x, double* partials, Ctl* ctl, cudaStream_
   const int G = L.g.ny < dev::NORM_BLOCKS_MAX ? L.g.ny : dev::NORM_BLOCKS_MAX;
   k_p_fcg_zq<FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, z, q, partials, ctl);
   count_launch();
-  k_p_fcg_direction<FU><<<pgrid(L.g.nx, L.g.ny), dim3(PBX, PBY), 0, s>>>(L.g, z, pv, ctl);
+  k_p_fcg_direction<FU><<<pgrid((L.g.nx + P_FCG_COLS - 1) / P_FCG_COLS, L.g.ny), dim3(PBX, PBY), 0, s>>>(L.g, z, pv, ctl);
   count_launch();
   if (L.kind == 9)
     k_p_fcg_matvec<true, FU><<<G, dev::NORM_THREADS, 0, s>>>(L.g, L.st, pv, r, q, partials, ctl);
