@@ -1609,13 +1609,14 @@ __device__ __forceinline__ double pow2_times_widened(double s, float e) {
 }
 
 // fl32(r * inv) for inv a power of two (the scaled FP32 residual of the
-// refinement).  Narrowed first and scaled in FP32, it is the same number
-// whenever fl32(r) and the scaled value lie in [2^-125, 2^127]: both r and
-// r * inv are then in normal binades, where rounding to 24 bits commutes with
-// scaling by a power of two, and the FP32 product is exact.  Everything else
-// (tiny, huge, non-finite values, or a scale outside the FP32 range, signalled
-// by inv32 = 0) takes the FP64 product; this spares the FP64 pipe one multiply
-// per point on the FP64-bound outer residual.
+// refinement), from the bit fields: r's exponent re-biased and raised by
+// log2(inv), its mantissa rounded to 23 bits, to nearest even, with an integer
+// add whose carry runs into the exponent. The product is exact, so this is the
+// same number whenever it is a normal float; zero is itself, and everything else
+// (tiny, huge, non-finite values, or an inv that is not a normal power of two,
+// signalled by NARROW_NEVER) takes the FP64 product. Both FP64 operations of the
+// general route, product and conversion, are spared on the FP64-bound outer
+// residual, which has ten others a point.
 static __device__ __noinline__ float narrow_scaled_slow(double r, double inv) {
   return __double2float_rn(rmul(r, inv));
 }
@@ -1630,19 +1631,26 @@ __device__ __forceinline__ double pow2_inverse(double s) {
   return rdiv(1.0, s);
 }
 
-// (on the bit pattern: inv is a power of two, or takes the FP64 product)
-__device__ __forceinline__ float narrow_scale32(double inv) {
-  const unsigned hi = (unsigned)__double2hiint(inv);
-  const int e = (int)(hi >> 20) - 1023;
-  return (hi & 0xfffffu) == 0 && __double2loint(inv) == 0 && e >= -125 && e <= 125 ? __uint_as_float((unsigned)(e + 127) << 23)
-                                                                                 : 0.0f;
+constexpr int NARROW_NEVER = -65536;
+
+// log2(inv) as the change of biased exponent from double to float. Kept to
+// [-1793, 0], where no subnormal, infinite or NaN r gets a normal float's exponent.
+__device__ __forceinline__ int narrow_bias(double inv) {
+  const unsigned hi = (unsigned)__double2hiint(inv), e = hi >> 20;
+  const int bias = (int)e - 1023 - 896;
+  return e - 1u < 2046u && (hi & 0xfffffu) == 0 && __double2loint(inv) == 0 && bias <= 0 && bias >= -1793 ? bias
+                                                                                                      : NARROW_NEVER;
 }
 
-__device__ __forceinline__ float narrow_scaled(double r, double inv, float inv32) {
-  const float a = __double2float_rn(r);
-  const float b = __fmul_rn(a, inv32);
-  const float ma = fabsf(a), mb = fabsf(b);
-  if (ma >= 0x1p-125f && ma <= 0x1p127f && mb >= 0x1p-125f && mb <= 0x1p127f) return b;
+__device__ __forceinline__ float narrow_scaled(double r, double inv, int bias) {
+  const unsigned hi = (unsigned)__double2hiint(r), lo = (unsigned)__double2loint(r);
+  const int ef = (int)((hi >> 20) & 0x7ffu) + bias;   // the float's biased exponent, before rounding
+  if (ef >= 1 && ef <= 253) {
+    const unsigned up = lo + 0x0fffffffu + ((lo >> 29) & 1u);
+    const unsigned m = ((unsigned)ef << 20 | (hi & 0xfffffu)) + (up < lo ? 1u : 0u);
+    return __uint_as_float((hi & 0x80000000u) | __funnelshift_l(up, m, 3));
+  }
+  if (((hi << 1) | lo) == 0) return __uint_as_float(hi);   // +-0 (inv is positive and finite)
   return narrow_scaled_slow(r, inv);
 }
 
@@ -1683,7 +1691,7 @@ __device__ __forceinline__ void ir_residual_body(const StencilView<double, doubl
   const int n = v.n, ld = v.ld;
   const double s = ctl->scale_next;
   const double inv = pow2_inverse(s);
-  const float inv32 = narrow_scale32(inv);
+  const int bias = narrow_bias(inv);
   double acc = 0.0;
   for (int j = 1 + b; j <= n; j += G)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS) {
@@ -1691,7 +1699,7 @@ __device__ __forceinline__ void ir_residual_body(const StencilView<double, doubl
       double rr = nine ? row_residual<double, double, true, true, FU>(v, x, p, f[p])
                        : row_residual<double, double, false, true, FU>(v, x, p, f[p]);
       if (BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * ld)) {
-        r32[p] = narrow_scaled(rr, inv, inv32);
+        r32[p] = narrow_scaled(rr, inv, bias);
         if (e32) e32[p] = 0.0f;
       }
       acc = madd<FU>(acc, rr, rr);

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_ir_update_b(const TopDesc* __r
 }
 
 template <bool FU>
-__global__ void __launch_bounds__(NORM_THREADS) k_ir_residual_b(const TopDesc* __restrict__ d,
+__global__ void __launch_bounds__(NORM_THREADS, 6) k_ir_residual_b(const TopDesc* __restrict__ d,
                                                                 const int2* __restrict__ bmap) {
   pdl_enter();
   const int2 m = bmap[blockIdx.x];

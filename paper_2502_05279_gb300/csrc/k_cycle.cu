@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(NORM_THREADS, 4) k_fcg_update(int n, double* _
   const int ld = n + 2;
   const double alpha = ctl->alpha;
   const double inv = MIXED ? pow2_inverse(ctl->scale_next) : 1.0;
-  const float inv32 = MIXED ? narrow_scale32(inv) : 1.0f;
+  const int bias = MIXED ? narrow_bias(inv) : 0;
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS * FCG_COLS) {
@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(NORM_THREADS, 4) k_fcg_update(int n, double* _
         const double rr = msub<FU>(rv[c], alpha, qv[c]);
         r[p] = rr;
         if constexpr (MIXED) {
-          r32[p] = narrow_scaled(rr, inv, inv32);
+          r32[p] = narrow_scaled(rr, inv, bias);
           if (z32) z32[p] = 0.0f;
         } else {
           if (z) z[p] = 0.0;
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
   const int n = v.n, ld = v.ld;
   const double s = ctl->scale_next;
   const double inv = pow2_inverse(s);
-  const float inv32 = narrow_scale32(inv);
+  const int bias = narrow_bias(inv);
   double acc = 0.0;
   for (int j = 1 + blockIdx.x; j <= n; j += gridDim.x)
     for (int i = 1 + threadIdx.x; i <= n; i += NORM_THREADS) {
@@ -921,7 +921,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_fcg_init(StencilView<double, d
                        : row_residual<double, double, false, true, FU>(v, x, p, f[p]);
       if (!BMG_IN(DBG_REFINE_STORE, p, (size_t)(n + 2) * ld)) continue;
       r[p] = rr;
-      if (r32) r32[p] = narrow_scaled(rr, inv, inv32);
+      if (r32) r32[p] = narrow_scaled(rr, inv, bias);
       if (z32) z32[p] = 0.0f;
       if (z) z[p] = 0.0;
       acc = madd<FU>(acc, rr, rr);
