@@ -2002,6 +2002,7 @@ struct bmg_batch {
   int nprob = 0, precision = BMG_FP64, nu1 = 2, nu2 = 1, inner = 1, use_graph = 1, arith = BMG_ARITH_ROUNDED;
   int smoother = BMG_SMOOTHER_AUTO;
   int rhs_block = BMG_RHS_BLOCK_AUTO;
+  int fuse_restrict = BMG_FUSE_AUTO;
   std::vector<bmg_hierarchy*> hs;
   cudaStream_t user = nullptr, ws = nullptr;
   cudaEvent_t ev = nullptr;
@@ -2012,6 +2013,8 @@ struct bmg_batch {
     int multi = 0;              // 2 or 4: one-pass sweeps with that many members per warp (shared operator)
     int dir = 0;                // while a cycle is enqueued: 0 = iterate in x, 1 = in x2
     int rows = 0;               // > 0: the stage runs by halves of the cycle, tiles of this many block rows
+    int pair_rr = 0;            // 1: pre-smoothing, residual and restriction in one pass
+    int tops = 0;               // members that are their problem's level 0
     size_t elem = 0;
     void* d = nullptr;
     std::vector<char> host;
@@ -2097,7 +2100,7 @@ int build_batch_tables(bmg_batch* B, const double* const* rhs, double* const* x)
   for (auto& st : B->stages)
     for (auto& g : st) {
       g.host.clear();
-      if (!rhs) g.count = 0;
+      if (!rhs) g.count = g.tops = 0;
     }
   for (auto& t : B->tail_host) t.clear();
   if (!rhs) std::fill(B->tail_count.begin(), B->tail_count.end(), 0);
@@ -2130,6 +2133,7 @@ int build_batch_tables(bmg_batch* B, const double* const* rhs, double* const* x)
       g.kind = lv.kind;
       if (!rhs) {
         ++g.count;
+        g.tops += l == 0;
         g.elem = storage == 0 ? sizeof(LevelDesc<double, double>)
                               : storage == 1 ? sizeof(LevelDesc<float, float>) : sizeof(LevelDesc<float, __nv_bfloat16>);
         continue;
@@ -2219,6 +2223,16 @@ void group_restrict(bmg_batch* B, bmg_batch::Group& g) {
     launch_resid_restrict_b(gdesc<float, __nv_bfloat16>(g), g.count, g.n, g.kind, B->ws, g.dir, B->arith);
 }
 
+// Pre-smoothing and restriction of a group in one pass; zero: every member's
+// iterate is zero.
+void group_pair_restrict(bmg_batch* B, bmg_batch::Group& g, bool zero) {
+  if (g.storage == 1)
+    launch_gs_pair_restrict_b(gdesc<float, float>(g), g.count, g.n, g.dir, zero, B->ws, B->arith);
+  else
+    launch_gs_pair_restrict_b(gdesc<float, __nv_bfloat16>(g), g.count, g.n, g.dir, zero, B->ws, B->arith);
+  g.dir ^= 1;
+}
+
 // x (or x2) += P e: reads the array g.dir names and writes the one from which
 // the post-smoothing launches end in x.
 void group_interp(bmg_batch* B, bmg_batch::Group& g) {
@@ -2251,13 +2265,18 @@ void group_half(bmg_batch* B, bmg_batch::Group& g, bool up) {
 }
 
 // One V(nu1, nu2) cycle of every problem: down the stages (largest first), the
-// coarsest solves, back up.
-void batch_vcycle(bmg_batch* B) {
+// coarsest solves, back up. zero: the problems' level-0 iterates are zero (the
+// first cycle on a refinement step's residual equation).
+void batch_vcycle(bmg_batch* B, bool zero) {
   for (int b = B->bmax; b >= 1; --b) {
     for (auto& g : B->stages[b]) {
       g.dir = 0;
       if (g.count && g.rows > 0) {
         group_half(B, g, false);
+        continue;
+      }
+      if (g.count && g.pair_rr) {
+        group_pair_restrict(B, g, zero || g.tops == 0);
         continue;
       }
       group_relax(B, g, B->nu1);
@@ -2286,10 +2305,10 @@ void batch_vcycle(bmg_batch* B) {
 
 void batch_iteration(bmg_batch* B) {
   if (B->precision == BMG_FP64) {
-    batch_vcycle(B);
+    batch_vcycle(B, false);
     launch_residual_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws, B->arith);
   } else {
-    for (int c = 0; c < B->inner; ++c) batch_vcycle(B);
+    for (int c = 0; c < B->inner; ++c) batch_vcycle(B, c == 0);
     launch_ir_update_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws);
     launch_ir_residual_b(B->d_top, B->d_bmap, (int)B->bmap.size(), B->ws, B->arith);
   }
@@ -2612,6 +2631,107 @@ int choose_batch_halves(bmg_batch* B) {
   return BMG_OK;
 }
 
+// (n, storage, count, arith, shared operator, members per warp, two-sweep shape) -> 0 / 1
+static std::map<std::tuple<int, int, int, int, int, int, int>, int> g_tuned_rr;
+
+// The pass that also restricts against the group's own two sweeps plus the
+// separate residual + restriction, timed on scratch iterates like the sweeps
+// (the coarse right-hand sides and iterates both write are rewritten every
+// cycle). 8 problems of 1023^2 FP32: 155 us by two launches, 134 in one; 16 right-
+// hand sides: 83 / 70 at 511^2, and at 1023^2 the sweeps that read the shared
+// stencil once stay the faster (226).
+template <typename S>
+int tune_group_restrict(bmg_batch* B, bmg_batch::Group& g, int b) {
+  const LevelDesc<float, S>* host = (const LevelDesc<float, S>*)g.host.data();
+  const int shared = group_shared(B, g, b) ? 1 : 0;
+  auto key = std::make_tuple(g.n, g.storage, g.count, B->arith, shared, g.multi, g.pair);
+  auto it = g_tuned_rr.find(key);
+  const std::string fkey = tune_key("group_restrict", {g.n, g.storage, g.count, B->arith, shared, g.multi, g.pair});
+  TuneRecord fr;
+  if (it == g_tuned_rr.end() && tune_file_get(fkey, 1, &fr) && (fr.v[0] == 0 || fr.v[0] == 1))
+    it = g_tuned_rr.emplace(key, fr.v[0]).first;
+  if (it == g_tuned_rr.end()) {
+    const size_t ps = plane_stride32(g.n);
+    float* scratch = nullptr;
+    LevelDesc<float, S>* dd = nullptr;
+    Arena tmp;
+    int rc = galloc(tmp, &scratch, g.n, 3 * g.count, B->ws);
+    if (rc) return rc;
+    std::vector<LevelDesc<float, S>> d(host, host + g.count);
+    for (int k = 0; k < g.count; ++k) {
+      d[k].x = scratch + 3 * ps * k;
+      d[k].x2 = scratch + 3 * ps * k + ps;
+      d[k].f = scratch + 3 * ps * k + 2 * ps;
+      d[k].done = nullptr;
+    }
+    rc = cuda_check(dev_malloc((void**)&dd, sizeof(LevelDesc<float, S>) * g.count), "tuning descriptors");
+    if (!rc)
+      rc = cuda_check(cudaMemcpyAsync(dd, d.data(), sizeof(LevelDesc<float, S>) * g.count, cudaMemcpyHostToDevice, B->ws),
+                      "tuning descriptors");
+    bmg_batch::Group t = g;   // the group's own sweeps, on the scratch descriptors
+    t.d = dd;
+    float ms_sep = 1e30f, ms_one = 1e30f;
+    for (int round = 0; round < 2 && !rc; ++round) {
+      float ms = 0;
+      rc = time_call(B->ws, [&] {
+        t.dir = 0;
+        group_relax(B, t, 2);
+        group_restrict(B, t);
+      }, &ms);
+      ms_sep = std::min(ms_sep, ms);
+      if (!rc)
+        rc = time_call(B->ws, [&] {
+          t.dir = 0;
+          group_pair_restrict(B, t, false);
+        }, &ms);
+      ms_one = std::min(ms_one, ms);
+    }
+    cudaFree(dd);
+    if (!rc && strip_timeouts_b()) rc = set_error(BMG_ETIMEOUT, "batched two-sweep pass: bulk copies did not complete");
+    if (rc) return rc;
+    it = g_tuned_rr.emplace(key, ms_one < ms_sep ? 1 : 0).first;
+    tune_file_put(fkey, TuneRecord{{it->second}, std::min(ms_one, ms_sep)});
+  }
+  g.pair_rr = it->second;
+  return BMG_OK;
+}
+
+// Whether the arrays of group g (stage b) suit the pass's bulk copies.
+bool group_can_restrict(const bmg_batch* B, const bmg_batch::Group& g, int b) {
+  for (const bmg_hierarchy* h : B->hs) {
+    const int l = h->nlev - 1 - b;
+    if (l < 0) continue;
+    const Level& lv = h->lv[l];
+    if (lv.n != g.n || lv.kind != g.kind || (lv.bf16 ? 2 : 1) != g.storage) continue;
+    const void* o = lv.bf16 ? (const void*)viewbf(lv).O : (const void*)view32(lv).O;
+    if (!lv.pk32 || ((uintptr_t)lv.pk32 & 15) || ((uintptr_t)o & 15) || !lv.x32b) return false;
+  }
+  return true;
+}
+
+// Groups of FP32 9-point levels with two pre-smoothing sweeps, not by halves:
+// BMG_FUSE_AUTO, the tuner's choice where the sweeps are one-pass launches of its
+// own choosing; BMG_FUSE_ON, every group whose sweeps are such launches.
+int choose_batch_restrict(bmg_batch* B) {
+  const bool on = B->fuse_restrict == BMG_FUSE_ON;
+  if (B->precision == BMG_FP64 || B->rhs_block > BMG_RHS_BLOCK_OFF || B->nu1 != 2 ||
+      B->fuse_restrict == BMG_FUSE_OFF || (!on && (!B->use_graph || B->smoother != BMG_SMOOTHER_AUTO)))
+    return BMG_OK;
+  std::lock_guard<std::mutex> guard(tune_lock());
+  for (int b = 1; b <= B->bmax; ++b)
+    for (auto& g : B->stages[b]) {
+      if (!g.count || g.kind != 9 || g.tile < 0 || g.rows > 0 || g.storage == 0 || !group_can_restrict(B, g, b))
+        continue;
+      if (on) {
+        g.pair_rr = 1;
+        continue;
+      }
+      int rc = g.storage == 1 ? tune_group_restrict<float>(B, g, b) : tune_group_restrict<__nv_bfloat16>(B, g, b);
+      if (rc) return rc;
+    }
+  return BMG_OK;
+}
+
 int autotune_batch(bmg_batch* B) {
   std::lock_guard<std::mutex> guard(tune_lock());
   // descriptor contents are needed: build the tables with the internal level
@@ -2662,6 +2782,7 @@ int batch_init(bmg_batch* B, const bmg_opts* o, bmg_opts* so) {
     B->user = (cudaStream_t)o->stream;
     B->arith = o->arith;
     B->rhs_block = o->rhs_block;
+    B->fuse_restrict = o->fuse_restrict;
   }
   if (B->rhs_block != BMG_RHS_BLOCK_AUTO && B->rhs_block != BMG_RHS_BLOCK_OFF && B->rhs_block != 2 &&
       B->rhs_block != 4)
@@ -2774,6 +2895,7 @@ int batch_finish(bmg_batch* B, int rc) {
   if (!rc && B->smoother >= BMG_SMOOTHER_TILE) rc = force_batch_onepass(B);
   if (!rc && B->use_graph) rc = autotune_batch(B);
   if (!rc) rc = choose_batch_halves(B);
+  if (!rc) rc = choose_batch_restrict(B);
   if (!rc) rc = force_rhs_block(B);
   if (!rc) rc = cuda_check(cudaStreamSynchronize(B->ws), "batched setup");
   return rc;

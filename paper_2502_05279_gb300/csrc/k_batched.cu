@@ -134,6 +134,32 @@ __global__ void __launch_bounds__(32 * STRIP_WARPS_B) k_gs_strip2_ring_b(const L
     atomicExch(&g_strip_timeout_b, 1);
 }
 
+// Two sweeps, residual and restriction of a group in one pass (44 x ty strips;
+// gs_strip2r_ring_body): warp g takes strip g % wpp of problem g / wpp. ZERO:
+// every member's iterate is zero on entry and is not read. Three resident blocks
+// (168 registers), as the single-problem kernel.
+template <typename S, int RING, bool FU, bool ZERO>
+__global__ void __launch_bounds__(32 * STRIP_WARPS_B, 3) k_gs_strip2r_ring_b(const LevelDesc<float, S>* __restrict__ d,
+                                                                          int count, int n, int dir, int ty) {
+  pdl_enter();
+  extern __shared__ __align__(128) unsigned char strip_smem[];
+  const int nbx = (n + 43) / 44, wpp = nbx * ((n + ty - 1) / ty);
+  const int w = threadIdx.x >> 5;
+  const long g = (long)blockIdx.x * STRIP_WARPS_B + w;
+  const int p = (int)(g / wpp), sidx = (int)(g % wpp);
+  if (p >= count) return;
+  const LevelDesc<float, S>& q = d[p];
+  if (stopped(q.done)) return;
+  unsigned char* ring = strip_smem + (size_t)w * RING * StripRingR<S>::SLOT;
+  unsigned long long* bars =
+      reinterpret_cast<unsigned long long*>(strip_smem + (size_t)STRIP_WARPS_B * RING * StripRingR<S>::SLOT) +
+      w * RING;
+  if (!gs_strip2r_ring_body<S, RING, FU, ZERO>(q.v, q.f, dir ? q.x2 : q.x, dir ? q.x : q.x2, q.ci, q.fc, q.xc,
+                                               sidx % nbx, sidx / nbx, ty, ring, bars) &&
+      (threadIdx.x & 31) == 0)
+    atomicExch(&g_strip_timeout_b, 1);
+}
+
 // FP64 one-pass sweeps of a group (strips of 56 x ty, rows copied per lane; see
 // gs_strip64_body): warp g takes strip g % wpp of problem g / wpp.
 template <int RING, bool FU>
@@ -359,6 +385,36 @@ static void gs_pair_b(const LevelDesc<float, S>* d, int count, int n, int shape,
   }
 }
 
+// Strip height: a warp walks ty rows and 11 of halo, and all strips of the group
+// run in whole waves of resident warps, so of the heights that fill 1 .. 4 waves
+// the one with the fewest rows walked in turn.
+template <typename S, int RING, bool FU, bool ZERO>
+static void strip2r_b_launch(const LevelDesc<float, S>* d, int count, int n, int dir, cudaStream_t s) {
+  if (count <= 0) return;
+  constexpr size_t bytes = (size_t)STRIP_WARPS_B * RING * (StripRingR<S>::SLOT + 8);
+  static const int resident_warps = [] {
+    auto k = k_gs_strip2r_ring_b<S, RING, FU, ZERO>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * STRIP_WARPS_B, bytes);
+    return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1) * STRIP_WARPS_B;
+  }();
+  const long cols = (long)count * ((n + 43) / 44);
+  long ty = n + 1, cost = 0;
+  for (int waves = 1; waves <= 4; ++waves) {
+    const long nby = (long)waves * resident_warps / cols;
+    if (nby < 1) continue;
+    const long t = 2 * ((n + 2 * nby - 1) / (2 * nby)), c = waves * (t + 11);
+    if (cost == 0 || c < cost) ty = t, cost = c;
+  }
+  const long warps = cols * ((n + ty - 1) / ty);
+  pdl_launch(k_gs_strip2r_ring_b<S, RING, FU, ZERO>, (unsigned)((warps + STRIP_WARPS_B - 1) / STRIP_WARPS_B),
+             32 * STRIP_WARPS_B, bytes, s, d, count, n, dir, (int)ty);
+  count_launch();
+}
+
 // ty = 0: the smallest even strip height whose strips, over all `count`
 // problems, fit into one wave of resident warps.
 template <int RING, bool FU>
@@ -466,6 +522,18 @@ void launch_gs_pair_b(const LevelDesc<float, S>* d, int count, int n, int shape,
   else
     gs_pair_b<S, false>(d, count, n, shape, dir, s);
 }
+template <typename S>
+void launch_gs_pair_restrict_b(const LevelDesc<float, S>* d, int count, int n, int dir, int zero, cudaStream_t s,
+                               int fused) {
+  if (fused)
+    zero ? strip2r_b_launch<S, 4, true, true>(d, count, n, dir, s) : strip2r_b_launch<S, 4, true, false>(d, count, n, dir, s);
+  else
+    zero ? strip2r_b_launch<S, 4, false, true>(d, count, n, dir, s)
+         : strip2r_b_launch<S, 4, false, false>(d, count, n, dir, s);
+}
+template void launch_gs_pair_restrict_b<float>(const LevelDesc<float, float>*, int, int, int, int, cudaStream_t, int);
+template void launch_gs_pair_restrict_b<__nv_bfloat16>(const LevelDesc<float, __nv_bfloat16>*, int, int, int, int,
+                                                       cudaStream_t, int);
 template void launch_gs_tile_b<float>(const LevelDesc<float, float>*, int, int, int, int, cudaStream_t, int);
 template void launch_gs_tile_b<__nv_bfloat16>(const LevelDesc<float, __nv_bfloat16>*, int, int, int, int,
                                               cudaStream_t, int);

@@ -270,6 +270,12 @@ bool launch_gs_tile_bk(const LevelDesc<float, S>* d, int count, int n, int k, in
 template <typename S>
 void launch_gs_pair_b(const LevelDesc<float, S>* d, int count, int n, int shape, int dir, cudaStream_t s,
                       int fused = 0);
+// Two sweeps, the residual and its restriction of a group of 9-point FP32 levels
+// in one pass (dir as launch_gs_tile_b; zero: the iterates are zero and are not
+// read). Needs the packed stencil and a 16-byte aligned diagonal plane.
+template <typename S>
+void launch_gs_pair_restrict_b(const LevelDesc<float, S>* d, int count, int n, int dir, int zero, cudaStream_t s,
+                               int fused = 0);
 // Batched FP64 one-pass sweeps (dir as launch_gs_tile_b); shapes as
 // launch_gs_tile64, with the one-wave height taken over all `count` problems.
 void launch_gs_tile64_b(const LevelDesc<double, double>* d, int count, int n, int shape, int dir, cudaStream_t s,
