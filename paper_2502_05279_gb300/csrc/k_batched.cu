@@ -212,25 +212,46 @@ __global__ void __launch_bounds__(NORM_THREADS) k_finalize_b(const TopDesc* __re
   finalize_body(q.partials, norm_blocks(q.v.n), q.ctl, phase, nullptr);
 }
 
+constexpr int IRB_ENTRIES = 4;
 // Over the blocks of bmap too: block b of a problem takes its rows 1 + b, 1 + b + G, ...
 // (a grid of the largest problem's size for every problem spent 61 us, half of
-// it on empty blocks, on 40 problems of 63^2 .. 1023^2).
+// it on empty blocks, on 40 problems of 63^2 .. 1023^2). Four entries a CTA: with
+// one, the dependent loads before its few points (entry, descriptor, control
+// block) took most of its time (16 problems of 1023^2: 69 us against 49 for the
+// bytes; an iteration 890 -> 876 us, of 40 problems 759 -> 743).
 __global__ void __launch_bounds__(NORM_THREADS) k_ir_update_b(const TopDesc* __restrict__ d,
-                                                              const int2* __restrict__ bmap) {
+                                                              const int2* __restrict__ bmap, int nblocks) {
   pdl_enter();
-  const int2 m = bmap[blockIdx.x];
-  const TopDesc& q = d[m.x];
-  if (q.ctl->done) return;
-  const int n = q.v.n, G = norm_blocks(n);
-  const double s = q.ctl->scale_applied;
-  for (int j = 1 + m.y; j <= n; j += G)
-    for (int i = 1 + (int)threadIdx.x; i <= n; i += NORM_THREADS * IRU_COLS)
-      ir_update_cols(n, q.x, q.e32, s, i, j, NORM_THREADS);
+  int prev = -1, n = 0, G = 1;
+  bool run = false;
+  double s = 0.0;
+  double* x = nullptr;
+  const float* e32 = nullptr;
+  for (int k = blockIdx.x * IRB_ENTRIES; k < nblocks && k < (int)(blockIdx.x + 1) * IRB_ENTRIES; ++k) {
+    const int2 m = bmap[k];
+    if (m.x != prev) {
+      const TopDesc& q = d[m.x];
+      prev = m.x;
+      run = !q.ctl->done;
+      s = q.ctl->scale_applied;
+      n = q.v.n;
+      G = norm_blocks(n);
+      x = q.x;
+      e32 = q.e32;
+    }
+    if (!run) continue;
+    for (int j = 1 + m.y; j <= n; j += G)
+      for (int i = 1 + (int)threadIdx.x; i <= n; i += NORM_THREADS * IRU_COLS)
+        ir_update_cols(n, x, e32, s, i, j, NORM_THREADS);
+  }
 }
 
+// One canonical block a CTA, six resident: taking two or four in turn spared
+// their start and end but not the registers (spills: 890 -> 921 / 940 us an
+// iteration of 16 right-hand sides of 1023^2).
 template <bool FU>
 __global__ void __launch_bounds__(NORM_THREADS, 6) k_ir_residual_b(const TopDesc* __restrict__ d,
-                                                                const int2* __restrict__ bmap) {
+                                                                   const int2* __restrict__ bmap) {
   pdl_enter();
   const int2 m = bmap[blockIdx.x];
   const TopDesc& q = d[m.x];
@@ -569,7 +590,7 @@ void launch_finalize_b(const TopDesc* d, int count, int phase, cudaStream_t s) {
 }
 
 void launch_ir_update_b(const TopDesc* d, const int2* bmap, int nblocks, cudaStream_t s) {
-  pdl_launch(k_ir_update_b, nblocks, NORM_THREADS, 0, s, d, bmap);
+  pdl_launch(k_ir_update_b, (nblocks + IRB_ENTRIES - 1) / IRB_ENTRIES, NORM_THREADS, 0, s, d, bmap, nblocks);
   count_launch();
 }
 
