@@ -128,7 +128,8 @@ typedef struct {
   int bf16_levels;      /* levels with BF16 stencils under BMG_BF16_IR (0 = 2) */
   int use_graph;        /* 1 (default): replay one captured CUDA graph per cycle, autotune the
                            row-kernel tiles and run the coarse levels (n <= 63 FP32, n <= 31 FP64)
-                           as one level-fused launch; 0: plain launches, one per step */
+                           as one level-fused launch, small levels above them as one launch
+                           down and one up; 0: plain launches, one per step */
   int krylov;           /* BMG_KRYLOV_NONE (default): stationary V-cycle iteration;
                            BMG_KRYLOV_FCG: flexible CG with one cycle as preconditioner */
   const void* mlp;      /* bmg_mlp* for interp = BMG_INTERP_LEARNED, else NULL */
@@ -153,7 +154,8 @@ typedef struct {
                            pass (nu1 = 2): BMG_FUSE_AUTO (0, default; the autotuner weighs one pass
                            that also forms the residual and restricts it -- temporal blocking --
                            against the two-sweep pass plus the separate residual + restriction),
-                           BMG_FUSE_OFF, or BMG_FUSE_ON (always the fused pass).  Same bits. */
+                           BMG_FUSE_OFF, or BMG_FUSE_ON (always the fused pass; in a batch, on every
+                           stage whose sweeps are one-pass launches).  Same bits. */
   int rhs_block;        /* batches of right-hand sides of one operator (bmg_batch_rhs), FP32 / BF16
                            levels swept by the one-pass kernel: BMG_RHS_BLOCK_AUTO (0, default; the
                            autotuner weighs sweeping 2 or 4 members per warp, each stencil value read
@@ -258,7 +260,8 @@ typedef struct {
   int kernel;           /* BMG_K_* */
   int fp32;             /* 1 = a kernel of the FP32 inner cycle */
   int launches;         /* kernel launches summed into this row */
-  double ms;            /* total device time */
+  double ms;            /* total device time (levels that a solve runs as one launch down and one
+                           up are timed step by step) */
 } bmg_prof_row;
 int bmg_profile(bmg_hierarchy* h, const double* rhs, double* x, int cycles, bmg_prof_row* rows, int cap);
 
