@@ -2609,9 +2609,10 @@ int force_rhs_block(bmg_batch* B) {
 //   10 problems BF16: -28 / -28 / -9 / -1
 //   16 right-hand sides of 1023^2 FP32: -13 / -8 / +17 / +148 (block sweeps read the shared stencil once)
 //   FP64 at 63 / 127: 40 problems -4 / +13, 10 problems -5 (8 rows) / -1, 8 right-hand sides -8 (8 rows) / -2:
-//   the halos' FP64 work costs more than the launches as soon as the problems fill the chip
+//   the halos' FP64 work costs more than the launches as soon as the problems fill the chip: 256
+//   problems' iteration takes 10486 us by halves at 63, 10359 step by step (64 problems: 2587 / 2584)
 int batch_rows(bool f64, int n, int count, bool shared) {
-  if (f64) return n > 63 ? 0 : count <= 16 ? 8 : 16;
+  if (f64) return n > 63 || count > 48 ? 0 : count <= 16 ? 8 : 16;
   return n <= 255 || (n <= 511 && !shared) ? 16 : 0;
 }
 
