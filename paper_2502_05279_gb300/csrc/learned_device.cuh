@@ -43,15 +43,28 @@ __device__ __forceinline__ float2 feature_pair(double w, double e, double s, dou
   return make_float2(feature_round(sx * y, sx, o), feature_round(sy * y, sy, o));
 }
 
-// exp(second logit) / exp(first logit): one exponential (about 25 FP64
-// operations) per edge point instead of two.
-__device__ __forceinline__ double logit_ratio(double second, double first) { return exp(rsub(second, first)); }
+// Share of the first of an edge point's two coarse points, u_1 / (u_1 + u_2) with
+// u_k = c_k exp(l_k): both terms divided by exp(l_1), one exponential (about 25
+// FP64 operations) instead of two.  Logits 600 and more apart (or NaN) take the
+// two exponentials: exp(l_2 - l_1) then leaves the FP64 range, or comes so near
+// its ends that a product with c_2 may, and with a c_k of zero (no coupling to
+// that side) the share would be NaN.  The test is on the bit pattern.
+static __device__ __noinline__ double first_share_apart(double c1, double c2, double l1, double l2) {
+  const double u1 = rmul(c1, exp(l1)), u2 = rmul(c2, exp(l2));
+  return rdiv(u1, radd(u1, u2));
+}
+
+__device__ __forceinline__ double first_share(double c1, double c2, double l1, double l2) {
+  const double d = rsub(l2, l1);
+  if (((unsigned)__double2hiint(d) & 0x7fffffffu) >= 0x4082c000u) return first_share_apart(c1, c2, l1, l2);
+  return rdiv(c1, radd(c1, rmul(c2, exp(d))));
+}
 
 // Edge points of cell (ic, jc), 0 <= ic, jc <= nc+1: x-edge (2ic-1, 2jc) between
 // (ic-1, jc) [its E logit] and (ic, jc) [its W logit]; y-edge (2ic, 2jc-1)
 // between (ic, jc-1) [N logit] and (ic, jc) [S logit].  An edge point keeps
 // Dendy's total weight S_D = -(col_1 + col_2)/D and splits it in the shares
-// u_k = -col_k exp(logit), both divided by exp(first logit).  aux (optional, 4 coarse planes) keeps S_D and the
+// u_k = -col_k exp(logit).  aux (optional, 4 coarse planes) keeps S_D and the
 // first share q for the gradient.
 __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int nc, const float* delta, int ic, int jc,
                                           double* ci, double* aux) {
@@ -64,8 +77,7 @@ __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int n
     double colE = radd(radd(A.a<8>(p, ld), A.a<2>(p, ld)), A.a<6>(p, ld));
     double D = radd(radd(A.a<3>(p, ld), A.a<0>(p, ld)), A.a<4>(p, ld));
     sdx = -rdiv(radd(colW, colE), D);
-    double uE = rmul(-colE, logit_ratio(delta_at(delta, nc, ic, jc, 0), delta_at(delta, nc, ic - 1, jc, 1)));
-    qx = rdiv(-colW, radd(-colW, uE));
+    qx = first_share(-colW, -colE, delta_at(delta, nc, ic - 1, jc, 1), delta_at(delta, nc, ic, jc, 0));
     ll = rmul(sdx, qx);
     lr = rmul(sdx, rsub(1.0, qx));
   }
@@ -75,8 +87,7 @@ __device__ __forceinline__ void edge_cell(const Planes<double>& A, int ld, int n
     double rowN = radd(radd(A.a<7>(p, ld), A.a<4>(p, ld)), A.a<6>(p, ld));
     double D = radd(radd(A.a<1>(p, ld), A.a<0>(p, ld)), A.a<2>(p, ld));
     sdy = -rdiv(radd(rowS, rowN), D);
-    double uN = rmul(-rowN, logit_ratio(delta_at(delta, nc, ic, jc, 2), delta_at(delta, nc, ic, jc - 1, 3)));
-    qy = rdiv(-rowS, radd(-rowS, uN));
+    qy = first_share(-rowS, -rowN, delta_at(delta, nc, ic, jc - 1, 3), delta_at(delta, nc, ic, jc, 2));
     lb = rmul(sdy, qy);
     la = rmul(sdy, rsub(1.0, qy));
   }
