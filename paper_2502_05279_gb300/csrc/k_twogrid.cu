@@ -71,12 +71,40 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // 1/d to about an ulp by Newton's iteration from the hardware's approximation
-// (a division would take 560 cycles in the factorisation's chain).
+// (a division would take 560 cycles in the factorisation's chain).  d normal and
+// below 2^1022, which the scaled band's pivots are.
 __device__ __forceinline__ double recip_newton(double d) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;\n" : "=d"(y) : "d"(d));
   y = __fma_rn(y, __fma_rn(-d, y, 1.0), y);
   return __fma_rn(y, __fma_rn(-d, y, 1.0), y);
+}
+
+// Scales the band of A_c by the power of two that brings its largest diagonal
+// entry into [1, 2), and returns it: band_factor multiplies two entries before it
+// divides by a pivot, which over- or underflows for operators beyond 2^+-500 (and
+// recip_newton beyond 2^+-1022) if the band is left as it is.  Exact, so results
+// scale with the operator bit for bit; the entries set are those of the 9-point
+// operator.  scratch: WARPS ints.
+template <int N>
+__device__ double band_scale(double* band, int* scratch) {
+  using L = TG<N>;
+  constexpr int M = L::M, NC = L::NC, BL = L::BL;
+  int top = 0;
+  for (int c = threadIdx.x; c < M; c += L::THREADS)
+    top = max(top, (int)(((unsigned)__double2hiint(band[c * BL]) >> 20) & 0x7ffu));
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = top;
+  __syncthreads();
+  for (int w = 0; w < L::WARPS; ++w) top = max(top, scratch[w]);
+  const int e = top == 2047 ? 1023 : min(max(2046 - top, 1), 2045);   // biased exponent of 2^(1023 - top)
+  const double s = __hiloint2double(e << 20, 0);
+  constexpr int at[5] = {0, 1, NC - 1, NC, NC + 1};
+  for (int c = threadIdx.x; c < M; c += L::THREADS)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) band[c * BL + at[q]] *= s;
+  __syncthreads();
+  return s;
 }
 
 // Banded L D L^T of the lower band (row i holds A(i, i-d) at d = 0..BW), by the
@@ -302,10 +330,12 @@ __global__ void __launch_bounds__(TG<N>::THREADS, 1)
     if (ic > 1 && jc < NC) band[(c + NC - 1) * BL + NC - 1] = rapdev::rap_entry<-1, 1>(A, LD, ci, PSC, LDC, NC, ic, jc);
   }
   __syncthreads();
+  const double scale = band_scale<N>(band, reinterpret_cast<int*>(red));
   if (!band_factor<N>(band, rd)) {   // every thread sees every pivot
     if (tid == 0) atomicExch(err, 1);
     return;
   }
+  for (int e = tid; e < M; e += NT) rd[e] *= scale;   // 1 / D of the unscaled operator (the first vectors' barriers order it)
   // this thread's block and coarse cell (bi + 1, bj + 1)
   const bool va = tid < L::NB2;
   const int bi = va ? tid % NB : 0, bj = va ? tid / NB : 0, i = 2 * bi + 1, j = 2 * bj + 1;
