@@ -16,9 +16,8 @@
 // takes the operands and the order of the colour-by-colour sweep.
 //
 // The stencil and the weights are constant over a solve, so they are loaded
-// before the wait for the preceding kernel; k_level_up also loads the level's
-// right-hand side and iterate there, which k_level_down (or the restriction
-// before it) wrote at least one completed kernel before the preceding one.
+// before the wait for the preceding kernel; everything that a cycle writes is
+// loaded after it.
 #include "block_device.cuh"
 
 namespace bmg {
@@ -194,10 +193,10 @@ __device__ __forceinline__ void up_body(const StencilView<T, S>& v, const LevelG
   T w[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) w[k] = ci[k * psc + pc];
-  const BlockX<T> fb = level_values(B, f);
-  BlockX<T> x = level_values(B, xin);
   pdl_enter();
   if (stopped(done)) return;
+  const BlockX<T> fb = level_values(B, f);
+  BlockX<T> x = level_values(B, xin);
   block_interp<FU>(x, ec[m.coarse(ic - 1, jc - 1)], ec[m.coarse(ic, jc - 1)], ec[m.coarse(ic - 1, jc)],
                    ec[m.coarse(ic, jc)], B.va, B.vb, B.vc, B.vd, [&](int k) { return w[k]; });
   level_planes(B, x);

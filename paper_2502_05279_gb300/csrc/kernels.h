@@ -146,8 +146,8 @@ void launch_gs_tile64(const StencilView<double, double>& v, const double* f, con
 // xin (NULL: zero) into xout, the residual restricted into fc, and xc (may be
 // NULL) zeroed.  up: xout = nu2 sweeps on xin + P ec.  xout != xin; 1 <= nu <=
 // LEVEL_NU_MAX and rows >= 2 nu1 + 4.  The same bits as the separate launches.
-// v, ci, and for up also f and xin, must have been written before the launch
-// that precedes on the stream started.
+// v and ci are read before the wait for the preceding kernel: constants of the
+// solve, written by the setup.
 constexpr int LEVEL_NU_MAX = 2;
 // Points of a level along x and y, and which of the axes are periodic.
 struct LevelGrid {
