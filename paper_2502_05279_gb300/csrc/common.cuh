@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "../../include/bmg.h"
+#include "per_device.h"
 
 namespace bmg {
 
@@ -127,6 +128,17 @@ __host__ __device__ inline Planes<S> planes_at(const S* base, size_t ps) {
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+// Raises kernel k's dynamic shared-memory limit to `bytes` on the current device;
+// `once` is a static of k's launch function.
+template <typename K>
+inline cudaError_t allow_smem(PerDevice& once, K k, size_t bytes) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return (cudaError_t)once.once(dev, [&] {
+    return (int)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
 }
 
 template <typename... KArgs, typename... Args>

@@ -361,21 +361,23 @@ void launch_interp_b(const LevelDesc<T, S>* d, int count, int n, cudaStream_t s,
   count_launch();
 }
 
+// How many warps of a strip kernel (CTAs of STRIP_WARPS_B warps, `bytes` of dynamic
+// shared memory, already allowed) fit on the device at once.
+template <typename K>
+static int resident_strip_warps_b(K kernel, size_t bytes) {
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * STRIP_WARPS_B, bytes);
+  return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1) * STRIP_WARPS_B;
+}
+
 template <typename S, int TY, int RING, bool PAIR, bool FU>
 static void strip_b_launch(const LevelDesc<float, S>* d, int count, int n, int dir, cudaStream_t s) {
   if (count <= 0) return;
   constexpr size_t bytes = (size_t)STRIP_WARPS_B * RING * (StripRing<S>::SLOT + 8);
-  // the shared-memory limit is raised once per kernel (thread-safe static initialisation)
-  static const bool attr = [] {
-    if (PAIR)
-      cudaFuncSetAttribute(k_gs_strip2_ring_b<S, TY, RING, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bytes);
-    else
-      cudaFuncSetAttribute(k_gs_strip_ring_b<S, TY, RING, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bytes);
-    return true;
-  }();
-  (void)attr;
+  static PerDevice smem;
+  allow_smem(smem, PAIR ? k_gs_strip2_ring_b<S, TY, RING, FU> : k_gs_strip_ring_b<S, TY, RING, FU>, bytes);
   const int width = PAIR ? 48 : 56;
   const long warps = (long)count * ((n + width - 1) / width) * ((n + TY - 1) / TY);
   const unsigned blocks = (unsigned)((warps + STRIP_WARPS_B - 1) / STRIP_WARPS_B);
@@ -413,15 +415,9 @@ template <typename S, int RING, bool FU, bool ZERO>
 static void strip2r_b_launch(const LevelDesc<float, S>* d, int count, int n, int dir, cudaStream_t s) {
   if (count <= 0) return;
   constexpr size_t bytes = (size_t)STRIP_WARPS_B * RING * (StripRingR<S>::SLOT + 8);
-  static const int resident_warps = [] {
-    auto k = k_gs_strip2r_ring_b<S, RING, FU, ZERO>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * STRIP_WARPS_B, bytes);
-    return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1) * STRIP_WARPS_B;
-  }();
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip2r_ring_b<S, RING, FU, ZERO>, bytes);
+  static const int resident_warps = resident_strip_warps_b(k_gs_strip2r_ring_b<S, RING, FU, ZERO>, bytes);
   const long cols = (long)count * ((n + 43) / 44);
   long ty = n + 1, cost = 0;
   for (int waves = 1; waves <= 4; ++waves) {
@@ -442,14 +438,9 @@ template <int RING, bool FU>
 static void strip64_b_launch(const LevelDesc<double, double>* d, int count, int n, int dir, cudaStream_t s, int ty) {
   if (count <= 0) return;
   constexpr size_t bytes = (size_t)STRIP_WARPS_B * RING * STRIP64_SLOT;
-  static const int resident_warps = [] {
-    cudaFuncSetAttribute(k_gs_strip64_b<RING, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gs_strip64_b<RING, FU>, 32 * STRIP_WARPS_B, bytes);
-    return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1) * STRIP_WARPS_B;
-  }();
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip64_b<RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps_b(k_gs_strip64_b<RING, FU>, bytes);
   const long cols = (long)count * ((n + 55) / 56);
   if (ty <= 0) {
     const long nby_max = resident_warps / cols > 1 ? resident_warps / cols : 1;
@@ -495,15 +486,9 @@ static void strip_bk_launch(const LevelDesc<float, S>* d, int count, int n, int 
   if (count <= 0) return;
   constexpr int RING = 4;
   constexpr size_t bytes = (size_t)STRIP_WARPS_B * RING * (StripRingK<S, K>::SLOT + 8);
-  static const int resident_warps = [] {
-    cudaFuncSetAttribute(k_gs_strip_ring_bk<S, K, RING, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gs_strip_ring_bk<S, K, RING, FU>, 32 * STRIP_WARPS_B,
-                                                  bytes);
-    return (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1) * STRIP_WARPS_B;
-  }();
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip_ring_bk<S, K, RING, FU>, bytes);
+  static const int resident_warps = resident_strip_warps_b(k_gs_strip_ring_bk<S, K, RING, FU>, bytes);
   const int groups = (count + K - 1) / K, nbx = (n + 55) / 56;
   const long cols = (long)groups * nbx;
   const int nby_max = resident_warps / cols > 1 ? (int)(resident_warps / cols) : 1;

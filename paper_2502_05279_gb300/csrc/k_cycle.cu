@@ -346,13 +346,11 @@ static void strip_launch(const StencilView<float, S>& v, const float* f, const f
   count_launch();
 }
 
-// Raise a kernel's dynamic shared-memory limit to `bytes` and return how many
-// warps of it (CTAs of STRIP_WARPS warps) fit on the device at once.  Callers
-// keep the result in a function-local static, whose initialisation C++ makes
-// thread-safe.
+// How many warps of a kernel (CTAs of STRIP_WARPS warps, `bytes` of dynamic shared
+// memory, already allowed) fit on the device at once.  Callers keep the result in
+// a function-local static, whose initialisation C++ makes thread-safe.
 template <typename K>
 static int resident_strip_warps(K kernel, size_t bytes) {
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -366,6 +364,8 @@ template <typename S, int RING, bool FU, bool ZERO>
 static void strip_ring_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                               const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRing<S>::SLOT + 8);
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip_ring<S, RING, FU, ZERO>, bytes);
   static const int resident_warps = resident_strip_warps(k_gs_strip_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 55) / 56;
   if (ty <= 0) {
@@ -412,6 +412,8 @@ template <int RING, bool FU, bool ZERO>
 static void strip64_launch(const StencilView<double, double>& v, const double* f, const double* xin, double* xout,
                            const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * STRIP64_SLOT;
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip64<RING, FU, ZERO>, bytes);
   static const int resident_warps = resident_strip_warps(k_gs_strip64<RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 55) / 56;
   if (ty <= 0) {
@@ -464,6 +466,8 @@ template <typename S, int RING, bool FU, bool ZERO>
 static void strip2_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                           const int* done, cudaStream_t s, int ty) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRing<S>::SLOT + 8);
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip2_ring<S, RING, FU, ZERO>, bytes);
   static const int resident_warps = resident_strip_warps(k_gs_strip2_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 47) / 48;
   if (ty <= 0) {
@@ -493,6 +497,8 @@ template <typename S, int RING, bool FU, bool ZERO>
 static void strip2r_launch(const StencilView<float, S>& v, const float* f, const float* xin, float* xout,
                            const float* ci, float* fc, float* xc, const int* done, cudaStream_t s) {
   constexpr size_t bytes = (size_t)STRIP_WARPS * RING * (StripRingR<S>::SLOT + 8);
+  static PerDevice smem;
+  allow_smem(smem, k_gs_strip2r_ring<S, RING, FU, ZERO>, bytes);
   static const int resident_warps = resident_strip_warps(k_gs_strip2r_ring<S, RING, FU, ZERO>, bytes);
   const int nbx = (v.n + 43) / 44;
   const int nby_max = resident_warps / nbx > 1 ? resident_warps / nbx : 1;

@@ -659,9 +659,8 @@ void launch_mlp_fwd(const float* X, int M, const float* par, float* Z1, float* Z
 
 void launch_mlp_bwd(const float* X, int M, const float* par, const float* Z1, const float* Z2, const float* dout,
                     float* partial, float* grad, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BwdShared));
-  (void)attr;   // a failure shows at the launch
+  static PerDevice smem;
+  allow_smem(smem, k_mlp_bwd, sizeof(BwdShared));   // a failure shows at the launch
   const int nb = mlp_backward_blocks(M);
   k_mlp_bwd<<<nb, 256, sizeof(BwdShared), s>>>(X, M, par, Z1, Z2, dout, partial);
   k_sum_partials<<<(NPAR + 31) / 32, 256, 0, s>>>(partial, nb, grad);

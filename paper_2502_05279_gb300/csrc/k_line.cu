@@ -228,14 +228,12 @@ void half_sweep(const StencilView<T, S>& v, int kind, const T* f, T* x, const Li
   constexpr size_t bytes = 2 * sizeof(LineStage<T, R>);
   const unsigned g = (unsigned)((lines + R - 1) / R);
   if (kind == 9) {
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        k_line_solve<T, S, true, AXIS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    (void)attr;
+    static PerDevice smem;
+    allow_smem(smem, k_line_solve<T, S, true, AXIS, R>, bytes);
     pdl_launch(k_line_solve<T, S, true, AXIS, R>, g, LINE_THREADS, bytes, s, v, f, x, fac, first, done);
   } else {
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        k_line_solve<T, S, false, AXIS, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    (void)attr;
+    static PerDevice smem;
+    allow_smem(smem, k_line_solve<T, S, false, AXIS, R>, bytes);
     pdl_launch(k_line_solve<T, S, false, AXIS, R>, g, LINE_THREADS, bytes, s, v, f, x, fac, first, done);
   }
   count_launch();

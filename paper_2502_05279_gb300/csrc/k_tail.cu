@@ -288,10 +288,8 @@ __global__ void __launch_bounds__(tail_blocks<T>() * tail_blocks<T>(), 1)
 
 template <typename T, bool FU>
 void tail_launch(const TailDesc<T>* d, int count, int top_n, int nlev, const int* done_any, cudaStream_t s) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_tail<T, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)(tail_layout<T>(tail_max_n<T>(), sizeof(T) == 8 ? 4 : 5, nullptr) * sizeof(T)));
-  (void)attr;
+  static PerDevice smem;
+  allow_smem(smem, k_tail<T, FU>, tail_layout<T>(tail_max_n<T>(), sizeof(T) == 8 ? 4 : 5, nullptr) * sizeof(T));
   const int b = (top_n + 1) / 2;
   pdl_launch(k_tail<T, FU>, count, b * b < 32 ? 32 : b * b, tail_layout<T>(top_n, nlev, nullptr) * sizeof(T), s, d,
              done_any);

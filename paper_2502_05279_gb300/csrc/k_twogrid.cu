@@ -556,9 +556,8 @@ __global__ void k_features_crops(int n, const double* __restrict__ coefs, float*
 template <int N>
 int launch_twogrid_n(int ncrop, int K, const double* coefs, const double* vecs, const float* delta, const double* eref,
                      double weight, double* energies, float* ddelta, double* aux, int* err, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(k_twogrid<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG<N>::BYTES);
-  if (attr != cudaSuccess) return cuda_check(attr, "two-grid kernel shared memory");
+  static PerDevice smem;
+  if (int rc = cuda_check(allow_smem(smem, k_twogrid<N>, TG<N>::BYTES), "two-grid kernel shared memory")) return rc;
   k_twogrid<N><<<ncrop, TG<N>::THREADS, TG<N>::BYTES, s>>>(K, coefs, vecs, delta, eref, weight, energies, ddelta,
                                                            eref ? aux : nullptr, err);
   count_launch();
