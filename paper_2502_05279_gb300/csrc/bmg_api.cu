@@ -215,45 +215,52 @@ StencilView<float, __nv_bfloat16> viewbf(const Level& L) {
 
 namespace {
 // Device memory of one hierarchy (or of one tuning run), given back as a whole
-// when its owner goes.  Arrays are cut from chunks, zeroed when they are made;
-// an array of more than half a chunk gets an allocation of its own.  A
-// cudaMalloc or cudaFree takes 10 to 20 us and a hierarchy has about ninety
-// arrays: at 1023^2 they were half of the 2.0 ms of a setup and all of the 1.2
-// ms of a release.
+// when its owner goes.  Arrays are cut from chunks, zeroed when they are made,
+// first fit over what is left of each; an array of more than half a chunk gets an
+// allocation of its own.  A cudaMalloc or cudaFree takes 10 to 20 us and a
+// hierarchy has about ninety arrays: at 1023^2 they were half of the 2.0 ms of a
+// setup and all of the 1.2 ms of a release.
 struct Arena {
+  struct Rest {
+    char* at;
+    size_t bytes;
+  };
   std::vector<void*> blocks;
-  char* cur = nullptr;
-  size_t left = 0, chunk = (size_t)2 << 20;
+  std::vector<Rest> rests;
+  size_t chunk = (size_t)2 << 20;
   Arena() = default;
   Arena(const Arena&) = delete;
   Arena& operator=(const Arena&) = delete;
   ~Arena() {
     for (void* b : blocks) cudaFree(b);
   }
-  // Chunks of about four planes of the finest level, 2 to 64 MB.
-  void size_for(int n) {
-    chunk = std::min(std::max(4 * plane_size(n) * sizeof(double), (size_t)2 << 20), (size_t)64 << 20);
+  // For a hierarchy whose arrays come to about `planes` FP64 planes of its finest
+  // level: one chunk that holds them where 2 MB do (a batch may hold thousands of
+  // small problems; 15^2 take 0.1 MB each, 2 MB with a chunk of 2 MB for each),
+  // else four planes, 4 to 64 MB in steps of the 2 MB that the driver hands out.
+  void size_for(int n, int planes) {
+    const size_t ps = plane_size(n) * sizeof(double), step = (size_t)2 << 20, all = planes * ps + ((size_t)48 << 10);
+    chunk = all <= step ? std::max(all, (size_t)64 << 10)
+                        : std::min(std::max(4 * ps / step * step, 2 * step), 32 * step);
   }
   int take(void** p, size_t bytes, bool zero, cudaStream_t s) {
     *p = nullptr;
     if (alloc_fault()) return cuda_check(cudaErrorMemoryAllocation, "cudaMalloc");
     bytes = (bytes + 255) & ~(size_t)255;
+    for (Rest& r : rests)
+      if (bytes <= r.bytes) {
+        *p = r.at;
+        r.at += bytes;
+        r.bytes -= bytes;
+        return BMG_OK;
+      }
     const bool own = bytes > chunk / 2;
-    if (!own && bytes <= left) {
-      *p = cur;
-      cur += bytes;
-      left -= bytes;
-      return BMG_OK;
-    }
     void* b = nullptr;
     CK(cudaMalloc(&b, own ? bytes : chunk));
     blocks.push_back(b);
     if (zero || !own) CK(cudaMemsetAsync(b, 0, own ? bytes : chunk, s));
     *p = b;
-    if (!own) {
-      cur = (char*)b + bytes;
-      left = chunk - bytes;
-    }
+    if (!own) rests.push_back(Rest{(char*)b + bytes, chunk - bytes});
     return BMG_OK;
   }
 };
@@ -1427,6 +1434,7 @@ int setup_periodic(bmg_hierarchy* h, const bmg_stencil* A, int nx, int ny, int p
   if (!rc) rc = cuda_check(cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming), "event");
   if (!rc) rc = cuda_check(host_malloc((void**)&h->ctl_host, sizeof(Ctl)), "pinned");
   if (!rc) rc = order_after_user(h);
+  h->mem.size_for(3, 1);   // the levels' arrays are per_setup's own
   if (!rc) rc = dalloc(h->mem, &h->partials, 2 * (size_t)norm_partials_max(), h->ws);
   if (!rc) rc = per_setup(&h->per, A->kind, A->coef, nx, ny, periodic, h->arith == BMG_ARITH_FUSED, h->nu1, h->nu2,
                           h->smoother == BMG_SMOOTHER_ROWS   ? PER_SWEEP_ROWS
@@ -1458,7 +1466,6 @@ int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* o, bmg_hiera
   h->nx = nx;
   h->ny = ny;
   h->n = embed_size(nx, ny);
-  h->mem.size_for(h->n);
   if (o) {
     h->precision = o->precision;
     h->coarsest = o->coarsest ? o->coarsest : 3;
@@ -1501,13 +1508,17 @@ int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* o, bmg_hiera
   }
   if (h->coarsest > h->n) h->coarsest = h->n;
   if (o && o->periodic) return setup_periodic(h, A, nx, ny, o->periodic, out);
+  // stencils, weights, iterates and right-hand sides of all levels; FCG's vectors;
+  // the embedded problem's; the factored lines of one or two axes
+  const bool line = is_line(h->smoother), f64 = h->precision == BMG_FP64;
+  h->mem.size_for(h->n, (f64 ? 13 : 24) + (h->krylov == BMG_KRYLOV_FCG ? 4 : 0) + (nx != h->n || ny != h->n ? 2 : 0) +
+                            (line ? (f64 ? 6 : 2) * (line_dir(h->smoother) == LINE_XY ? 2 : 1) : 0));
   CounterScope cs(&h->launches);
   int rc = cuda_check(cudaStreamCreateWithFlags(&h->ws, cudaStreamNonBlocking), "stream");
   if (!rc) rc = cuda_check(cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming), "event");
   if (!rc) rc = cuda_check(host_malloc((void**)&h->ctl_host, sizeof(Ctl)), "pinned");
   if (!rc) rc = order_after_user(h);
   if (!rc) rc = setup_impl(h, A, h->n, o);
-  const bool line = is_line(h->smoother);
   if (!rc && line) rc = build_lines(h);
   if (!rc && !line && h->smoother >= BMG_SMOOTHER_TILE) rc = force_tile(h);
   if (!rc && !line && h->use_graph)   // the level-fused tail relaxes by points
@@ -2808,7 +2819,7 @@ int clone_state(const bmg_hierarchy* h0, cudaStream_t s, bmg_hierarchy** out) {
   bmg_hierarchy* h = new bmg_hierarchy();
   h->member = true;
   h->n = h0->n;
-  h->mem.size_for(h->n);
+  h->mem.size_for(h->n, 3);   // iterates and right-hand sides only
   h->nlev = h0->nlev;
   h->precision = h0->precision;
   h->nu1 = h0->nu1;
