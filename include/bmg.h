@@ -127,9 +127,11 @@ typedef struct {
   int inner_cycles;     /* FP32 V-cycles per refinement step (0 = 1) */
   int bf16_levels;      /* levels with BF16 stencils under BMG_BF16_IR (0 = 2) */
   int use_graph;        /* 1 (default): replay one captured CUDA graph per cycle, autotune the
-                           row-kernel tiles and run the coarse levels (n <= 63 FP32, n <= 31 FP64)
-                           as one level-fused launch, small levels above them as one launch
-                           down and one up; 0: plain launches, one per step */
+                           row-kernel tiles and run the coarse levels (n <= 63 FP32; FP64 n <= 15,
+                           or n <= 31 in a batch and where no level runs as follows) as one
+                           level-fused launch, small levels above them as one launch down and one
+                           up (with point smoothing, smoother and fuse_restrict left to the
+                           library, nu1 and nu2 1 or 2); 0: plain launches, one per step */
   int krylov;           /* BMG_KRYLOV_NONE (default): stationary V-cycle iteration;
                            BMG_KRYLOV_FCG: flexible CG with one cycle as preconditioner */
   const void* mlp;      /* bmg_mlp* for interp = BMG_INTERP_LEARNED, else NULL */
@@ -155,7 +157,8 @@ typedef struct {
                            that also forms the residual and restricts it -- temporal blocking --
                            against the two-sweep pass plus the separate residual + restriction),
                            BMG_FUSE_OFF, or BMG_FUSE_ON (always the fused pass; in a batch, on every
-                           stage whose sweeps are one-pass launches).  Same bits. */
+                           stage whose sweeps are one-pass launches).  Small levels run as one
+                           launch down and one up (use_graph) with BMG_FUSE_AUTO only.  Same bits. */
   int rhs_block;        /* batches of right-hand sides of one operator (bmg_batch_rhs), FP32 / BF16
                            levels swept by the one-pass kernel: BMG_RHS_BLOCK_AUTO (0, default; the
                            autotuner weighs sweeping 2 or 4 members per warp, each stencil value read

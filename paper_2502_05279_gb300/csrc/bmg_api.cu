@@ -2628,10 +2628,12 @@ int batch_rows(bool f64, int n, int count, bool shared) {
 }
 
 // The stages that run by halves, and their second iterates: graphs on, no
-// smoother or right-hand-side blocking forced, sweep counts the tiles allow.
+// smoother, right-hand-side blocking or fused restriction forced or forbidden,
+// sweep counts the tiles allow.
 int choose_batch_halves(bmg_batch* B) {
-  if (!B->use_graph || B->smoother != BMG_SMOOTHER_AUTO || B->rhs_block > BMG_RHS_BLOCK_OFF || B->nu1 < 1 ||
-      B->nu2 < 1 || B->nu1 > LEVEL_NU_MAX || B->nu2 > LEVEL_NU_MAX)
+  if (!B->use_graph || B->smoother != BMG_SMOOTHER_AUTO || B->fuse_restrict != BMG_FUSE_AUTO ||
+      B->rhs_block > BMG_RHS_BLOCK_OFF || B->nu1 < 1 || B->nu2 < 1 || B->nu1 > LEVEL_NU_MAX ||
+      B->nu2 > LEVEL_NU_MAX)
     return BMG_OK;
   for (int b = 1; b <= B->bmax; ++b)
     for (auto& g : B->stages[b]) {

@@ -1,0 +1,54 @@
+"""Which launches an iteration is made of, counted on the library's own counter:
+levels by halves are two launches each, the level-fused tail one, so that a rule
+of choice that no longer picks them shows here (their results are the same bits
+as the step-by-step cycle's either way)."""
+import pytest
+import torch
+
+import workloads as w
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(n, kind=9):
+    _, planes, f = w.general_size_problem(n, n, kind)
+    return torch.from_numpy(planes[:3] if kind == 5 else planes).cuda().contiguous(), torch.from_numpy(f).cuda()
+
+
+def batch_iteration(bmg, monkeypatch, probs, fuse=0, **kw):
+    """Launches of one iteration, and the iterates and histories of four."""
+    opts = bmg._lib.Opts
+
+    def make(*a):
+        o = opts(*a)
+        o.fuse_restrict = fuse
+        return o
+    monkeypatch.setattr(bmg._lib, "Opts", make)
+    B = bmg.Batch(9, [p[0] for p in probs], **kw)
+    monkeypatch.undo()
+    rhs = [p[1] for p in probs]
+    counts = []
+    for maxit in (0, 4):
+        before = B.launch_count
+        xs, _, _, _ = B.solve(rhs, tol=0.0, maxit=maxit)
+        counts.append(B.launch_count - before)
+    out = [x.clone() for x in xs], [B.history(k) for k in range(len(probs))]
+    B.close()
+    # (four iterations are one chunk, after which the done flags are gathered once more)
+    return (counts[1] - counts[0] - 1) / 4, out
+
+
+@pytest.mark.parametrize("precision,tail", [("fp32", 1), ("fp64", 1)])
+def test_batched_halves_follow_the_restriction_option(bmg, monkeypatch, precision, tail):
+    """BMG_FUSE_AUTO: the stages at 255 and 127 (FP64: 63) by halves; OFF: every step a launch of its own; ON: no
+    halves either, so that one-pass stages take the pass that the option asks for.  Same bits."""
+    probs = [problem(n) for n in ((255, 255, 127) if precision == "fp32" else (63, 63))]
+    kw = dict(precision=precision, arith="fused")
+    auto, a = batch_iteration(bmg, monkeypatch, probs, 0, **kw)
+    off, b = batch_iteration(bmg, monkeypatch, probs, 1, **kw)
+    on, c = batch_iteration(bmg, monkeypatch, probs, 2, **kw)
+    # two launches a stage, the tail, then FP64 residual and norm, or FP32 update, residual and norm
+    assert auto == (2 * 2 + tail + 3 if precision == "fp32" else 2 * 1 + tail + 2)
+    assert off > auto and on > auto
+    for x in (b, c):
+        assert all(torch.equal(p, q) for p, q in zip(a[0], x[0])) and a[1] == x[1]
