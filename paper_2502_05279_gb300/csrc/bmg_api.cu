@@ -1056,9 +1056,15 @@ int autotune_solo(bmg_hierarchy* h) {
 // side and iterate are written by both (they are rewritten every cycle). FP32
 // points, fused pass against the two: 842 / 907 us at 8191^2, 212 / 253 at
 // 4095^2, 66 / 84 at 2047^2.
+//
+// The revision is part of the record's key: raised when the pass or what it is
+// weighed against changes its speed, so that an older library's records, which
+// would keep the slower choice without a word, are timed again.
+constexpr int PAIR_RESTRICT_REVISION = 2;
 template <typename S>
 int tune_pair_restrict(Level& L, Level& C, const StencilView<float, S>& v, cudaStream_t s) {
-  const std::string fkey = tune_key("pair_restrict", {v.n, (int)sizeof(S), v.fused, L.pair32});
+  const std::string fkey =
+      tune_key("pair_restrict", {v.n, (int)sizeof(S), v.fused, L.pair32, PAIR_RESTRICT_REVISION});
   TuneRecord fr;
   if (tune_file_get(fkey, 1, &fr) && (fr.v[0] == 0 || fr.v[0] == 1)) {
     L.pair_rr = fr.v[0];
