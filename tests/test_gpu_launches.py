@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import workloads as w
+from test_gpu_periodic import problem as periodic_problem
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +53,49 @@ def test_batched_halves_follow_the_restriction_option(bmg, monkeypatch, precisio
     assert off > auto and on > auto
     for x in (b, c):
         assert all(torch.equal(p, q) for p, q in zip(a[0], x[0])) and a[1] == x[1]
+
+
+def solve_iteration(h, rhs):
+    """Launches of one iteration of h."""
+    counts = []
+    for maxit in (0, 4):
+        before = h.launch_count
+        h.solve(rhs, tol=0.0, maxit=maxit)
+        counts.append(h.launch_count - before)
+    return (counts[1] - counts[0]) / 4
+
+
+# levels by halves of a single problem: FP64 31 .. 511 over a tail from 15, FP32 and BF16 up to 1023 over a tail from
+# 63 (the first level below it that is not BF16); with FP32 63 the whole cycle is the tail
+@pytest.mark.parametrize("precision,n,halves", [("fp64", 31, 1), ("fp64", 63, 2), ("fp64", 511, 5), ("fp32", 63, 0),
+                                                ("fp32", 127, 1), ("fp32", 1023, 4), ("bf16", 127, 2),
+                                                ("bf16", 1023, 4)])
+@pytest.mark.parametrize("kind", [5, 9])
+def test_levels_by_halves(bmg, precision, n, halves, kind):
+    coef, f = problem(n, kind)
+    outer = 2 if precision == "fp64" else 3          # residual and norm; update, residual and norm
+    h = bmg.Hierarchy(kind, coef, precision=precision, arith="fused")
+    assert solve_iteration(h, f) == 2 * halves + 1 + outer
+    h.close()
+    h = bmg.Hierarchy(kind, coef, precision=precision, arith="fused", use_graph=False)
+    assert solve_iteration(h, f) > 2 * halves + 1 + outer
+    h.close()
+
+
+@pytest.mark.parametrize("precision,n,halves", [("fp32", 127, 1), ("fp64", 255, 4)])
+def test_levels_by_halves_in_flexible_cg(bmg, precision, n, halves):
+    coef, f = problem(n)
+    h = bmg.Hierarchy(9, coef, precision=precision, krylov="fcg")
+    # z.q, its sum, direction, A p, its sums, update, norm
+    assert solve_iteration(h, f) == 2 * halves + 1 + 7
+    h.close()
+
+
+@pytest.mark.parametrize("axes", ["x", "y", "xy"])
+@pytest.mark.parametrize("n", [15, 255, 511])
+def test_periodic_levels_by_halves(bmg, axes, n):
+    kind, planes, f, px, py = periodic_problem(n, axes, seed=80 + n, kind=9)
+    for krylov, outer in (("none", 1), ("fcg", 4)):   # residual; z.q, direction, A p, update (each with its sum)
+        h = bmg.Hierarchy(kind, torch.from_numpy(planes).cuda(), periodic=axes, krylov=krylov)
+        assert solve_iteration(h, torch.from_numpy(f).cuda()) == 2 * (h.num_levels - 1) + 1 + outer
+        h.close()
