@@ -282,7 +282,7 @@ struct bmg_hierarchy {
   cudaStream_t ws = nullptr;     // internal non-blocking work stream
   cudaEvent_t ev = nullptr;
   double* Lfac = nullptr;        // coarsest Cholesky factor (m x m)
-  double* work = nullptr;        // m x m factor workspace, then m doubles for substitutions
+  double* work = nullptr;        // m x m factor workspace
   int m = 0;
   double* partials = nullptr;
   int* err = nullptr;            // device error word of setup kernels
@@ -389,7 +389,7 @@ void vcycle64(bmg_hierarchy* h, int l, double* x, const double* f, const int* do
     return;
   }
   if (l == h->nlev - 1) {
-    step(h, l, BMG_K_COARSE, 0, [&] { launch_coarse_solve<double>(L.n, h->Lfac, f, x, h->work, done, s); });
+    step(h, l, BMG_K_COARSE, 0, [&] { launch_coarse_solve<double>(L.n, h->Lfac, f, x, done, s); });
     return;
   }
   auto v = view64(L);
@@ -496,7 +496,7 @@ void vcycle32(bmg_hierarchy* h, int l, const int* done, bool zero) {
   }
   if (l == h->nlev - 1) {
     step(h, l, BMG_K_COARSE, 1,
-         [&] { launch_coarse_solve<float>(L.n, h->Lfac, (const float*)L.f32, L.x32, h->work, done, s); });
+         [&] { launch_coarse_solve<float>(L.n, h->Lfac, (const float*)L.f32, L.x32, done, s); });
     return;
   }
   Level& C = h->lv[l + 1];
@@ -952,10 +952,10 @@ int build_tail(bmg_hierarchy* h, int lmin) {
     Level* C = lt + k + 1 < h->nlev ? &h->lv[lt + k + 1] : nullptr;
     if constexpr (sizeof(T) == 8)
       d.lv[k] = LevelDesc<double, double>{view64(L), L.ci, L.x, L.f, C ? C->x : nullptr, C ? C->f : nullptr,
-                                          nullptr, h->Lfac, h->work};
+                                          nullptr, h->Lfac};
     else
       d.lv[k] = LevelDesc<float, float>{view32(L), L.ci32, L.x32, L.f32, C ? C->x32 : nullptr,
-                                        C ? C->f32 : nullptr, nullptr, h->Lfac, h->work};
+                                        C ? C->f32 : nullptr, nullptr, h->Lfac};
   }
   if (int rc = h->mem.take(&h->d_tail, sizeof(d), false, h->ws)) return rc;
   CK(cudaMemcpyAsync(h->d_tail, &d, sizeof(d), cudaMemcpyHostToDevice, h->ws));   // (pageable: returns once copied)
@@ -1283,7 +1283,7 @@ int setup_impl(bmg_hierarchy* h, const bmg_stencil* A, int n, const bmg_opts* o)
   }
   h->m = h->coarsest * h->coarsest;
   if ((rc = dalloc(h->mem, &h->Lfac, (size_t)h->m * h->m, s))) return rc;
-  if ((rc = dalloc(h->mem, &h->work, (size_t)h->m * h->m + h->m, s))) return rc;
+  if ((rc = dalloc(h->mem, &h->work, (size_t)h->m * h->m, s))) return rc;
   if ((rc = dalloc(h->mem, &h->partials, 2 * (size_t)norm_partials_max(), s))) return rc;
   if (h->krylov == BMG_KRYLOV_FCG) {
     size_t ps = plane_size(n);
@@ -1986,10 +1986,7 @@ int bmg_coarse_factor(int n, const double* coef, double* L, void* stream) {
 int bmg_coarse_solve(int n, const double* L, const double* f, double* x, void* stream) {
   if (!is_level_size(n) || n > 15 || !L || !f || !x) return set_error(BMG_EINVAL, "bmg_coarse_solve: bad argument");
   cudaStream_t s = (cudaStream_t)stream;
-  double* y = nullptr;
-  CK(cudaMallocAsync((void**)&y, (size_t)n * n * sizeof(double), s));
-  launch_coarse_solve<double>(n, L, f, x, y, (const int*)nullptr, s);
-  CK(cudaFreeAsync(y, s));
+  launch_coarse_solve<double>(n, L, f, x, (const int*)nullptr, s);
   return step_done(s, "bmg_coarse_solve");
 }
 
@@ -2023,7 +2020,7 @@ struct bmg_batch {
   std::vector<bmg_hierarchy*> hs;
   cudaStream_t user = nullptr, ws = nullptr;
   cudaEvent_t ev = nullptr;
-  int bmax = 0, maxn = 0;
+  int bmax = 0;
   struct Group {
     int n = 0, count = 0, cl = 1, storage = 0, kind = 9;
     int tile = -1, pair = -1;   // one-pass / two-sweep shapes chosen for an FP32 group (-1: row kernel / none)
@@ -2101,10 +2098,10 @@ void append_tail(bmg_batch* B, bmg_hierarchy* h, int lt, const int* done, int b)
     Level* C = lt + k + 1 < h->nlev ? &h->lv[lt + k + 1] : nullptr;
     if constexpr (sizeof(T) == 8)
       d.lv[k] = LevelDesc<double, double>{view64(L), L.ci, L.x, L.f, C ? C->x : nullptr, C ? C->f : nullptr,
-                                          nullptr, h->Lfac, h->work};
+                                          nullptr, h->Lfac};
     else
       d.lv[k] = LevelDesc<float, float>{view32(L), L.ci32, L.x32, L.f32, C ? C->x32 : nullptr,
-                                        C ? C->f32 : nullptr, nullptr, h->Lfac, h->work};
+                                        C ? C->f32 : nullptr, nullptr, h->Lfac};
   }
   const char* c = (const char*)&d;
   B->tail_host[b].insert(B->tail_host[b].end(), c, c + sizeof(d));
@@ -2157,15 +2154,15 @@ int build_batch_tables(bmg_batch* B, const double* const* rhs, double* const* x)
       }
       if (storage == 0) {
         LevelDesc<double, double> d{view64(lv), lv.ci, l == 0 ? x[p] : lv.x, l == 0 ? rhs[p] : lv.f,
-                                    C ? C->x : nullptr, C ? C->f : nullptr, done, h->Lfac, h->work, lv.x64b, l > 0};
+                                    C ? C->x : nullptr, C ? C->f : nullptr, done, h->Lfac, lv.x64b, l > 0};
         append_desc(g, d);
       } else if (storage == 2) {
         LevelDesc<float, __nv_bfloat16> d{viewbf(lv), lv.ci32, lv.x32, lv.f32, C ? C->x32 : nullptr,
-                                          C ? C->f32 : nullptr, done, h->Lfac, h->work, lv.x32b, l > 0};
+                                          C ? C->f32 : nullptr, done, h->Lfac, lv.x32b, l > 0};
         append_desc(g, d);
       } else {
         LevelDesc<float, float> d{view32(lv), lv.ci32, lv.x32, lv.f32, C ? C->x32 : nullptr, C ? C->f32 : nullptr,
-                                  done, h->Lfac, h->work, lv.x32b, l > 0};
+                                  done, h->Lfac, lv.x32b, l > 0};
         append_desc(g, d);
       }
     }
@@ -2838,7 +2835,6 @@ int clone_state(const bmg_hierarchy* h0, cudaStream_t s, bmg_hierarchy** out) {
   h->arith = h0->arith;
   h->m = h0->m;
   h->Lfac = h0->Lfac;
-  h->work = h0->work;
   h->lv.resize(h0->lv.size());
   int rc = BMG_OK;
   for (size_t l = 0; l < h0->lv.size() && !rc; ++l) {
@@ -2946,7 +2942,6 @@ int bmg_setup_batched(int nprob, const bmg_stencil* A, const int* n, const bmg_o
     if (!rc) {
       B->hs.push_back(h);
       B->launches += h->launches;
-      B->maxn = std::max(B->maxn, n[p]);
       B->bmax = std::max(B->bmax, h->nlev - 1);
     }
   }
@@ -2986,7 +2981,6 @@ int bmg_batch_rhs(const bmg_hierarchy* h0, int k, const bmg_opts* o, bmg_batch**
     rc = clone_state(h0, B->ws, &h);
     if (!rc) {
       B->hs.push_back(h);
-      B->maxn = h0->n;
       B->bmax = h0->nlev - 1;
     }
   }

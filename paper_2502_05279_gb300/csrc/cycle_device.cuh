@@ -1127,7 +1127,7 @@ __device__ __forceinline__ bool gs_strip2r_ring_body(const StencilView<float, S>
     const int a = j0 - 4 + 2 * m, b = a - 2;
     // the coarse row restricted at the end of this step, and its weights, requested
     // before the step's arithmetic: loaded where they are used they kept every
-    // step of the few resident warps (4 to a scheduler, 128 registers) waiting for
+    // step of the few resident warps (3 to a scheduler, 168 registers) waiting for
     // memory once more: 8191^2 FP32 1020 -> 842 us, 4095^2 256 -> 212, 2047^2 76 -> 66
     const int jc = (b - 3) / 2;
     const bool coarse = m >= 5 && own_c && b - 3 >= j0 + 1 && b - 3 <= j1 - 1 && jc >= 1 && jc <= nc;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(NORM_THREADS) k_norm_finalize(const double* __
 
 template <typename T>
 __global__ void k_coarse_solve(int n, const double* __restrict__ L, const T* __restrict__ f, T* __restrict__ x,
-                               double* __restrict__ y, const int* done) {
+                               const int* done) {
   pdl_enter();
   if (stopped(done)) return;
   coarse_body<T>(n, L, f, x);
@@ -615,8 +615,8 @@ int launch_residual(const StencilView<T, S>& v, int kind, const T* x, const T* f
 }
 
 template <typename T>
-void launch_coarse_solve(int n, const double* L, const T* f, T* x, double* y, const int* done, cudaStream_t s) {
-  pdl_launch(k_coarse_solve<T>, 1, 32, 0, s, n, L, f, x, y, done);
+void launch_coarse_solve(int n, const double* L, const T* f, T* x, const int* done, cudaStream_t s) {
+  pdl_launch(k_coarse_solve<T>, 1, 32, 0, s, n, L, f, x, done);
   count_launch();
 }
 
@@ -692,10 +692,8 @@ template void launch_interp_to<double>(int, const double*, const double*, const 
                                        cudaStream_t, int);
 template void launch_interp_to<float>(int, const float*, const float*, const float*, float*, const int*,
                                       cudaStream_t, int);
-template void launch_coarse_solve<double>(int, const double*, const double*, double*, double*, const int*,
-                                          cudaStream_t);
-template void launch_coarse_solve<float>(int, const double*, const float*, float*, double*, const int*,
-                                         cudaStream_t);
+template void launch_coarse_solve<double>(int, const double*, const double*, double*, const int*, cudaStream_t);
+template void launch_coarse_solve<float>(int, const double*, const float*, float*, const int*, cudaStream_t);
 template int rows_cluster<double>(int);
 template int rows_cluster<float>(int);
 

@@ -184,7 +184,7 @@ template <typename T, typename S>
 int launch_residual(const StencilView<T, S>& v, int kind, const T* x, const T* f, T* r, double* partials,
                     const int* done, cudaStream_t s);
 template <typename T>
-void launch_coarse_solve(int n, const double* L, const T* f, T* x, double* y, const int* done, cudaStream_t s);
+void launch_coarse_solve(int n, const double* L, const T* f, T* x, const int* done, cudaStream_t s);
 
 int norm_partials_max();
 // Sum partials in a fixed order and record the norm in ctl (phase 0 = initial
@@ -225,8 +225,7 @@ struct LevelDesc {
   T* xc;              // next coarser level's iterate and right-hand side
   T* fc;
   const int* done;    // the problem's control flag
-  const double* L;    // coarsest level: Cholesky factor and substitution workspace
-  double* y;
+  const double* L;    // coarsest level: Cholesky factor
   T* x2 = nullptr;    // second iterate of a level swept by the one-pass kernels or run by halves (else NULL)
   int zero = 0;       // 1: a coarse level of its problem, whose iterate is zero when the cycle comes down to it
 };
