@@ -210,7 +210,11 @@ typedef struct {
  * may free it on return.  nx x ny interior points: nx == ny == 2^m - 1 >= 3
  * natively, any 1 <= nx, ny <= 65535 by embedding (see "General sizes"; not
  * with learned interpolation).  Stencil planes are (ny+2) x (nx+2).  opts may
- * be NULL.  Returns BMG_EINVAL (sizes, kind, options), BMG_ENOMEM, BMG_ECUDA
+ * be NULL.  Device memory, in FP64 planes (n+2)^2 of the finest level and over
+ * all levels: about 12 for an FP64 hierarchy, 23 for an FP32 or BF16 one, 4 more
+ * for flexible CG, and for line relaxation 5.3 (FP64) or 1.3 (FP32) per axis
+ * for the factored lines, held in chunks of 2 to 64 MB (smaller for small
+ * problems).  Returns BMG_EINVAL (sizes, kind, options), BMG_ENOMEM, BMG_ECUDA
  * or BMG_ESINGULAR; *out is NULL on failure. */
 int bmg_setup(const bmg_stencil* A, int nx, int ny, const bmg_opts* opts, bmg_hierarchy** out);
 
@@ -251,8 +255,10 @@ int bmg_time_cycles(bmg_hierarchy* h, const double* rhs, double* x, int cycles, 
 
 /* Per-level, per-kernel device time of `cycles` iterations launched one step
  * at a time without the graph, each step bracketed by CUDA events on the
- * hierarchy's stream (the Fig. 10 breakdown).  Fills up to `cap` rows of the
- * host array `rows` and returns the number of rows. */
+ * hierarchy's stream (the Fig. 10 breakdown).  With periodic sides the last sum
+ * of a norm or inner product is part of the kernel that forms it: no
+ * BMG_K_FINALIZE row.  Fills up to `cap` rows of the host array `rows` and
+ * returns the number of rows. */
 enum { BMG_K_RELAX = 0, BMG_K_RESID_RESTRICT = 1, BMG_K_INTERP = 2, BMG_K_COARSE = 3, BMG_K_NORM = 4,
        BMG_K_FINALIZE = 5, BMG_K_IR_UPDATE = 6, BMG_K_IR_RESIDUAL = 7, BMG_K_FCG = 8,
        BMG_K_TAIL = 9 /* the level-fused coarse levels, counted at their top level */,
@@ -279,8 +285,9 @@ int bmg_profile(bmg_hierarchy* h, const double* rhs, double* x, int cycles, bmg_
  * height whose strips fit into one wave of resident warps), or 0 (default;
  * not tuned).  With periodic sides: BMG_TILE_SWEEP for a level swept by the
  * one-pass strip kernel, 1 for the row-parity pair (or, on a 5-point level 0,
- * one launch per colour), 0 for the coarsest level.  Every choice computes the
- * same bits. */
+ * one launch per colour), 0 for the coarsest level.  Of a level that a solve
+ * runs as one launch down and one up, the kernel that its sweeps take when it is
+ * run step by step (bmg_profile).  Every choice computes the same bits. */
 #define BMG_TILE_SWEEP 16
 int bmg_tuned_cluster(const bmg_hierarchy* h, int level);
 
@@ -373,7 +380,8 @@ int bmg_time_cycles_batched(bmg_batch* b, const double* const* rhs, double* cons
  * the autotuner chose for stage `stage` (0 = coarsest): the row kernel's
  * cluster size, BMG_TILE_SWEEP + s for the one-pass kernel of shape s (stages
  * with n >= 255, FP64 or FP32/BF16; in FP32/BF16 stages pairs of sweeps may then
- * run as two-sweep passes), or 0 (not tuned). */
+ * run as two-sweep passes), or 0 (not tuned); of a stage that runs as one launch
+ * down and one up, the kernel that would sweep it otherwise. */
 long long bmg_batched_launch_count(const bmg_batch* b);
 int bmg_batched_tuned_cluster(const bmg_batch* b, int stage);
 
