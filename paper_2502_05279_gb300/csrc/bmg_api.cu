@@ -2617,17 +2617,27 @@ int force_rhs_block(bmg_batch* B) {
 }
 
 // Block rows per tile of a batched stage that runs by halves (0: step by step).
-// The change of a whole batch iteration when one stage runs by halves, us,
-// fused arithmetic, 16 rows (FP64 also 8), at 127 / 255 / 511 / 1023:
-//   40 problems FP32: -8 / -5 / -22 / +44    10 problems FP32: -13 / -15 / -8 / -7
-//   10 problems BF16: -28 / -28 / -9 / -1
-//   16 right-hand sides of 1023^2 FP32: -13 / -8 / +17 / +148 (block sweeps read the shared stencil once)
-//   FP64 at 63 / 127: 40 problems -4 / +13, 10 problems -5 (8 rows) / -1, 8 right-hand sides -8 (8 rows) / -2:
-//   the halos' FP64 work costs more than the launches as soon as the problems fill the chip: 256
-//   problems' iteration takes 10486 us by halves at 63, 10359 step by step (64 problems: 2587 / 2584)
+// The halos' work grows with the problems, the launches saved do not. One
+// iteration of `count` problems of n^2, us, step by step / by halves, fused
+// arithmetic (unless it says otherwise), each with its lower levels as they are:
+//   FP64 63, 8 rows:   8: 69.7 / 61.5   9: 69.7 / 61.5   10: 69.7 / 69.7   16: 73.8 / 77.9
+//     one rounding per operation: 9: 92.3 / 90.2   10: 96.3 / 108.6
+//     16 rows: 16: 73.8 / 69.9 but 100.4 / 108.6 with one rounding; 24: 79.9 / 81.7   64: 115 / 137
+//   FP64 127: 2: 77.9 / 69.7 but 4: 82.0 / 82.0   8: 96.7 / 94.1, with one rounding 139 / 148
+//   FP32 127: 16: 72.8 / 63.6   64: 144 / 144   128: 246 / 256   512: 964 / 941, BF16 512: 961 / 970
+//   FP32 255: 16: 132 / 131   24: 173 / 172   32: 211 / 216   64: 393 / 383   96: 502 / 551   256: 1274 / 1419
+//     right-hand sides of one operator: 24: 150 / 146   32: 178 / 180   64: 300 / 327   256: 1071 / 1211
+//   FP32 511: 4: 135 / 131   12: 277 / 275   18: 402 / 387   20: 399 / 428   32: 588 / 648   128: 2159 / 2423,
+//     BF16: 18: 378 / 387   20: 424 / 428   22: 425 / 463   128: 2135 / 2445
+//   (at 16 and 18 of 511^2, 64 of 255^2 the stencils of a stage step by step no longer fit into L2)
+//   FP32 1023 loses from 8 problems on (+44 us in a batch of 40 uneven ones); so do right-hand sides of 511^2
+//   (16: 285 / 309), whose sweeps read the shared stencil once.
 int batch_rows(bool f64, int n, int count, bool shared) {
-  if (f64) return n > 63 || count > 48 ? 0 : count <= 16 ? 8 : 16;
-  return n <= 255 || (n <= 511 && !shared) ? 16 : 0;
+  if (f64) return n <= 63 && count <= 9 ? 8 : 0;
+  if (n <= 127) return 16;
+  const long long points = (long long)n * n * count;
+  if (n <= 255) return points <= (shared ? 2100000 : 4800000) ? 16 : 0;
+  return n <= 511 && !shared && points <= 4800000 ? 16 : 0;
 }
 
 // The stages that run by halves, and their second iterates: graphs on, no

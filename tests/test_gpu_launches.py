@@ -55,6 +55,28 @@ def test_batched_halves_follow_the_restriction_option(bmg, monkeypatch, precisio
         assert all(torch.equal(p, q) for p, q in zip(a[0], x[0])) and a[1] == x[1]
 
 
+@pytest.mark.parametrize("precision,n,count,shared,halves", [
+    ("fp64", 63, 9, False, 1), ("fp64", 63, 10, False, 0), ("fp32", 127, 130, False, 1), ("fp32", 255, 72, False, 2),
+    ("fp32", 255, 74, False, 1), ("fp32", 255, 32, True, 2), ("fp32", 255, 33, True, 1), ("bf16", 511, 18, False, 3),
+    ("bf16", 511, 19, False, 2), ("fp32", 511, 2, True, 2)])
+def test_batched_halves_end_where_their_halos_cost_more(bmg, monkeypatch, precision, n, count, shared, halves):
+    """On both sides of the lines that the rule draws; stages below the one named stay by halves."""
+    coef, f = problem(n)
+    h = bmg.Hierarchy(9, coef, precision=precision, arith="fused")
+    B = bmg.Batch.from_hierarchy(h, count) if shared else bmg.Batch(9, [coef] * count, precision=precision, arith="fused")
+    counts = []
+    for maxit in (0, 4):
+        before = B.launch_count
+        B.solve([f] * count, tol=0.0, maxit=maxit)
+        counts.append(B.launch_count - before)
+    got, outer = (counts[1] - counts[0] - 1) / 4, 2 if precision == "fp64" else 3
+    by_halves = 2 * halves + 1 + outer
+    stages = {63: 1, 127: 1, 255: 2, 511: 3}[n]
+    assert got == by_halves if halves == stages else got >= by_halves + 3
+    B.close()
+    h.close()
+
+
 def solve_iteration(h, rhs):
     """Launches of one iteration of h."""
     counts = []
