@@ -369,11 +369,14 @@ int galloc(Arena& m, T** p, int n, int planes, cudaStream_t s) {
 }
 
 // Level l, started from a zero iterate, does not read one (and nothing has to
-// write the zeros): the tail, a level that runs by halves, an FP64 level whose
-// first sweep is a one-pass sweep, an FP32 level whose first pass streams rows.
+// write the zeros): the tail below level 0 (TailDesc::zero; at level 0 it reads
+// the iterate, whatever kernel is forced on the level), a level that runs by
+// halves, an FP64 level whose first sweep is a one-pass sweep, an FP32 level
+// whose first pass streams rows.
 bool zero_aware(const bmg_hierarchy* h, int l) {
   const Level& L = h->lv[l];
-  if ((l > 0 && l == h->tail_l) || (L.lrows > 0 && !h->prof)) return true;
+  if (l == h->tail_l) return l > 0;
+  if (L.lrows > 0 && !h->prof) return true;
   if (h->nu1 < 1 || is_line(h->smoother)) return false;
   if (h->precision == BMG_FP64) return L.tile64 >= 0;
   return L.tile32 >= 0 && (L.tile32 < 4 || (L.pair32 >= 0 && h->nu1 >= 2));
