@@ -3,7 +3,6 @@ FP64 planes of its finest level (stencil 6, weights 2, FP32 copies, packed
 stencils and iterates 10, a third more for the coarser levels) and some 50 KB
 that do not depend on the size, a member of a batch of right-hand sides' to 3
 planes; twice that is the bound, over a batch whose own tables are small."""
-import numpy as np
 import pytest
 import torch
 
